@@ -287,7 +287,6 @@ struct Ctx {
   bool exact = false;         // standard FETI-DP: every cell's own K_rr^{-1} (nrb = N, no ROM)
   float* Udp_f = nullptr;     // [N][nd][np] mixed path: the dual rows of U_rp_ring in FP32
   double* Urp_c = nullptr;    // [N][nr][np]
-  double* UrpT_c = nullptr;   // [N][np][nr]
   // coarse solve
   CoarseBCR bcr;
   // right-hand side of Eq. 16: [m][ntot] = (f_R, f_P, d = 0)
@@ -457,6 +456,8 @@ fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int 
 fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride, int ld, int mrows,
                                   int mcols, CCellVec x, CellVec y, double alpha, double beta,
                                   int nrhs);
+fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin,
+                           CCellVec x, CellVec y, double alpha, double beta, int nrhs);
 fetidp_status k_grouped_gemm(Ctx& c, const double* A, long long a_stride_k, int lda, int M, int K,
                              CCellVec X, CellVec Y, const double* coef, double alpha, double beta,
                              int nrhs, bool separate, long long y_k_stride);

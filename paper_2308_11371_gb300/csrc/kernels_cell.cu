@@ -536,40 +536,71 @@ __global__ void __launch_bounds__(352, 2) krr_spmm_nodal_f32_kernel(
     }
 }
 
-// Per-cell dense operators: y[rhs,cell] = alpha M_cell x[rhs,cell] + beta y, M_cell at
-// mats + cell*mstride with row stride ld (sub-blocks of the per-cell ROM operators).
+// Per-cell dense operators in FP64: y[rhs][cell][i] = alpha sum_j M_cell[j ld + i] x[rhs][cell][j] + beta y,
+// i < nout, j < nin -- the stored rows multiply x (M^T x; M x for the symmetric operators).
+//
+// Bound: GB300 issues two FP64 FMAs per clock and SM, and every 8-byte entry takes MR of them, so the
+// kernel is FP64-bound for every MR (5.0 TB/s of operator at MR = 1).  What matters is that all SMs have
+// the same share of FMAs and that nothing else uses the FP64 pipe: a CTA takes TI outputs of one cell
+// (32, or all of a narrower operator), its threads are S interleaved slices of the stored rows, a thread
+// keeps the MR sums of one output in registers, so a warp reads 256 consecutive bytes of a row, x comes
+// as shared-memory broadcasts, and only S - 1 additions per output are outside the FMA chain.  One CTA
+// per 32 outputs also gives 20 CTAs per 6^3 cell where a lattice has few cells.  The kernel it replaces
+// (one CTA per cell, a warp per row, five shuffle-adds per row and RHS) took 679 us per launch of this
+// class on 32 cells of n_d = 630 with 6 RHS, this one 96 us; the three products of an F_ring application
+// on 256 such cells took 1.90 ms and take 1.15 ms (FP64 bound 1.04 ms).
 constexpr int kMaxRhsGemv = 8;
-__global__ void cell_gemv_kernel(const double* __restrict__ mats, long long mstride, int ld,
-                                 int mrows, int mcols, const double* __restrict__ x, long long x_rs,
-                                 int x_cs, double* __restrict__ y, long long y_rs, int y_cs,
-                                 double alpha, double beta, int nrhs) {
-  extern __shared__ double xs[];   // [nrhs][mcols]
-  const long long cell = blockIdx.x;
-  for (int t = threadIdx.x; t < nrhs * mcols; t += blockDim.x) {
-    const int r = t / mcols, q = t - r * mcols;
-    xs[t] = x[r * x_rs + cell * x_cs + q];
-  }
+constexpr int kGemvThreads = 256;
+template <int MR>
+__global__ void __launch_bounds__(kGemvThreads) cell_gemvt_kernel(const double* __restrict__ mats, long long mstride,
+                                                                  int ld, int nout, int nin, int TI, int S,
+                                                                  const double* __restrict__ x, long long x_rs,
+                                                                  int x_cs, double* __restrict__ y, long long y_rs,
+                                                                  int y_cs, double alpha, double beta, int ntile) {
+  extern __shared__ __align__(16) double gvs[];   // x as [nin][MR]; then the slice sums [S][TI][MR]
+  constexpr int U = MR <= 2 ? 8 : 4;              // entries loaded ahead of their FMAs
+  const long long cell = blockIdx.x / ntile;
+  const int i0 = (int)(blockIdx.x - cell * ntile) * TI;
+  const double* xc = x + cell * x_cs;
+#pragma unroll
+  for (int r = 0; r < MR; ++r)
+    for (int j = threadIdx.x; j < nin; j += blockDim.x) gvs[j * MR + r] = xc[r * x_rs + j];
   __syncthreads();
-  const double* M = mats + cell * mstride;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int row = warp; row < mrows; row += nw) {
-    for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsGemv) {
-      const int rb = min(kMaxRhsGemv, nrhs - r0);
-      double acc[kMaxRhsGemv];
-      for (int r = 0; r < kMaxRhsGemv; ++r) acc[r] = 0.0;
-      for (int q = lane; q < mcols; q += 32) {
-        const double mv = M[(size_t)row * ld + q];
-        for (int r = 0; r < rb; ++r) acc[r] += mv * xs[(r0 + r) * mcols + q];
-      }
-      for (int r = 0; r < rb; ++r) {
-        double s = acc[r];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-          double* dst = y + (r0 + r) * y_rs + cell * y_cs + row;
-          *dst = (beta == 0.0) ? alpha * s : alpha * s + beta * (*dst);
-        }
-      }
+  const int il = threadIdx.x % TI, sl = threadIdx.x / TI;
+  const bool live = sl < S && i0 + il < nout;
+  double acc[MR];
+#pragma unroll
+  for (int r = 0; r < MR; ++r) acc[r] = 0.0;
+  if (live) {
+    const double* M = mats + cell * mstride + i0 + il;
+    int j = sl;
+    for (; j + (U - 1) * S < nin; j += U * S) {
+      double mv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) mv[u] = __ldcs(M + (long long)(j + u * S) * ld);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < MR; ++r) acc[r] = fma(mv[u], gvs[(j + u * S) * MR + r], acc[r]);
     }
+    for (; j < nin; j += S) {
+      const double mv = __ldcs(M + (long long)j * ld);
+#pragma unroll
+      for (int r = 0; r < MR; ++r) acc[r] = fma(mv, gvs[j * MR + r], acc[r]);
+    }
+  }
+  __syncthreads();                                // x is no longer read
+  if (sl < S)
+#pragma unroll
+    for (int r = 0; r < MR; ++r) gvs[(sl * TI + il) * MR + r] = acc[r];
+  __syncthreads();
+  for (int t = threadIdx.x; t < TI * MR; t += blockDim.x) {
+    const int r = t / TI, i = t - r * TI;
+    if (i0 + i >= nout) continue;
+    double s = gvs[i * MR + r];
+    for (int q = 1; q < S; ++q) s += gvs[(q * TI + i) * MR + r];
+    double* dst = y + r * y_rs + cell * y_cs + i0 + i;
+    *dst = (beta == 0.0) ? alpha * s : alpha * s + beta * (*dst);
   }
 }
 
@@ -1971,12 +2002,43 @@ fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride,
     FD_CHECK_LAUNCH();
     return FETIDP_OK;
   }
-  const size_t smem = (size_t)nrhs * mcols * sizeof(double);
-  cudaFuncSetAttribute(cell_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cell_gemv_kernel<<<(unsigned)c.N, 256, smem, c.stream>>>(mats, mstride, ld, mrows, mcols, x.p,
-                                                           x.rs, x.cs, y.p, y.rs, y.cs, alpha, beta,
-                                                           nrhs);
+  set_error("narrow per-cell operators: at most 32 columns");
+  return FETIDP_EINVAL;
+}
+
+template <int MR>
+static fetidp_status gemvt_launch(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin, CCellVec x,
+                                  CellVec y, double alpha, double beta) {
+  const int TI = std::min(nout, 32), S = kGemvThreads / TI, ntile = ceil_div(nout, TI);
+  const size_t smem = sizeof(double) * MR * (size_t)std::max(nin, S * TI);
+  if (smem > 227 * 1024) { set_error("per-cell operators: too many columns for shared memory"); return FETIDP_EINVAL; }
+  cudaFuncSetAttribute(cell_gemvt_kernel<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cell_gemvt_kernel<MR><<<(unsigned)(c.N * ntile), kGemvThreads, smem, c.stream>>>(
+      mats, mstride, ld, nout, nin, TI, S, x.p, x.rs, x.cs, y.p, y.rs, y.cs, alpha, beta, ntile);
   FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin, CCellVec x,
+                           CellVec y, double alpha, double beta, int nrhs) {
+  ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nout * nin * (double)c.N * nrhs,
+               8.0 * c.N * ((double)nout * nin + (double)nrhs * (nout + nin)));
+  // RHS per launch: eight, fewer where their x would not fit shared memory
+  const int most = (int)std::max<long long>(1, std::min<long long>(kMaxRhsGemv, 227 * 1024 / (8LL * nin)));
+  for (int r0 = 0; r0 < nrhs; r0 += most) {
+    const CCellVec xr{x.p + r0 * x.rs, x.rs, x.cs};
+    const CellVec yr{y.p + r0 * y.rs, y.rs, y.cs};
+    switch (std::min(most, nrhs - r0)) {
+      case 1: FD_TRY(gemvt_launch<1>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 2: FD_TRY(gemvt_launch<2>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 3: FD_TRY(gemvt_launch<3>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 4: FD_TRY(gemvt_launch<4>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 5: FD_TRY(gemvt_launch<5>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 6: FD_TRY(gemvt_launch<6>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      case 7: FD_TRY(gemvt_launch<7>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+      default: FD_TRY(gemvt_launch<8>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
+    }
+  }
   return FETIDP_OK;
 }
 

@@ -547,7 +547,7 @@ __global__ void split_planes_kernel(const double* __restrict__ x, long long n, f
 __global__ void rom_combine_kernel(const double* __restrict__ src, long long kstride, int ld,
                                    int r0, int c0, int rows, int cols,
                                    const double* __restrict__ coef, int nrb, long long ncell,
-                                   double* __restrict__ out, bool transpose) {
+                                   double* __restrict__ out) {
   const long long per = (long long)rows * cols;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < ncell * per;
        t += (long long)gridDim.x * blockDim.x) {
@@ -557,8 +557,7 @@ __global__ void rom_combine_kernel(const double* __restrict__ src, long long kst
     double s = 0.0;
     for (int k = 0; k < nrb; ++k)
       s += coef[cell * nrb + k] * src[k * kstride + (long long)(r0 + r) * ld + c0 + cc];
-    if (transpose) out[cell * per + (long long)cc * rows + r] = s;
-    else out[t] = s;
+    out[t] = s;
   }
 }
 
@@ -776,9 +775,9 @@ fetidp_status k_trace_tables(Ctx& c, const TraceTableSpec* specs_dev, int ntab, 
 }
 
 fetidp_status k_rom_combine(Ctx& c, const double* src, long long kstride, int ld, int r0, int c0,
-                            int rows, int cols, const double* coef, double* out, bool transpose) {
+                            int rows, int cols, const double* coef, double* out) {
   rom_combine_kernel<<<gridn(c.N * rows * cols), kThreads, 0, c.stream>>>(
-      src, kstride, ld, r0, c0, rows, cols, coef, c.nrb, c.N, out, transpose);
+      src, kstride, ld, r0, c0, rows, cols, coef, c.nrb, c.N, out);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

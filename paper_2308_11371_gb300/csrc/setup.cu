@@ -33,7 +33,7 @@ fetidp_status k_split_planes(Ctx& c, const double* x, long long n, float* hi, fl
 fetidp_status k_trace_tables_df(Ctx& c, const TraceTableSpecDF* specs_dev, int ntab, float* Th, float* Tl,
                                 long long ldt);
 fetidp_status k_rom_combine(Ctx& c, const double* src, long long kstride, int ld, int r0, int c0,
-                            int rows, int cols, const double* coef, double* out, bool transpose);
+                            int rows, int cols, const double* coef, double* out);
 
 namespace {
 
@@ -739,8 +739,8 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   } else if (!c.mixed) {   // FP64 path: per-cell assembled F_dd_ring, S_dd_ring
     FD_TRY(dalloc_t(c, &c.Fdd_c, (size_t)c.N * nd * nd));
     FD_TRY(dalloc_t(c, &c.Sdd_c, (size_t)c.N * nd * nd));
-    FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nd, c.delta, c.Fdd_c, false));
-    FD_TRY(k_rom_combine(c, c.Sdd, (long long)nd * nd, nd, 0, 0, nd, nd, c.alpha, c.Sdd_c, false));
+    FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nd, c.delta, c.Fdd_c));
+    FD_TRY(k_rom_combine(c, c.Sdd, (long long)nd * nd, nd, 0, 0, nd, nd, c.alpha, c.Sdd_c));
   } else {          // mixed path: principal operators packed for the tensor cores
     FD_TRY(k_element_matrices_f32(c));
     {
@@ -885,12 +885,9 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   }
   if (c.exact) {
     c.Urp_c = c.Urp;
-    c.UrpT_c = c.UrpT;
   } else {
     FD_TRY(dalloc_t(c, &c.Urp_c, (size_t)c.N * nr * np));
-    FD_TRY(dalloc_t(c, &c.UrpT_c, (size_t)c.N * nr * np));
-    FD_TRY(k_rom_combine(c, c.Urp, (long long)nr * np, np, 0, 0, nr, np, c.pi, c.Urp_c, false));
-    FD_TRY(k_rom_combine(c, c.Urp, (long long)nr * np, np, 0, 0, nr, np, c.pi, c.UrpT_c, true));
+    FD_TRY(k_rom_combine(c, c.Urp, (long long)nr * np, np, 0, 0, nr, np, c.pi, c.Urp_c));
   }
   if (c.mixed && (np == 8 || np == 24)) {   // the inner iterations' coarse term (Eq. 48) in FP32
     FD_TRY(dalloc_t(c, &c.Udp_f, (size_t)c.N * nd * np));

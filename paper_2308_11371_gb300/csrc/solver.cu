@@ -235,11 +235,17 @@ fetidp_status axpby(Ctx& c, const double* x, long long xs, const double* y, long
   return FETIDP_OK;
 }
 
-// Per-cell operator sub-blocks (FP64 path): y = alpha M x + beta y, M rows x cols with
-// row stride ld and per-cell stride mstride.
+// Per-cell operator sub-blocks in FP64 (row stride ld, per-cell stride mstride).
+// cell_op: y = alpha M x + beta y for a narrow M (rows x cols, the prolongations by U_rp).
 fetidp_status cell_op(Ctx& c, const double* mats, long long mstride, int ld, int rows, int cols,
                       CCellVec x, CellVec y, double alpha, double beta) {
   return k_cell_gemv_strided(c, mats, mstride, ld, rows, cols, x, y, alpha, beta, c.m);
+}
+
+// cell_opt: y = alpha M^T x + beta y, M of nin stored rows of nout entries (M x where M is symmetric).
+fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin,
+                       CCellVec x, CellVec y, double alpha, double beta) {
+  return k_cell_gemvt(c, mats, mstride, ld, nout, nin, x, y, alpha, beta, c.m);
 }
 
 }  // namespace
@@ -256,14 +262,14 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
   else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cFdd, cview(g), c.delta, c.delta, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
   else
-    FD_TRY(cell_op(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
+    FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
   // coarse correction: c_p = (T_dr U_rp_ring)^T g, assembled, S_PP^{-1}, prolonged.  The mixed path
   // applies it with FP32 copies of U_dp_ring and of the S_PP factor (a fixed perturbation of the
   // operator of the inner iterations, well inside their 1e-6 tolerance; the outer FGMRES is FP64).
   if (c.Udp_f)
     FD_TRY(k_udp_f32(c, true, cview(g), cp, 1.0, 0.0, m));
   else
-    FD_TRY(cell_op(c, c.UrpT_c + ni, (long long)np * nr, nr, np, nd, cview(g), cp, 1.0, 0.0));
+    FD_TRY(cell_opt(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, np, nd, cview(g), cp, 1.0, 0.0));
   FD_TRY(k_primal_assemble(c, cview(cp), c.w_P1, c.nP, 1.0, 0.0, m));
   if (c.bcr.mats_f)
     FD_TRY(coarse_solve_f32(c, c.w_P1, c.nP, c.w_P2, c.nP, m));
@@ -290,7 +296,7 @@ fetidp_status op_apply_MD(Ctx& c, const double* r, long long r_rs, double* z, lo
   else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cSdd, cview(g), c.alpha, c.alpha, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
   else
-    FD_TRY(cell_op(c, c.Sdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
+    FD_TRY(cell_opt(c, c.Sdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
   FD_TRY(k_scatter_B(c, cview(yd), z, z_rs, c.dinfo, 1.0, 0.0, m));
   return FETIDP_OK;
 }
@@ -330,13 +336,13 @@ fetidp_status U_apply(Ctx& c, CCellVec vR, const double* vP, long long vP_rs, do
                       long long out_rs) {
   const int m = c.m, nd = c.nd, np = c.np, nr = c.nr, ni = c.ni;
   CellVec cp{c.w_p1, c.N * np, np}, td{c.w_d1, c.N * nd, nd};
-  FD_TRY(cell_op(c, c.UrpT_c, (long long)np * nr, nr, np, nr, vR, cp, 1.0, 0.0));
+  FD_TRY(cell_opt(c, c.Urp_c, (long long)nr * np, np, np, nr, vR, cp, 1.0, 0.0));
   FD_TRY(k_copy_scale(c, vP, c.w_P1, c.nP, m, vP_rs, c.nP, nullptr, 1.0));
   FD_TRY(k_primal_assemble(c, cview(cp), c.w_P1, c.nP, -1.0, 1.0, m));
   FD_TRY(coarse_solve(c, c.w_P1, c.nP, c.w_zP, c.nP, m));
   // t_d = U_rd_ring^T v_r - T_dr U_rp_ring A_p^T z_P
-  if (c.exact)   // standard FETI-DP: rows d of each cell's own K_rr^{-1} (symmetric)
-    FD_TRY(cell_op(c, c.Kinv + (size_t)ni * nr, (long long)nr * nr, nr, nd, nr, vR, td, 1.0, 0.0));
+  if (c.exact)   // standard FETI-DP: columns d of each cell's own K_rr^{-1} (symmetric)
+    FD_TRY(cell_opt(c, c.Kinv + ni, (long long)nr * nr, nr, nd, nr, vR, td, 1.0, 0.0));
   else if (c.Uid_f) {   // assembled FP32 blocks: U_id^T v_i + F_dd v_d
     FD_TRY(k_cell_gemm_f32(c, c.Uid_f, c.ld_id, nd, ni, vR, td, 1.0, 0.0, m));
     const CCellVec vd{vR.p + ni, vR.rs, vR.cs};
@@ -359,7 +365,7 @@ fetidp_status U_apply(Ctx& c, CCellVec vR, const double* vP, long long vP_rs, do
 // standard FETI-DP: x_r = K_rr^(s)^{-1} v_r with the cell's own inverse
 fetidp_status local_rom(Ctx& c, CCellVec vR, CellVec xR) {
   const int m = c.m, nr = c.nr, nrb = c.nrb;
-  if (c.exact) return cell_op(c, c.Kinv, (long long)nr * nr, nr, nr, nr, vR, xR, 1.0, 0.0);
+  if (c.exact) return cell_opt(c, c.Kinv, (long long)nr * nr, nr, nr, nr, vR, xR, 1.0, 0.0);
   if (c.mixed) {
     float* Rf = reinterpret_cast<float*>(c.w_R);
     float* KRf = reinterpret_cast<float*>(c.w_KR);
@@ -613,11 +619,11 @@ fetidp_status op_precondition(Ctx& c, const double* x, double* y) {
   // U_ring^T y = (U_RD B_R^T y - U_RP z'_P, z'_P), z'_P = S_PP^{-1}(-U_RP^T B_R^T y)
   CellVec g{c.w_d1, c.N * nd, nd};
   FD_TRY(k_gather_BT(c, yL, nt, nullptr, g, m, 0.0));
-  FD_TRY(cell_op(c, c.UrpT_c + ni, (long long)np * nr, nr, np, nd, cview(g), cp, 1.0, 0.0));
+  FD_TRY(cell_opt(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, np, nd, cview(g), cp, 1.0, 0.0));
   FD_TRY(k_primal_assemble(c, cview(cp), c.w_P1, c.nP, -1.0, 0.0, m));
   FD_TRY(coarse_solve(c, c.w_P1, c.nP, c.w_P1, c.nP, m));
-  if (c.exact)   // columns d of each cell's own K_rr^{-1}
-    FD_TRY(cell_op(c, c.Kinv + ni, (long long)nr * nr, nr, nr, nd, cview(g), yR, -1.0, 1.0));
+  if (c.exact)   // rows d of each cell's own K_rr^{-1}, applied transposed (symmetric)
+    FD_TRY(cell_opt(c, c.Kinv + (size_t)ni * nr, (long long)nr * nr, nr, nr, nd, cview(g), yR, -1.0, 1.0));
   else if (c.Uid_f) {   // assembled FP32 blocks: y_i -= U_id g, y_d -= F_dd g
     FD_TRY(k_cell_gemm_f32(c, c.Udi_f, c.ld_di, ni, nd, cview(g), yR, -1.0, 1.0, m));
     const CellVec yd{yR.p + ni, yR.rs, yR.cs};

@@ -1,0 +1,67 @@
+"""Per-cell operator kernels at the sizes where their tilings change, against the FP64 CPU oracle.
+
+Tolerances are those of the operator parity tests (quantities behind a dense factorisation 1e-9,
+pure applications of a Dirichlet operator 1e-11): the kernels only order the sums differently.
+"""
+import numpy as np
+import pytest
+
+from paper_2308_11371_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _rel(a, b):
+    a, b = np.asarray(a), np.asarray(b)
+    return np.abs(a - b).max() / max(np.abs(b).max(), 1e-300)
+
+
+def _dev(x):
+    return torch.as_tensor(np.ascontiguousarray(x), dtype=torch.float64, device="cuda")
+
+
+def _loads(dim, count):
+    rng = np.random.default_rng(count)
+    return [W.Load(W.LOAD_BODY, tuple(rng.standard_normal(dim))) for _ in range(count)]
+
+
+def _problem(kind, n_rhs):
+    if kind == "2d_e3":     # n_d = 16: one narrow tile; n_p = 8
+        p = W.lattice_2d(3, 2, 3, a=0.2, r=0.2, n_rb=2)
+        p.loads = _loads(2, n_rhs)
+    elif kind == "2d_e9":   # n_d = 64: two full tiles of 32 outputs
+        p = W.lattice_2d(2, 2, 9, a=0.2, r=0.12, n_rb=2)
+        p.loads = _loads(2, n_rhs)
+    else:                   # n_d = 270, n_r = 351: a ragged last tile; n_p = 24
+        p = W.lattice_3d(2, 2, 1, e=4, r=0.2, r_spread=0.05, seed=3, n_rb=3, mask_kind=W.MASK_BCC_SIGMOID,
+                         map_kind=W.MAP_SHEAR_BEND_3D, map_params=(0.3, 2.0, 0.1, -0.15), loads=_loads(3, n_rhs))
+    return p
+
+
+_ORACLE = {}
+
+
+def _oracle(kind):
+    if kind not in _ORACLE:
+        from oracle import feti_dp, ifeti_dp
+        from oracle.discretization import Lattice
+        lat = Lattice(_problem(kind, 1))
+        blocks = [feti_dp.CellBlocks(lat, s) for s in range(lat.N)]
+        _ORACLE[kind] = ifeti_dp.InexactFETIDP(lat, blocks=blocks)
+    return _ORACLE[kind]
+
+
+@pytest.mark.parametrize("kind", ["2d_e3", "2d_e9", "3d_e4"])
+@pytest.mark.parametrize("n_rhs", [1, 2, 3, 4, 5, 6, 7, 8, 11])
+def test_fp64_cell_operators_for_every_rhs_count(kind, n_rhs):
+    from paper_2308_11371_gb300 import binding
+    ref = _oracle(kind)
+    s = binding.Solver(_problem(kind, n_rhs))
+    rng = np.random.default_rng(n_rhs)
+    lam = rng.standard_normal((s.n_rhs, s.L))
+    y, z = s.apply_F(_dev(lam)).cpu().numpy(), s.precond(_dev(lam)).cpu().numpy()
+    for r in range(n_rhs):
+        assert _rel(y[r], ref.apply_F(lam[r])) < 1e-9
+        assert _rel(z[r], ref.apply_MD(lam[r])) < 1e-11
