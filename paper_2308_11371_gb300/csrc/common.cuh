@@ -273,6 +273,10 @@ struct Ctx {
   // ROM per-cell operators (assembled, Eq. 43)
   double* Fdd_c = nullptr;    // [N][nd][nd]
   double* Sdd_c = nullptr;    // [N][nd][nd]
+  // FP64 path, lattices up to kUidBytes: U_id_ring (Algorithm 3) assembled in both orientations,
+  // [N][n_i][n_d] and [N][n_d][n_i]; larger lattices combine the principal operators at every use
+  double* Uid_c = nullptr;
+  double* Udi_c = nullptr;
   // mixed path, large cells: the same operators assembled in FP32, rows padded to ld_f (16 bytes)
   float* Fdd_f = nullptr;     // [N][nd][ld_f]
   float* Sdd_f = nullptr;     // [N][nd][ld_f]
@@ -461,10 +465,8 @@ fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld
 fetidp_status k_grouped_gemm(Ctx& c, const double* A, long long a_stride_k, int lda, int M, int K,
                              CCellVec X, CellVec Y, const double* coef, double alpha, double beta,
                              int nrhs, bool separate, long long y_k_stride);
-fetidp_status k_grouped_gemm_n(Ctx& c, const double* A, long long a_stride_k, int lda, int M,
-                               int K, int nk, CCellVec X, CellVec Y, const double* coef,
-                               double alpha, double beta, long long ncell, int nrhs, bool separate,
-                               long long y_k_stride, int prof_class = FETIDP_K_GROUPED_GEMM);
+fetidp_status k_trace_gemm(Ctx& c, const double* A, int lda, int M, int K, const double* X, int x_cs,
+                           long long ncols, double* Y, int y_cs);
 fetidp_status k_gram_solve(Ctx& c, const double* R, const double* KR, CCellVec v, CellVec x,
                            int nrhs, int len = -1);
 fetidp_status k_grad(Ctx& c, const double* u, const double* w, double* g);

@@ -1048,32 +1048,43 @@ __global__ void __launch_bounds__(1024) udp_n_f32_kernel(const float* __restrict
   }
 }
 
-// Grouped FP64 GEMM, 64x64 output tile per block, 4x4 per thread, K chunks of 16.
+// Grouped FP64 GEMM, 64 x TN output tile per block (256 threads, 4 x TN/16 per thread), K chunks of 16.
+// Bound: the FP64 pipe (2 FMA per clock and SM; 1 FMA per output and k), so a launch needs blocks on
+// every SM and little padding: TN is the narrowest of 16, 32, 64 that holds the columns (32 columns on a
+// 64-wide tile are half padding) and separate outputs take one principal per blockIdx.z.  With one block
+// per tile running the principals one after the other, the 16 local bases of 32 cells of 6^3 elements
+// and 6 RHS kept 48 blocks busy for 17 ms; they take 6.2 ms now (FP64 bound 4.9 ms).
 constexpr int GT = 64, GK = 16;
+template <int TN>
 __global__ void __launch_bounds__(256) grouped_gemm_kernel(
     const double* __restrict__ A, long long a_stride_k, int lda, int M, int K, int nk,
     const double* __restrict__ X, long long x_rs, int x_cs, double* __restrict__ Y, long long y_rs,
     int y_cs, const double* __restrict__ coef, double alpha, double beta, long long ncell, int nrhs,
     bool separate, long long y_k_stride) {
+  constexpr int NJ = TN / 16;
   __shared__ double As[GK][GT + 1];
-  __shared__ double Xs[GK][GT + 1];
+  __shared__ double Xs[GK][TN + 1];
   const long long ncols = ncell * nrhs;
-  const long long col0 = (long long)blockIdx.x * GT;
+  const long long col0 = (long long)blockIdx.x * TN;
   const int m0 = blockIdx.y * GT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // 16 x 16 threads
-  double tot[4][4];
+  const int kb = separate ? blockIdx.z : 0, ke = separate ? kb + 1 : nk;
+  double tot[4][NJ];
   for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) tot[i][j] = 0.0;
-  for (int k = 0; k < nk; ++k) {
+    for (int j = 0; j < NJ; ++j) tot[i][j] = 0.0;
+  for (int k = kb; k < ke; ++k) {
     const double* Ak = A + k * a_stride_k;
-    double acc[4][4];
+    double acc[4][NJ];
     for (int i = 0; i < 4; ++i)
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+      for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0;
     for (int kk0 = 0; kk0 < K; kk0 += GK) {
       for (int t = threadIdx.x; t < GK * GT; t += 256) {
         const int r = t / GK, q = t - r * GK;     // A: row r, k q  (q fastest -> coalesced rows)
         const int gm = m0 + r, gk = kk0 + q;
         As[q][r] = (gm < M && gk < K) ? Ak[(size_t)gm * lda + gk] : 0.0;
+      }
+      for (int t = threadIdx.x; t < GK * TN; t += 256) {
+        const int r = t / GK, q = t - r * GK, gk = kk0 + q;
         const long long gc = col0 + r;            // X: column r, k q
         double xv = 0.0;
         if (gc < ncols && gk < K) {
@@ -1086,16 +1097,16 @@ __global__ void __launch_bounds__(256) grouped_gemm_kernel(
       __syncthreads();
 #pragma unroll
       for (int q = 0; q < GK; ++q) {
-        double a[4], b[4];
+        double a[4], b[NJ];
         for (int i = 0; i < 4; ++i) a[i] = As[q][ty + 16 * i];
-        for (int j = 0; j < 4; ++j) b[j] = Xs[q][tx + 16 * j];
+        for (int j = 0; j < NJ; ++j) b[j] = Xs[q][tx + 16 * j];
         for (int i = 0; i < 4; ++i)
-          for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
+          for (int j = 0; j < NJ; ++j) acc[i][j] += a[i] * b[j];
       }
       __syncthreads();
     }
     if (separate) {
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < NJ; ++j) {
         const long long gc = col0 + tx + 16 * j;
         if (gc >= ncols) continue;
         const int rhs = (int)(gc / ncell);
@@ -1107,7 +1118,7 @@ __global__ void __launch_bounds__(256) grouped_gemm_kernel(
         }
       }
     } else {
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < NJ; ++j) {
         const long long gc = col0 + tx + 16 * j;
         double cf = 1.0;
         if (coef != nullptr && gc < ncols) {
@@ -1119,7 +1130,7 @@ __global__ void __launch_bounds__(256) grouped_gemm_kernel(
     }
   }
   if (!separate) {
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < NJ; ++j) {
       const long long gc = col0 + tx + 16 * j;
       if (gc >= ncols) continue;
       const int rhs = (int)(gc / ncell);
@@ -1131,6 +1142,51 @@ __global__ void __launch_bounds__(256) grouped_gemm_kernel(
       }
     }
   }
+}
+
+// One operator against every column, Y[col][m] = sum_k A[m][k] X[col][k] (the Eq. 42 traces), K summed
+// in one chain of FMAs per output as the tiled kernel does: the traces of nearly dependent principal
+// fields are solved by a pivoted Gram solve that amplifies a change of summation order by ~1e7, so K is
+// not split.  The FP64 pipe takes 64 cycles per warp instruction and sub-partition, so a T x T tile of
+// T^2 threads with one output each already keeps it busy (two 8-byte shared reads per FMA are hidden),
+// and small tiles spread few outputs over all SMs: 288 traces of 32 cells were 5 blocks of 64 x 64 and
+// 92 ms, now 4.4 ms (one chain of 77,760 FMAs: 2.4 ms); of 256 cells 94 ms, now 9.9 ms (FP64 bound 9.1).
+constexpr int kTraceK = 32, kTraceLd = 33;   // row stride: a warp's 16 (or 8) rows hit different banks
+template <int T>
+__global__ void __launch_bounds__(T * T) trace_gemm_kernel(const double* __restrict__ A, int lda, int M, int K,
+                                                           const double* __restrict__ X, long long x_cs,
+                                                           double* __restrict__ Y, long long y_cs, long long ncols) {
+  __shared__ double As[2][T][kTraceLd], Xs[2][T][kTraceLd];
+  const int m0 = blockIdx.x * T;
+  const long long col0 = (long long)blockIdx.y * T;
+  const int tx = threadIdx.x % T, ty = threadIdx.x / T;
+  auto load = [&](int buf, int k0) {
+    for (int t = threadIdx.x; t < 2 * T * kTraceK; t += T * T) {
+      const int q = t % kTraceK, row = (t / kTraceK) % T, gk = k0 + q;
+      const bool isx = t >= T * kTraceK;
+      const long long g = isx ? col0 + row : m0 + row;
+      const bool in = gk < K && g < (isx ? ncols : (long long)M);
+      const double* src = isx ? X + (in ? g * x_cs + gk : 0) : A + (in ? g * lda + gk : 0);
+      const unsigned d = (unsigned)__cvta_generic_to_shared(isx ? &Xs[buf][row][q] : &As[buf][row][q]);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  double acc = 0.0;
+  load(0, 0);
+  for (int k0 = 0, buf = 0; k0 < K; k0 += kTraceK, buf ^= 1) {
+    if (k0 + kTraceK < K) {
+      load(buf ^ 1, k0 + kTraceK);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kTraceK; ++q) acc = fma(As[buf][ty][q], Xs[buf][tx][q], acc);
+    __syncthreads();                              // this buffer is refilled by the next iteration's load
+  }
+  if (m0 + ty < M && col0 + tx < ncols) Y[(col0 + tx) * y_cs + m0 + ty] = acc;
 }
 
 // Eq. 46b for one (rhs, cell) per warp.
@@ -2045,21 +2101,35 @@ fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld
 fetidp_status k_grouped_gemm(Ctx& c, const double* A, long long a_stride_k, int lda, int M, int K,
                              CCellVec X, CellVec Y, const double* coef, double alpha, double beta,
                              int nrhs, bool separate, long long y_k_stride) {
-  return k_grouped_gemm_n(c, A, a_stride_k, lda, M, K, c.nrb, X, Y, coef, alpha, beta, c.N, nrhs,
-                          separate, y_k_stride);
+  const int nk = c.nrb;
+  const long long ncell = c.N;
+  const long long ncols = ncell * nrhs;
+  ProfScope ps(c, FETIDP_K_GROUPED_GEMM, 2.0 * M * K * nk * (double)ncols,
+               8.0 * ((double)nk * M * K + (double)ncols * K + (double)ncols * M * (separate ? nk : 1)));
+  const int TN = ncols <= 16 ? 16 : ncols <= 32 ? 32 : 64;
+  const dim3 grid((unsigned)ceil_div(ncols, TN), (unsigned)ceil_div(M, GT), (unsigned)(separate ? nk : 1));
+#define FD_GROUPED(T)                                                                                              \
+  grouped_gemm_kernel<T><<<grid, 256, 0, c.stream>>>(A, a_stride_k, lda, M, K, nk, X.p, X.rs, X.cs, Y.p, Y.rs, Y.cs, \
+                                                     coef, alpha, beta, ncell, nrhs, separate, y_k_stride)
+  if (TN == 16) FD_GROUPED(16);
+  else if (TN == 32) FD_GROUPED(32);
+  else FD_GROUPED(64);
+#undef FD_GROUPED
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
 }
 
-fetidp_status k_grouped_gemm_n(Ctx& c, const double* A, long long a_stride_k, int lda, int M,
-                               int K, int nk, CCellVec X, CellVec Y, const double* coef,
-                               double alpha, double beta, long long ncell, int nrhs, bool separate,
-                               long long y_k_stride, int prof_class) {
-  const long long ncols = ncell * nrhs;
-  ProfScope ps(c, prof_class, 2.0 * M * K * nk * (double)ncols,
-               8.0 * ((double)nk * M * K + (double)ncols * K + (double)ncols * M * (separate ? nk : 1)));
-  dim3 grid((unsigned)ceil_div(ncols, GT), (unsigned)ceil_div(M, GT));
-  grouped_gemm_kernel<<<grid, 256, 0, c.stream>>>(A, a_stride_k, lda, M, K, nk, X.p, X.rs, X.cs,
-                                                  Y.p, Y.rs, Y.cs, coef, alpha, beta, ncell, nrhs,
-                                                  separate, y_k_stride);
+fetidp_status k_trace_gemm(Ctx& c, const double* A, int lda, int M, int K, const double* X, int x_cs, long long ncols,
+                           double* Y, int y_cs) {
+  if (M <= 0 || ncols <= 0) return FETIDP_OK;
+  ProfScope ps(c, FETIDP_K_TRACES, 2.0 * M * (double)K * ncols, 8.0 * ((double)M * K + (double)ncols * (K + M)));
+  // 16 x 16 outputs per block; 8 x 8 while those blocks do not cover the SMs twice over
+  const bool small = (long long)ceil_div(M, 16) * ceil_div(ncols, 16) < 2 * 152;
+  const int T = small ? 8 : 16;
+  if (ceil_div(ncols, T) > 65535) { set_error("trace contraction: too many cells for one launch"); return FETIDP_EINVAL; }
+  const dim3 grid((unsigned)ceil_div(M, T), (unsigned)ceil_div(ncols, T));
+  if (small) trace_gemm_kernel<8><<<grid, 64, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols);
+  else trace_gemm_kernel<16><<<grid, 256, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

@@ -39,6 +39,12 @@ namespace {
 
 constexpr double kTieRel = 1e-12;     // greedy argmax ties (lowest cell index wins)
 constexpr double kDropRel = 1e-12;    // pivot drop of the N_rb x N_rb Gram systems
+// FP64 path: U_id_ring is assembled per cell (both orientations) up to this size.  Combining the
+// principal operators at every use costs n_rb m FMAs per entry and application on the FP64 pipe, the
+// assembly n_rb once and m per application: 17 ms per application on 32 cells of 6^3 elements with 16
+// principals and 6 RHS against 0.2 ms.  8 GB (2,200 such cells) leaves the largest lattices, whose
+// F_dd and S_dd already fill most of the memory, on the combined form.
+constexpr size_t kUidBytes = (size_t)8 << 30;
 
 struct RefCell {
   std::vector<int> perm;        // idp -> natural
@@ -714,8 +720,7 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
                               cudaMemcpyHostToDevice, c.stream));
       FD_TRY(k_trace_tables(c, static_cast<const TraceTableSpec*>(specs_dev), (int)specs.size(), Tab, c.nsnap));
       phase("  gradients + trace tables");
-      FD_TRY(k_grouped_gemm_n(c, Tab, 0, (int)c.nsnap, ntab, (int)c.nsnap, 1, CCellVec{c.snap, 0, (int)c.nsnap},
-                              CellVec{Y, 0, ntab}, nullptr, 1.0, 0.0, c.N, 1, false, 0, FETIDP_K_TRACES));
+      FD_TRY(k_trace_gemm(c, Tab, (int)c.nsnap, ntab, (int)c.nsnap, c.snap, (int)c.nsnap, c.N, Y, ntab));
     }
     phase("  trace contraction");
     // the two Gram systems of every cell, solved on the device (one warp per system)
@@ -741,6 +746,12 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
     FD_TRY(dalloc_t(c, &c.Sdd_c, (size_t)c.N * nd * nd));
     FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nd, c.delta, c.Fdd_c));
     FD_TRY(k_rom_combine(c, c.Sdd, (long long)nd * nd, nd, 0, 0, nd, nd, c.alpha, c.Sdd_c));
+    if (ni > 0 && (size_t)c.N * ni * nd * 2 * sizeof(double) <= kUidBytes) {
+      FD_TRY(dalloc_t(c, &c.Uid_c, (size_t)c.N * ni * nd));
+      FD_TRY(dalloc_t(c, &c.Udi_c, (size_t)c.N * ni * nd));
+      FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, 0, ni, ni, nd, c.delta, c.Uid_c));
+      FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, ni, 0, nd, ni, c.delta, c.Udi_c));
+    }
   } else {          // mixed path: principal operators packed for the tensor cores
     FD_TRY(k_element_matrices_f32(c));
     {

@@ -352,7 +352,10 @@ fetidp_status U_apply(Ctx& c, CCellVec vR, const double* vP, long long vP_rs, do
       FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, vd, td, 1.0, 1.0, m));
   } else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cUrdT, vR, c.delta, c.delta, td.p, true, td.rs, td.cs, 1.0, 0.0, m, c.N));
-  else
+  else if (c.Uid_c) {   // assembled blocks: U_id^T v_i + F_dd v_d
+    FD_TRY(cell_opt(c, c.Uid_c, (long long)ni * nd, nd, nd, ni, vR, td, 1.0, 0.0));
+    FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, CCellVec{vR.p + ni, vR.rs, vR.cs}, td, 1.0, 1.0));
+  } else
     FD_TRY(k_grouped_gemm(c, c.Kinv + (size_t)ni * nr, (long long)nr * nr, nr, nd, nr, vR, td, c.delta,
                           1.0, 0.0, m, false, 0));
   FD_TRY(k_primal_extract(c, c.w_zP, c.nP, cp, m));
@@ -633,7 +636,10 @@ fetidp_status op_precondition(Ctx& c, const double* x, double* y) {
       FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, cview(g), yd, -1.0, 1.0, m));
   } else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cUrd, cview(g), c.delta, c.delta, yR.p, true, yR.rs, yR.cs, -1.0, 1.0, m, c.N));
-  else
+  else if (c.Uid_c) {   // assembled blocks: y_i -= U_id g, y_d -= F_dd g
+    FD_TRY(cell_opt(c, c.Udi_c, (long long)ni * nd, ni, ni, nd, cview(g), yR, -1.0, 1.0));
+    FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), CellVec{yR.p + ni, yR.rs, yR.cs}, -1.0, 1.0));
+  } else
     FD_TRY(k_grouped_gemm(c, c.Kinv + ni, (long long)nr * nr, nr, nr, nd, cview(g), yR, c.delta, -1.0,
                           1.0, m, false, 0));
   FD_TRY(k_primal_extract(c, c.w_P1, c.nP, cp, m));

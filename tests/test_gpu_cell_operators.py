@@ -65,3 +65,34 @@ def test_fp64_cell_operators_for_every_rhs_count(kind, n_rhs):
     for r in range(n_rhs):
         assert _rel(y[r], ref.apply_F(lam[r])) < 1e-9
         assert _rel(z[r], ref.apply_MD(lam[r])) < 1e-11
+
+
+@pytest.mark.parametrize("cells", [(4, 3), (8, 3), (11, 3), (13, 5)])
+def test_fp64_principal_contractions_at_each_column_tile(cells):
+    """12, 24, 33 and 65 columns: the 16-, 32- and 64-wide tiles and their remainders, the trace tiles
+    and theirs.  Projections against the oracle, then Eq. 46a-b."""
+    from oracle import feti_dp, ifeti_dp
+    from oracle.discretization import Lattice
+    from paper_2308_11371_gb300 import binding
+    p = W.lattice_2d(cells[0], cells[1], 8, a=0.3, r=0.12, r_grade=0.03, n_rb=3)
+    lat = Lattice(p)
+    ref = ifeti_dp.InexactFETIDP(lat, blocks=[feti_dp.CellBlocks(lat, s) for s in range(lat.N)])
+    s = binding.Solver(p)
+    sigma, alpha, pi, delta = s.rom_data()
+    assert list(sigma) == list(ref.rom.sigma)
+    assert _rel(pi, ref.rom.pi) < 1e-9 and _rel(delta, ref.rom.delta) < 1e-9
+    v = np.random.default_rng(1).standard_normal((s.n_rhs, s.N, s.n_r))
+    x = s.local_rom_solve(_dev(v)).cpu().numpy()
+    assert _rel(x[0], ref.rom.local_rom_solve(v[0])) < 1e-9
+
+
+@pytest.mark.parametrize("cells", [(3, 2, 2), (13, 13, 13)])
+def test_identical_cells_converge_in_one_outer_iteration_fp64(cells):
+    """Identical cells make the reduced model exact, so the block preconditioner of Eq. 44 is the inverse
+    and FGMRES needs one iteration (a second only to confirm).  2,197 cells of 6^3 elements are above the
+    size up to which U_id_ring is assembled: both forms of Algorithm 3 are covered."""
+    from paper_2308_11371_gb300 import binding
+    p = W.lattice_3d(*cells, e=6, r=0.2, n_rb=1, mask_kind=W.MASK_BCC_SIGMOID)
+    s = binding.Solver(p)
+    u, lam, info = s.solve()
+    assert info["n_rb"] == 1 and info["outer_its"] <= 2 and info["rel_residual"] < 1e-8
