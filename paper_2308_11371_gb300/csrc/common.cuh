@@ -248,10 +248,16 @@ struct Ctx {
   int* corner_v = nullptr;    // [N*ncorner] free vertex index or -1 (A_p)
   int* vert_cells = nullptr;  // [nV*ncorner] (cell*ncorner + k) or -1 (A_p^T gather)
   double* r_dev = nullptr;    // [N]
-  // snapshots = C_hat at every Gauss point, [N][nsnap]
+  // snapshots = C_hat at every Gauss point, [N][nsnap]; released at the end of setup
   double* snap = nullptr;
-  // mixed path: FP32 element matrices [N][nelem][ND][ND] for the Eq. 46b K_s products
-  float* Ke_all = nullptr;
+  // sparse K_s of every cell, FP64 block-ELL over the cell's node graph (local node order):
+  // neighbour K_nbr[K_nk][n/d] (-1: none), neighbours per node, natural index of a local node, and
+  // values [N][K_nk][d*d][n/d]
+  int K_nk = 0;
+  int* K_nbr = nullptr;
+  int* K_cnt = nullptr;
+  int* K_nat = nullptr;
+  double* K_val = nullptr;
   // sparse K_rr of every cell in ELL form (mixed path, Eq. 46b): columns [nnz][nr] shared by all
   // cells, FP32 values [N][nnz][nr]
   int* krr_col = nullptr;
@@ -371,6 +377,7 @@ struct ProfScope {
 
 // ---------------------------------------------------------------- allocation
 fetidp_status dalloc(Ctx& c, void** p, size_t bytes);
+void dfree(Ctx& c, void* p, size_t bytes);   // gives one dalloc'ed block back before the context ends
 template <typename T>
 fetidp_status dalloc_t(Ctx& c, T** p, size_t count) {
   return dalloc(c, reinterpret_cast<void**>(p), count * sizeof(T));
@@ -450,8 +457,10 @@ fetidp_status k_gram_direct(Ctx& c, const double* Y, int ntab, const double* dve
                            double drop_rel);
 fetidp_status k_batched_diag_sum(Ctx& c, const double* A, long long stride, int lda, int r0, int m, int batch,
                                  double* out);
-fetidp_status k_apply_K(Ctx& c, CCellVec u, CellVec y, int nvec_per_col, int ncols, bool idp,
-                        bool r_only, const double* chat, double chat_scale_dr, int len_override = 0);
+fetidp_status k_apply_K(Ctx& c, CCellVec u, CellVec y, int nvec_per_col, int nrhs, int len);
+fetidp_status k_apply_K_natural(Ctx& c, CCellVec u, CellVec y, int nrhs);
+fetidp_status k_apply_K_split(Ctx& c, CCellVec ur, CCellVec up, CellVec yr, CellVec yp, int nrhs);
+fetidp_status k_krr_f32(Ctx& c);
 fetidp_status k_rom_combine_f32(Ctx& c, const double* src, long long kstride, int ld, int r0, int c0, int rows,
                                 int cols, const double* coef, float* out, int ldo, int symT = 0);
 fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
@@ -470,10 +479,8 @@ fetidp_status k_trace_gemm(Ctx& c, const double* A, int lda, int M, int K, const
 fetidp_status k_gram_solve(Ctx& c, const double* R, const double* KR, CCellVec v, CellVec x,
                            int nrhs, int len = -1);
 fetidp_status k_grad(Ctx& c, const double* u, const double* w, double* g);
-fetidp_status k_element_matrices_f32(Ctx& c);
-fetidp_status k_krr_ell_assemble(Ctx& c, const int* cnt, const int* idx, int cmax);
-fetidp_status k_apply_K_f32(Ctx& c, const float* u, long long u_rs, int u_cs, float* y, long long y_rs,
-                            int y_cs, int nvec, int nrhs, bool idp, bool r_only, long long ext = -1);
+fetidp_status k_krr_apply_f32(Ctx& c, const float* u, long long u_rs, int u_cs, float* y, long long y_rs,
+                              int y_cs, int nvec, int nrhs, long long ext = -1);
 fetidp_status k_gram_solve_f32(Ctx& c, const float* R, const float* KR, CCellVec v, CellVec x,
                                int nrhs, long long r_ext = -1);
 

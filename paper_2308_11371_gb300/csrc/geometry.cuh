@@ -158,6 +158,26 @@ FD_HD int chat_upper(int d, double nu, const double J[3][3], double E, double* o
   return c;
 }
 
+// Ji = J^-1 (row = xi component, column = x component); returns det J.
+FD_HD double jacobian_inverse(int d, const double J[3][3], double Ji[3][3]) {
+  if (d == 2) {
+    const double det = J[0][0] * J[1][1] - J[0][1] * J[1][0], id = 1.0 / det;
+    Ji[0][0] = J[1][1] * id; Ji[0][1] = -J[0][1] * id;
+    Ji[1][0] = -J[1][0] * id; Ji[1][1] = J[0][0] * id;
+    return det;
+  }
+  double det = 0.0;
+  for (int k = 0; k < 3; ++k)
+    det += J[0][k] * (J[1][(k + 1) % 3] * J[2][(k + 2) % 3] - J[1][(k + 2) % 3] * J[2][(k + 1) % 3]);
+  const double id = 1.0 / det;
+  for (int a = 0; a < 3; ++a)
+    for (int k = 0; k < 3; ++k) {
+      const int r1 = (k + 1) % 3, r2 = (k + 2) % 3, c1 = (a + 1) % 3, c2 = (a + 2) % 3;
+      Ji[a][k] = (J[r1][c1] * J[r2][c2] - J[r1][c2] * J[r2][c1]) * id;
+    }
+  return det;
+}
+
 // Lattice coordinate of Gauss point gp of element (ex,ey,ez) in cell (cx,cy,cz).
 FD_HD void gauss_point(const Geo& g, int cx, int cy, int cz, int ex, int ey, int ez, int gp,
                        double* eta, double* xi) {

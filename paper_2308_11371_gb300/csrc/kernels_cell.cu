@@ -1,11 +1,5 @@
-// Cell-level FP64 kernels of the hot path.
+// Cell-level kernels of the hot path.
 //
-// * snapshots: C_hat (Eq. 52) at every Gauss point of every cell; these are
-//   the snapshot vectors of the greedy (Sec. 4.2.2) and the per-Gauss-point
-//   macro data that the matrix-free K_s reads.
-// * apply_K: y = K_s u (Eq. 5a through Eq. 52), matrix-free Q1 element loop,
-//   elements processed in 2^d colours so that no two threads of a colour
-//   touch the same node (deterministic, no atomics).
 // * cell_gemv: per-cell dense operators assembled from the ROM (Eq. 43).
 // * grouped_gemm: Y = sum_k c_k (A_k X), one principal operator A_k serving
 //   every cell's column (Remark 7; Eq. 46a with separate outputs).
@@ -21,373 +15,11 @@ namespace {
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
-__global__ void snapshot_kernel(Geo g, const double* __restrict__ r_cell, long long ncell,
-                                int nelem, int ngp, int nc, double* __restrict__ snap) {
-  const long long total = ncell * nelem * ngp;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long cell = t / (nelem * ngp);
-    const int rem = (int)(t - cell * nelem * ngp);
-    const int el = rem / ngp, gp = rem - el * ngp;
-    const int cx = (int)(cell % g.nc[0]);
-    const int cy = (int)((cell / g.nc[0]) % g.nc[1]);
-    const int cz = (int)(cell / ((long long)g.nc[0] * g.nc[1]));
-    const int ex = el % g.e, ey = (el / g.e) % g.e, ez = el / (g.e * g.e);
-    double eta[3], xi[3], J[3][3];
-    gauss_point(g, cx, cy, cz, ex, ey, ez, gp, eta, xi);
-    macro_jacobian(g, xi, J);
-    const double E = youngs(g, strut_distance(g, eta), r_cell[cell]);
-    double out[45];
-    chat_upper(g.dim, g.nu, J, E, out);
-    double* dst = snap + cell * (long long)nelem * ngp * nc + (long long)rem * nc;
-    for (int k = 0; k < nc; ++k) dst[k] = out[k];
-  }
-}
-
-// Contribution of one Gauss point gp of one element: f = w dN^T C_hat(gp) dN u_e (Eq. 52).
-template <int D, typename T>
-__device__ __forceinline__ void gp_apply(const double* __restrict__ chat_gp, int gp, T wq, T inv_h, const T* ue,
-                                         T* fe) {
-  constexpr int NA = 1 << D;
-  constexpr int NI = D * D;
-  T t[D];
-  for (int k = 0; k < D; ++k) t[k] = (T)gauss_t((gp >> k) & 1);
-  T dN[NA][D];
-  for (int A = 0; A < NA; ++A)
-    for (int a = 0; a < D; ++a) {
-      T v = inv_h;
-      for (int k = 0; k < D; ++k) {
-        const int off = (A >> k) & 1;
-        if (k == a) v *= off ? T(1) : T(-1);
-        else v *= off ? t[k] : T(1) - t[k];
-      }
-      dN[A][a] = v;
-    }
-  T G[NI];
-  for (int I = 0; I < NI; ++I) G[I] = T(0);
-  for (int A = 0; A < NA; ++A)
-    for (int i = 0; i < D; ++i)
-      for (int a = 0; a < D; ++a) G[i * D + a] += ue[A * D + i] * dN[A][a];
-  T S[NI];
-  for (int I = 0; I < NI; ++I) S[I] = T(0);
-  int q = 0;
-  for (int I = 0; I < NI; ++I)
-    for (int J = I; J < NI; ++J) {
-      const T cij = (T)chat_gp[q++];
-      S[I] += cij * G[J];
-      if (J != I) S[J] += cij * G[I];
-    }
-  for (int A = 0; A < NA; ++A)
-    for (int i = 0; i < D; ++i) {
-      T v = T(0);
-      for (int a = 0; a < D; ++a) v += dN[A][a] * S[i * D + a];
-      fe[A * D + i] = wq * v;
-    }
-}
-
-// One block per (cell, rhs) column, the cell slowest (the RHS of a cell share its C_hat in L2);
-// vectors of the column processed VB at a time.  Within a colour group (elements that share no
-// node) one thread per (vector, element, Gauss point); the 2^D threads of an element are adjacent
-// lanes and sum their contributions with a fixed butterfly before one of them adds the element
-// into the column's shared accumulator.  T = double (FP64 path) or float.
-template <int D, typename T>
-__global__ void apply_K_kernel(int e, long long ncell, int n, int len, const int* __restrict__ perm,
-                               const int* __restrict__ iperm, bool idp, const T* __restrict__ u,
-                               long long u_rs, int u_cs, T* __restrict__ y, long long y_rs,
-                               int y_cs, int nvec, int VB, const double* __restrict__ chat, int nc,
-                               T wq, T inv_h, long long u_ext, long long y_ext) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  T* sm = reinterpret_cast<T*>(sm_raw);
-  constexpr int NA = 1 << D;
-  const int nrhs = (int)(gridDim.x / ncell);
-  const long long cell = blockIdx.x / nrhs;
-  const int rhs = (int)(blockIdx.x - cell * nrhs);
-  const T* uc = u + rhs * u_rs + cell * u_cs;
-  T* yc = y + rhs * y_rs + cell * y_cs;
-  const double* chat_cell = chat + cell * (long long)nc * NA * (e * e * (D == 3 ? e : 1));
-  T* us = sm;
-  T* ys = sm + (size_t)VB * n;
-  const int ecount[3] = {e, e, D == 3 ? e : 1};
-  for (int v0 = 0; v0 < nvec; v0 += VB) {
-    const int vb = min(VB, nvec - v0);
-    for (int t = threadIdx.x; t < vb * n; t += blockDim.x) {
-      const int v = t / n, i = t - v * n;     // i natural index
-      T val;
-      if (idp) {
-        const int li = iperm[i];
-        val = (li < len && FD_INB(rhs * u_rs + cell * u_cs + (long long)(v0 + v) * len + li, u_ext, 201))
-                  ? uc[(size_t)(v0 + v) * len + li]
-                  : T(0);
-      } else {
-        val = FD_INB(rhs * u_rs + cell * u_cs + (long long)(v0 + v) * len + i, u_ext, 201)
-                  ? uc[(size_t)(v0 + v) * len + i]
-                  : T(0);
-      }
-      us[t] = val;
-      ys[t] = T(0);
-    }
-    __syncthreads();
-    for (int color = 0; color < NA; ++color) {
-      int cnt[3], par[3];
-      int nel = 1;
-      for (int k = 0; k < 3; ++k) {
-        par[k] = (k < D) ? ((color >> k) & 1) : 0;
-        cnt[k] = (k < D) ? (ecount[k] - par[k] + 1) / 2 : 1;
-        nel *= cnt[k];
-      }
-      // uniform trip count (total and blockDim are multiples of NA): every lane reaches the shuffles
-      const int total = vb * nel * NA;
-      for (int t0 = 0; t0 < total; t0 += blockDim.x) {
-        const int t = t0 + threadIdx.x;
-        const bool live = t < total;
-        const int gp = t & (NA - 1);
-        const int vq = live ? t / NA : 0;
-        const int v = vq / nel, q = vq - v * nel;
-        const int qx = q % cnt[0], qy = (q / cnt[0]) % cnt[1], qz = q / (cnt[0] * cnt[1]);
-        const int ex = par[0] + 2 * qx, ey = par[1] + 2 * qy, ez = par[2] + 2 * qz;
-        const int el = ex + e * (ey + e * ez);
-        int nodes[NA];
-        for (int A = 0; A < NA; ++A) {
-          const int ax = A & 1, ay = (A >> 1) & 1, az = (A >> 2) & 1;
-          nodes[A] = (ex + ax) + (e + 1) * ((ey + ay) + (e + 1) * (D == 3 ? (ez + az) : 0));
-        }
-        T ue[NA * D], fe[NA * D];
-        const T* uv = us + (size_t)v * n;
-        for (int A = 0; A < NA; ++A)
-          for (int i = 0; i < D; ++i) ue[A * D + i] = live ? uv[nodes[A] * D + i] : T(0);
-        gp_apply<D, T>(chat_cell + ((size_t)el * NA + gp) * nc, gp, wq, inv_h, ue, fe);
-#pragma unroll
-        for (int k = 0; k < NA * D; ++k)
-          for (int o = 1; o < NA; o <<= 1) fe[k] += __shfl_xor_sync(0xffffffffu, fe[k], o);
-        if (live && gp == 0) {
-          T* yv = ys + (size_t)v * n;
-          for (int A = 0; A < NA; ++A)
-            for (int i = 0; i < D; ++i) yv[nodes[A] * D + i] += fe[A * D + i];
-        }
-      }
-      __syncthreads();
-    }
-    for (int t = threadIdx.x; t < vb * len; t += blockDim.x) {
-      const int v = t / len, li = t - v * len;
-      const int nat = idp ? perm[li] : li;
-      if (FD_INB(rhs * y_rs + cell * y_cs + (long long)(v0 + v) * len + li, y_ext, 202))
-        yc[(size_t)(v0 + v) * len + li] = ys[(size_t)v * n + nat];
-    }
-    __syncthreads();
-  }
-}
-
-// Index of entry (I, J) of a symmetric d^2 x d^2 matrix kept as its upper triangle, row-major.
-__device__ __forceinline__ int sym_index(int I, int J, int NI) {
-  if (I > J) { const int t = I; I = J; J = t; }
-  return I * NI - I * (I - 1) / 2 + (J - I);
-}
-
-// Element matrices K_e = sum_gp w B^T C_hat B of every element of every cell in FP32 (C_hat
-// rounded to FP32 first), row-major ND x ND, for the Eq. 46b products of the mixed path.  They
-// depend on the cell's C_hat only, so they are formed once per setup instead of in every local
-// ROM solve.  One thread per (cell, element, row (A, i)).
-constexpr int kMultiThreads = 512;
-template <int D>
-__global__ void element_matrices_f32_kernel(const double* __restrict__ chat, long long ncell, int e, int nc,
-                                            float wq, float inv_h, float* __restrict__ Kall) {
-  constexpr int NA = 1 << D;
-  constexpr int ND = NA * D;
-  constexpr int NI = D * D;
-  const int nel = e * e * (D == 3 ? e : 1);
-  const int cpe = NA * nc;
-  const long long total = ncell * nel * ND;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int row = (int)(t % ND);
-    const long long ce = t / ND;                    // cell * nel + el
-    const int A = row / D, i = row - A * D;
-    const double* Ce = chat + ce * cpe;
-    float krow[ND];
-#pragma unroll
-    for (int k = 0; k < ND; ++k) krow[k] = 0.f;
-    for (int gp = 0; gp < NA; ++gp) {
-      float dn[NA * D];                             // shape-function gradients at this Gauss point
-#pragma unroll
-      for (int B = 0; B < NA; ++B)
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          float v = inv_h;
-#pragma unroll
-          for (int k = 0; k < D; ++k) {
-            const int off = (B >> k) & 1;
-            const float tk = (float)gauss_t((gp >> k) & 1);
-            if (k == a) v *= off ? 1.f : -1.f;
-            else v *= off ? tk : 1.f - tk;
-          }
-          dn[B * D + a] = v;
-        }
-      float w[D][D];   // w[j][b] = sum_a dN_A[a] C[(i,a),(j,b)]
-#pragma unroll
-      for (int j = 0; j < D; ++j)
-#pragma unroll
-        for (int b = 0; b < D; ++b) {
-          float sacc = 0.f;
-#pragma unroll
-          for (int a = 0; a < D; ++a)
-            sacc += dn[A * D + a] * (float)Ce[gp * nc + sym_index(i * D + a, j * D + b, NI)];
-          w[j][b] = sacc;
-        }
-#pragma unroll
-      for (int B = 0; B < NA; ++B)
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          float sacc = 0.f;
-#pragma unroll
-          for (int b = 0; b < D; ++b) sacc += w[j][b] * dn[B * D + b];
-          krow[B * D + j] += wq * sacc;
-        }
-    }
-    float* kr = Kall + t * ND;
-#pragma unroll
-    for (int k = 0; k < ND; k += 4)
-      *reinterpret_cast<float4*>(kr + k) = make_float4(krow[k], krow[k + 1], krow[k + 2], krow[k + 3]);
-  }
-}
-
-// Multi-vector K_s application in FP32 (the Eq. 46b products K_s R of the mixed path).  One
-// block per (cell, rhs, chunk of VB vectors), the cell slowest: the blocks of one cell run side
-// by side and read its element matrices from L2, not once per chunk from HBM.  For each colour group (elements that share no node) the precomputed
-// element matrices of its elements are staged in shared memory (contiguous, coalesced) and
-// applied to all vectors of the chunk, one thread per (element, vector).  Vectors are stored
-// dof-major with a padded stride, so the threads of an element read consecutive words and every
-// K_e entry is a broadcast.  Global vectors are read and written in local order through the
-// staged permutation, so no load depends on another.
-// padded K_e row stride (in floats): 4 mod 32 so that neighbouring elements hit different banks;
-// rows stay 16-byte aligned
-__host__ __device__ constexpr int multi_ke_stride(int D) { return (D == 2 ? 64 : 576) + 4; }
-template <int D>
-__global__ void __launch_bounds__(kMultiThreads, 2) apply_K_multi_kernel(
-    int e, long long ncell, int n, int len, const int* __restrict__ perm, bool idp,
-    const float* __restrict__ u, long long u_rs, int u_cs, float* __restrict__ y, long long y_rs, int y_cs,
-    int nvec, int VB, int nchunk, int nrhs, const float* __restrict__ Kall, int nelc_max, long long u_ext,
-    long long y_ext) {
-  constexpr int NA = 1 << D;
-  constexpr int ND = NA * D;
-  constexpr int KES = multi_ke_stride(D);
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int VBp = VB + 1;
-  float* us = reinterpret_cast<float*>(sm_raw);        // [n][VBp]
-  float* ys = us + (size_t)n * VBp;                     // [n][VBp]
-  float* Ke = ys + (size_t)n * VBp;                     // [nelc_max][KES], rows of ND
-  Ke = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(Ke) + 15) & ~uintptr_t(15));
-  int* perm_s = reinterpret_cast<int*>(Ke + (size_t)nelc_max * KES);   // [n] local -> natural
-  const int chunk = (int)(blockIdx.x % nchunk);
-  const long long rest = blockIdx.x / nchunk;
-  const int rhs = (int)(rest % nrhs);
-  const long long cell = rest / nrhs;
-  const float* uc = u + rhs * u_rs + cell * u_cs;
-  float* yc = y + rhs * y_rs + cell * y_cs;
-  const int nel = e * e * (D == 3 ? e : 1);
-  const float* Kcell = Kall + cell * (long long)nel * ND * ND;
-  const int ecount[3] = {e, e, D == 3 ? e : 1};
-  for (int li = threadIdx.x; li < n; li += blockDim.x) perm_s[li] = idp ? perm[li] : li;
-  __syncthreads();
-  {
-    const int v0 = chunk * VB;
-    const int vb = min(VB, nvec - v0);
-#pragma unroll 4
-    for (int t = threadIdx.x; t < vb * len; t += blockDim.x) {
-      const int v = t / len, li = t - v * len;
-      float val = 0.f;
-      if (FD_INB(rhs * u_rs + cell * u_cs + (long long)(v0 + v) * len + li, u_ext, 203))
-        val = uc[(size_t)(v0 + v) * len + li];
-      us[(size_t)perm_s[li] * VBp + v] = val;
-    }
-    for (int t = threadIdx.x; t < vb * (n - len); t += blockDim.x) {   // dofs outside the vector
-      const int v = t / (n - len), r = t - v * (n - len);
-      us[(size_t)perm_s[len + r] * VBp + v] = 0.f;
-    }
-    for (int t = threadIdx.x; t < n * VBp; t += blockDim.x) ys[t] = 0.f;
-    for (int color = 0; color < NA; ++color) {
-      int cnt[3], par[3];
-      int nelc = 1;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        par[k] = (k < D) ? ((color >> k) & 1) : 0;
-        cnt[k] = (k < D) ? (ecount[k] - par[k] + 1) / 2 : 1;
-        nelc *= cnt[k];
-      }
-      __syncthreads();   // previous colour's K_e no longer read
-      // the colour's element matrices, 16-byte loads
-      for (int t = threadIdx.x; t < nelc * ND * (ND / 4); t += blockDim.x) {
-        const int q = t / (ND * ND / 4), r = t - q * (ND * ND / 4);
-        const int qx = q % cnt[0], qy = (q / cnt[0]) % cnt[1], qz = q / (cnt[0] * cnt[1]);
-        const int el = (par[0] + 2 * qx) + e * ((par[1] + 2 * qy) + e * (par[2] + 2 * qz));
-        const int row = (4 * r) / ND, k = 4 * r - row * ND;
-        *reinterpret_cast<float4*>(Ke + (size_t)q * KES + row * ND + k) =
-            *reinterpret_cast<const float4*>(Kcell + ((size_t)el * ND + row) * ND + k);
-      }
-      __syncthreads();
-      // apply to every vector of the chunk
-      for (int t = threadIdx.x; t < nelc * vb; t += blockDim.x) {
-        const int q = t / vb, v = t - q * vb;
-        const int qx = q % cnt[0], qy = (q / cnt[0]) % cnt[1], qz = q / (cnt[0] * cnt[1]);
-        const int ex = par[0] + 2 * qx, ey = par[1] + 2 * qy, ez = par[2] + 2 * qz;
-        int dof0[NA];
-#pragma unroll
-        for (int B = 0; B < NA; ++B) {
-          const int bx = B & 1, by = (B >> 1) & 1, bz = (B >> 2) & 1;
-          dof0[B] = D * ((ex + bx) + (e + 1) * ((ey + by) + (e + 1) * (D == 3 ? (ez + bz) : 0)));
-        }
-        float ue[ND];
-#pragma unroll
-        for (int B = 0; B < NA; ++B)
-#pragma unroll
-          for (int j = 0; j < D; ++j) ue[B * D + j] = us[(size_t)(dof0[B] + j) * VBp + v];
-        const float* kq = Ke + (size_t)q * KES;
-#pragma unroll
-        for (int A = 0; A < NA; ++A)
-#pragma unroll
-          for (int i = 0; i < D; ++i) {
-            const float* kr = kq + (A * D + i) * ND;
-            float sacc = 0.f;
-#pragma unroll
-            for (int k = 0; k < ND; k += 4) {
-              const float4 k4 = *reinterpret_cast<const float4*>(kr + k);
-              sacc += k4.x * ue[k] + k4.y * ue[k + 1] + k4.z * ue[k + 2] + k4.w * ue[k + 3];
-            }
-            ys[(size_t)(dof0[A] + i) * VBp + v] += sacc;
-          }
-      }
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int t = threadIdx.x; t < vb * len; t += blockDim.x) {
-      const int v = t / len, li = t - v * len;
-      if (FD_INB(rhs * y_rs + cell * y_cs + (long long)(v0 + v) * len + li, y_ext, 204))
-        yc[(size_t)(v0 + v) * len + li] = ys[(size_t)perm_s[li] * VBp + v];
-    }
-    __syncthreads();
-  }
-}
-
 // ---- K_rr^(s) R for many vectors as a sparse product (Eq. 46b, mixed path)
 // Every cell has the same sparsity pattern, so K_rr^(s) (remaining DOF, local (i, d) order) is
 // stored in ELL form: one column table [slot][row] shared by all cells and FP32 values
-// [cell][slot][row] (row fastest, so a warp's 32 rows read 128 contiguous bytes per slot).  The
-// values are summed from the element matrices once per setup, in a fixed order.
-
-// val[cell][slot][row] = sum over the entry's contributions of Ke[cell][el][a][b]
-__global__ void krr_ell_assemble_kernel(const float* __restrict__ Ke, long long ke_cell, const int* __restrict__ cnt,
-                                        const int* __restrict__ idx, int cmax, int nnz, int nr, long long ncell,
-                                        float* __restrict__ val) {
-  const long long per = (long long)nnz * nr;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < ncell * per;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long cell = t / per;
-    const int e = (int)(t - cell * per);
-    const float* kc = Ke + cell * ke_cell;
-    float v = 0.f;
-    for (int q = 0; q < cnt[e]; ++q) v += kc[idx[(long long)e * cmax + q]];
-    val[t] = v;
-  }
-}
+// [cell][slot][row] (row fastest, so a warp's 32 rows read 128 contiguous bytes per slot), rounded
+// once per setup from the FP64 K_s.
 
 constexpr int kSpVB = 16;   // vectors per block
 constexpr int kSpLd = 20;   // shared row stride (floats): 16 vectors + 4, conflict-free 16-byte reads
@@ -1784,158 +1416,32 @@ __global__ void grad_kernel(Geo g, const double* __restrict__ r_cell, long long 
 
 }  // namespace
 
-fetidp_status k_snapshots(Ctx& c) {
-  ProfScope ps(c, FETIDP_K_SETUP, 0.0, (double)c.N * c.nsnap * 8.0);
-  const long long total = c.N * c.nelem * c.ngp;
-  int grid = ceil_div(total, 256);
-  if (grid > 152 * 32) grid = 152 * 32;
-  for (const LatticeSpan& ls : c.lat) {   // one launch per lattice: its own geometry and radii
-    snapshot_kernel<<<grid, 256, 0, c.stream>>>(ls.geo, c.r_dev + ls.cell0, ls.ncell, c.nelem, c.ngp, c.nc,
-                                                c.snap + ls.cell0 * c.nsnap);
-    FD_CHECK_LAUNCH();
-  }
-  return FETIDP_OK;
-}
-
-// u, y: column (rhs, cell) holds nvec vectors of length len (n, or n_r when r_only).
-fetidp_status k_apply_K(Ctx& c, CCellVec u, CellVec y, int nvec, int nrhs, bool idp, bool r_only,
-                        const double* chat, double /*unused*/, int len_override) {
-  const int len = len_override > 0 ? len_override : (r_only ? c.nr : c.n);
-  const int VB = nvec < 8 ? nvec : 8;
-  {
-    const double D = c.d, NA = c.ngp;
-    const double fma = NA * D * D * 2.0 + D * D * D * D;   // gradient + stress + scatter per gp
-    const double cols = (double)c.N * nrhs;
-    c.prof_pending_flops = 2.0 * fma * c.nelem * c.ngp * nvec * cols;
-    c.prof_pending_bytes = cols * (c.nsnap * 8.0 + 2.0 * nvec * len * 8.0);
-  }
-  ProfScope ps(c, FETIDP_K_APPLY_K, c.prof_pending_flops, c.prof_pending_bytes);
-  const size_t smem = 2 * (size_t)VB * c.n * sizeof(double);
-  const double h = 1.0 / c.e;
-  const double wq = pow(0.5 * h, c.d);
-  const dim3 grid((unsigned)(c.N * nrhs));
-  if (c.d == 2) {
-    cudaFuncSetAttribute(apply_K_kernel<2, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    apply_K_kernel<2, double><<<grid, 256, smem, c.stream>>>(
-        c.e, c.N, c.n, len, c.perm, c.perm + c.n, idp, u.p, u.rs, u.cs, y.p, y.rs, y.cs, nvec, VB,
-        chat, c.nc, wq, 1.0 / h, u.ext, y.ext);
-  } else {
-    cudaFuncSetAttribute(apply_K_kernel<3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    apply_K_kernel<3, double><<<grid, 256, smem, c.stream>>>(
-        c.e, c.N, c.n, len, c.perm, c.perm + c.n, idp, u.p, u.rs, u.cs, y.p, y.rs, y.cs, nvec, VB,
-        chat, c.nc, wq, 1.0 / h, u.ext, y.ext);
-  }
-  FD_CHECK_LAUNCH();
-  return FETIDP_OK;
-}
-
-// FP32 element matrices of every cell (mixed path), formed once per setup.
-fetidp_status k_krr_ell_assemble(Ctx& c, const int* cnt, const int* idx, int cmax) {
-  const int NA = 1 << c.d, ND = NA * c.d;
-  FD_TRY(dalloc_t(c, &c.krr_val, (size_t)c.N * c.krr_nnz * c.nr));
-  ProfScope ps(c, FETIDP_K_SETUP, 0.0, 4.0 * (double)c.N * c.krr_nnz * c.nr * 2.0);
-  const long long work = c.N * (long long)c.krr_nnz * c.nr;
-  const int grid = (int)std::min<long long>((work + 255) / 256, 152LL * 64);
-  krr_ell_assemble_kernel<<<grid, 256, 0, c.stream>>>(c.Ke_all, (long long)c.nelem * ND * ND, cnt, idx, cmax,
-                                                     c.krr_nnz, c.nr, c.N, c.krr_val);
-  FD_CHECK_LAUNCH();
-  return FETIDP_OK;
-}
-
-fetidp_status k_element_matrices_f32(Ctx& c) {
-  const int NA = 1 << c.d, ND = NA * c.d;
-  FD_TRY(dalloc_t(c, &c.Ke_all, (size_t)c.N * c.nelem * ND * ND));
-  ProfScope ps(c, FETIDP_K_SETUP, 0.0, (double)c.N * (c.nsnap * 8.0 + (double)c.nelem * ND * ND * 4.0));
-  const float h = 1.0f / c.e;
-  const float wq = (float)pow(0.5 / c.e, c.d);
-  const long long work = c.N * c.nelem * ND;
-  const int grid = (int)std::min<long long>((work + 255) / 256, 152LL * 64);
-  if (c.d == 2)
-    element_matrices_f32_kernel<2><<<grid, 256, 0, c.stream>>>(c.snap, c.N, c.e, c.nc, wq, 1.0f / h, c.Ke_all);
-  else
-    element_matrices_f32_kernel<3><<<grid, 256, 0, c.stream>>>(c.snap, c.N, c.e, c.nc, wq, 1.0f / h, c.Ke_all);
-  FD_CHECK_LAUNCH();
-  return FETIDP_OK;
-}
-
-// FP32 variant (local ROM bases of the mixed path): u, y float with the same view strides.
-fetidp_status k_apply_K_f32(Ctx& c, const float* u, long long u_rs, int u_cs, float* y, long long y_rs,
-                            int y_cs, int nvec, int nrhs, bool idp, bool r_only, long long ext) {
-  if (idp && r_only && c.krr_val) {   // sparse K_rr in ELL form
-    const int nchunk = (nvec + kSpVB - 1) / kSpVB;
-    const size_t smem = (size_t)c.nr * kSpLd * sizeof(float);
-    // algorithmic work: one FMA per stored entry and vector; bytes: the values once per cell, the
-    // vectors in and out
-    ProfScope ps(c, FETIDP_K_MULTI_K, 2.0 * (double)c.N * nrhs * nvec * c.krr_nnz * c.nr,
-                 4.0 * (double)c.N * c.krr_nnz * c.nr + 8.0 * (double)c.N * nrhs * nvec * c.nr);
-    const int nnode = c.nr / c.d;
-    const size_t smem_n = smem + sizeof(float) * 2 * (size_t)c.d * c.nr;
-    if (c.krr_nbr && nnode <= 352 && smem_n <= 113 * 1024) {
-      const int threads = (nnode + 31) / 32 * 32;
-      if (c.d == 3) {
-        cudaFuncSetAttribute(krr_spmm_nodal_f32_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_n);
-        krr_spmm_nodal_f32_kernel<3><<<(unsigned)(c.N * nrhs * nchunk), threads, smem_n, c.stream>>>(
-            c.krr_nbr, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
-      } else {
-        cudaFuncSetAttribute(krr_spmm_nodal_f32_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_n);
-        krr_spmm_nodal_f32_kernel<2><<<(unsigned)(c.N * nrhs * nchunk), threads, smem_n, c.stream>>>(
-            c.krr_nbr, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
-      }
+// K_rr^(s) times nvec FP32 vectors per (rhs, cell) column (the local ROM bases of the mixed path).
+fetidp_status k_krr_apply_f32(Ctx& c, const float* u, long long u_rs, int u_cs, float* y, long long y_rs,
+                              int y_cs, int nvec, int nrhs, long long ext) {
+  const int nchunk = (nvec + kSpVB - 1) / kSpVB;
+  const size_t smem = (size_t)c.nr * kSpLd * sizeof(float);
+  // algorithmic work: one FMA per stored entry and vector; bytes: the values once per cell, the
+  // vectors in and out
+  ProfScope ps(c, FETIDP_K_MULTI_K, 2.0 * (double)c.N * nrhs * nvec * c.krr_nnz * c.nr,
+               4.0 * (double)c.N * c.krr_nnz * c.nr + 8.0 * (double)c.N * nrhs * nvec * c.nr);
+  const int nnode = c.nr / c.d;
+  const size_t smem_n = smem + sizeof(float) * 2 * (size_t)c.d * c.nr;
+  if (c.krr_nbr && nnode <= 352 && smem_n <= 113 * 1024) {
+    const int threads = (nnode + 31) / 32 * 32;
+    if (c.d == 3) {
+      cudaFuncSetAttribute(krr_spmm_nodal_f32_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_n);
+      krr_spmm_nodal_f32_kernel<3><<<(unsigned)(c.N * nrhs * nchunk), threads, smem_n, c.stream>>>(
+          c.krr_nbr, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
     } else {
-      cudaFuncSetAttribute(krr_spmm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      krr_spmm_f32_kernel<<<(unsigned)(c.N * nrhs * nchunk), 256, smem, c.stream>>>(
-          c.krr_col, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
+      cudaFuncSetAttribute(krr_spmm_nodal_f32_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_n);
+      krr_spmm_nodal_f32_kernel<2><<<(unsigned)(c.N * nrhs * nchunk), threads, smem_n, c.stream>>>(
+          c.krr_nbr, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
     }
-    FD_CHECK_LAUNCH();
-    return FETIDP_OK;
-  }
-  if (!c.Ke_all) {
-    set_error("multi-vector K_s: element matrices not formed");
-    return FETIDP_EINVAL;
-  }
-  const int len = r_only ? c.nr : c.n;
-  const int NA = 1 << c.d, ND = NA * c.d;
-  const int half = (c.e + 1) / 2;
-  const int nelc_max = half * half * (c.d == 3 ? half : 1);
-  const int kes = c.d == 2 ? multi_ke_stride(2) : multi_ke_stride(3);
-  const size_t fixed = (size_t)nelc_max * kes * sizeof(float) + 16 + (size_t)c.n * sizeof(int);
-  // vectors per chunk: as many as fit beside one colour's element matrices (<= 16) with two
-  // blocks per SM (one block's global loads and stores overlap the other's arithmetic), else
-  // as many as fit with one
-  auto bytes = [&](int vb) { return fixed + 2 * (size_t)c.n * (vb + 1) * sizeof(float); };
-  size_t budget = 110 * 1024;
-  int VB = (int)std::min<long long>(16, nvec);
-  while (VB > 1 && bytes(VB) > budget) --VB;
-  if (bytes(VB) > budget) {
-    budget = 220 * 1024;
-    VB = (int)std::min<long long>(32, nvec);
-    while (VB > 1 && bytes(VB) > budget) --VB;
-  }
-  if (bytes(VB) > budget) {
-    set_error("multi-vector K_s: cell too large for shared memory");
-    return FETIDP_EINVAL;
-  }
-  {
-    // algorithmic work: one K_e product (ND^2 FMA) per element and vector; bytes: the element
-    // matrices once per cell, the vectors in and out
-    const double cols = (double)c.N * nrhs;
-    c.prof_pending_flops = 2.0 * cols * c.nelem * (double)nvec * ND * ND;
-    c.prof_pending_bytes = (double)c.N * c.nelem * (double)ND * ND * 4.0 + cols * 2.0 * nvec * len * 4.0;
-  }
-  ProfScope ps(c, FETIDP_K_MULTI_K, c.prof_pending_flops, c.prof_pending_bytes);
-  const size_t smem = bytes(VB);
-  const int nchunk = (nvec + VB - 1) / VB;
-  const dim3 grid((unsigned)(c.N * nrhs * nchunk));
-  if (c.d == 2) {
-    cudaFuncSetAttribute(apply_K_multi_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    apply_K_multi_kernel<2><<<grid, kMultiThreads, smem, c.stream>>>(
-        c.e, c.N, c.n, len, c.perm, idp, u, u_rs, u_cs, y, y_rs, y_cs, nvec, VB, nchunk, nrhs, c.Ke_all, nelc_max,
-        ext, ext);
   } else {
-    cudaFuncSetAttribute(apply_K_multi_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    apply_K_multi_kernel<3><<<grid, kMultiThreads, smem, c.stream>>>(
-        c.e, c.N, c.n, len, c.perm, idp, u, u_rs, u_cs, y, y_rs, y_cs, nvec, VB, nchunk, nrhs, c.Ke_all, nelc_max,
-        ext, ext);
+    cudaFuncSetAttribute(krr_spmm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    krr_spmm_f32_kernel<<<(unsigned)(c.N * nrhs * nchunk), 256, smem, c.stream>>>(
+        c.krr_col, c.krr_val, c.krr_nnz, c.nr, nrhs, nchunk, u, u_rs, u_cs, y, y_rs, y_cs, nvec, ext);
   }
   FD_CHECK_LAUNCH();
   return FETIDP_OK;

@@ -5,12 +5,12 @@
 // GPU: snapshots (Eq. 52), the greedy passes of Algorithm 4, the projection
 // traces of Eq. 42 (one GEMM against the snapshot matrix) and the ROM local
 // operators of Eq. 43.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
 #include <thread>
 
 #include "common.cuh"
@@ -533,6 +533,36 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   phase("primal maps + loads");
 
   // ---------------------------------------------------------------- snapshots (Eq. 52)
+  // node graph of the reference cell in local order: the up to 3^d nodes that share an element
+  std::vector<int> K_nbr;
+  {
+    const int nn = c.n / d;
+    std::vector<int> nat(nn), loc(nn), cnt(nn, 0);
+    for (int n = 0; n < nn; ++n) {
+      nat[n] = ref.perm[(size_t)n * d] / d;
+      loc[nat[n]] = n;
+    }
+    c.K_nk = d == 2 ? 9 : 27;
+    K_nbr.assign((size_t)c.K_nk * nn, -1);
+    for (int n = 0; n < nn; ++n) {
+      const int ijk[3] = {nat[n] % nn1, (nat[n] / nn1) % nn1, d == 3 ? nat[n] / (nn1 * nn1) : 0};
+      std::vector<int> list;
+      for (int dz = d == 3 ? -1 : 0; dz <= (d == 3 ? 1 : 0); ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+          for (int dx = -1; dx <= 1; ++dx) {
+            const int q[3] = {ijk[0] + dx, ijk[1] + dy, ijk[2] + dz};
+            if (q[0] < 0 || q[0] > e || q[1] < 0 || q[1] > e || q[2] < 0 || (d == 3 && q[2] > e)) continue;
+            list.push_back(loc[q[0] + nn1 * (q[1] + nn1 * q[2])]);
+          }
+      std::sort(list.begin(), list.end());
+      cnt[n] = (int)list.size();
+      for (size_t k = 0; k < list.size(); ++k) K_nbr[k * nn + n] = list[k];
+    }
+    FD_TRY(upload(c, &c.K_nbr, K_nbr));
+    FD_TRY(upload(c, &c.K_cnt, cnt));
+    FD_TRY(upload(c, &c.K_nat, nat));
+    FD_CUDA(cudaStreamSynchronize(c.stream));   // host tables go out of scope
+  }
   FD_TRY(dalloc_t(c, &c.snap, (size_t)c.N * c.nsnap));
   FD_TRY(k_snapshots(c));
   phase("snapshots");
@@ -753,74 +783,31 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
       FD_TRY(k_rom_combine(c, c.Kinv, (long long)nr * nr, nr, ni, 0, nd, ni, c.delta, c.Udi_c));
     }
   } else {          // mixed path: principal operators packed for the tensor cores
-    FD_TRY(k_element_matrices_f32(c));
     {
-      // ELL pattern of K_rr on the reference cell (remaining DOF, local order) and, for each
-      // stored entry, the element-matrix entries that sum into it (at most 2^d, fixed order)
-      const int d = c.d, e = c.e, NA = 1 << d, ND = NA * d, nn1 = e + 1;
-      std::vector<std::map<int, std::vector<int>>> rows(nr);
-      for (int el = 0; el < c.nelem; ++el) {
-        const int ex = el % e, ey = (el / e) % e, ez = d == 3 ? el / (e * e) : 0;
-        for (int a = 0; a < ND; ++a) {
-          const int A = a / d, ia = a % d;
-          const int na = (ex + (A & 1)) + nn1 * ((ey + ((A >> 1) & 1)) + nn1 * (d == 3 ? ez + ((A >> 2) & 1) : 0));
-          const int ga = ref.iperm[na * d + ia];
-          if (ga >= nr) continue;
-          for (int b = 0; b < ND; ++b) {
-            const int B = b / d, ib = b % d;
-            const int nb = (ex + (B & 1)) + nn1 * ((ey + ((B >> 1) & 1)) + nn1 * (d == 3 ? ez + ((B >> 2) & 1) : 0));
-            const int gb = ref.iperm[nb * d + ib];
-            if (gb >= nr) continue;
-            rows[ga][gb].push_back(el * ND * ND + a * ND + b);
-          }
-        }
+      // FP32 ELL form of K_rr from the sparse K_s: the remaining neighbours of a remaining node are the
+      // first slots of its list (local order), padding slots point at the node itself with value 0
+      const int nnode = nr / d, nn = c.n / d;
+      int nk = 0;
+      for (int n = 0; n < nnode; ++n) {
+        int k = 0;
+        while (k < c.K_nk && K_nbr[(size_t)k * nn + n] >= 0 && K_nbr[(size_t)k * nn + n] < nnode) ++k;
+        nk = std::max(nk, k);
       }
-      int nnz = 0;
-      for (const auto& r : rows) nnz = std::max(nnz, (int)r.size());
-      const int cmax = NA;
-      std::vector<int> col((size_t)nnz * nr), cnt((size_t)nnz * nr, 0), idx((size_t)nnz * nr * cmax, 0);
-      for (int r = 0; r < nr; ++r) {
-        int sl = 0;
-        for (const auto& kv : rows[r]) {
-          col[(size_t)sl * nr + r] = kv.first;
-          cnt[(size_t)sl * nr + r] = (int)kv.second.size();
-          for (size_t q = 0; q < kv.second.size() && q < (size_t)cmax; ++q)
-            idx[((size_t)sl * nr + r) * cmax + q] = kv.second[q];
-          ++sl;
+      std::vector<int> nbr((size_t)nk * nnode), col((size_t)nk * d * nr);
+      for (int k = 0; k < nk; ++k)
+        for (int n = 0; n < nnode; ++n) {
+          const int mq = K_nbr[(size_t)k * nn + n];
+          const bool pad = mq < 0 || mq >= nnode;
+          nbr[(size_t)k * nnode + n] = pad ? n : mq;
+          for (int cq = 0; cq < d; ++cq)
+            for (int a = 0; a < d; ++a)
+              col[((size_t)k * d + cq) * nr + (size_t)d * n + a] = pad ? d * n + a : d * mq + cq;
         }
-        for (; sl < nnz; ++sl) col[(size_t)sl * nr + r] = r;   // padding: value 0 on the diagonal column
-      }
-      c.krr_nnz = nnz;
-      // nodal structure: the d rows of a node share their neighbour nodes, slot d k + c' of row
-      // d n + a holding component c' of the k-th neighbour (columns sorted, components interleaved)
-      bool nodal = nr % d == 0 && nnz % d == 0;
-      const int nnode = nr / d, nk = nnz / d;
-      std::vector<int> nbr;
-      if (nodal) nbr.assign((size_t)nk * nnode, 0);
-      for (int n = 0; nodal && n < nnode; ++n)
-        for (int k = 0; nodal && k < nk; ++k) {
-          const size_t e0 = (size_t)(d * k) * nr + (size_t)d * n;
-          const bool pad = cnt[e0] == 0;
-          const int c0 = col[e0];
-          if (!pad && c0 % d != 0) nodal = false;
-          for (int a = 0; nodal && a < d; ++a)
-            for (int cq = 0; cq < d; ++cq) {
-              const size_t e = (size_t)(d * k + cq) * nr + (size_t)d * n + a;
-              if ((cnt[e] == 0) != pad || (!pad && col[e] != c0 + cq)) { nodal = false; break; }
-            }
-          if (nodal) nbr[(size_t)k * nnode + n] = pad ? n : c0 / d;
-        }
-      if (nodal) FD_TRY(upload(c, &c.krr_nbr, nbr));
-      int *cnt_d = nullptr, *idx_d = nullptr;
+      c.krr_nnz = nk * d;
+      FD_TRY(upload(c, &c.krr_nbr, nbr));
       FD_TRY(upload(c, &c.krr_col, col));
-      FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&cnt_d), sizeof(int) * cnt.size()));
-      FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&idx_d), sizeof(int) * idx.size()));
-      FD_CUDA(cudaMemcpyAsync(cnt_d, cnt.data(), sizeof(int) * cnt.size(), cudaMemcpyHostToDevice, c.stream));
-      FD_CUDA(cudaMemcpyAsync(idx_d, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice, c.stream));
-      FD_TRY(k_krr_ell_assemble(c, cnt_d, idx_d, cmax));
-      FD_CUDA(cudaStreamSynchronize(c.stream));
-      tmp_free(c, cnt_d);
-      tmp_free(c, idx_d);
+      FD_TRY(k_krr_f32(c));
+      FD_CUDA(cudaStreamSynchronize(c.stream));   // host tables go out of scope
     }
     const int split = o.tc_split == 3 ? 3 : 1;
     const long long ncols = c.N * c.m;
@@ -936,6 +923,8 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   }
 
   // ---------------------------------------------------------------- workspace
+  dfree(c, c.snap, sizeof(double) * (size_t)c.N * c.nsnap);   // every later use of K_s is the sparse form
+  c.snap = nullptr;
   const size_t m = c.m;
   const size_t ncell_max = (size_t)c.N * std::max(c.n, c.nr);
   FD_TRY(dalloc_t(c, &c.w_cell_a, m * ncell_max));

@@ -219,6 +219,14 @@ fetidp_status dalloc(Ctx& c, void** p, size_t bytes) {
   return FETIDP_OK;
 }
 
+void dfree(Ctx& c, void* p, size_t bytes) {
+  const auto it = std::find(c.allocations.begin(), c.allocations.end(), p);
+  if (!p || it == c.allocations.end()) return;
+  c.allocations.erase(it);
+  c.device_bytes -= bytes;
+  cudaFreeAsync(p, c.stream);
+}
+
 namespace {
 
 fetidp_status copy_cells(Ctx& c, CCellVec x, CellVec y, int len, int nrhs, double scale = 1.0) {
@@ -315,16 +323,16 @@ fetidp_status op_apply_MD_rom(Ctx& c, const double* r, long long r_rs, double* z
   CellVec ua{c.w_cell_a, c.N * n, n}, kb{c.w_cell_b, c.N * n, n};
   FD_CUDA(cudaMemsetAsync(c.w_cell_a, 0, sizeof(double) * (size_t)m * c.N * n, c.stream));
   FD_TRY(copy_cells(c, cview(g), CellVec{c.w_cell_a + ni, c.N * n, n}, nd, m));
-  FD_TRY(k_apply_K(c, cview(ua), kb, 1, m, true, false, c.snap, 0.0));
+  FD_TRY(k_apply_K(c, cview(ua), kb, 1, m, n));
   // x_i ~ K_ii^{-1} K_id g
   CCellVec vi{c.w_cell_b, c.N * n, n};
   CellVec R{c.w_R, c.N * nrb * ni, nrb * ni}, KR{c.w_KR, c.N * nrb * ni, nrb * ni}, xi{c.w_i, c.N * ni, ni};
   FD_TRY(k_grouped_gemm(c, c.Kii_inv, (long long)ni * ni, ni, ni, ni, vi, R, nullptr, 1.0, 0.0, m, true, ni));
-  FD_TRY(k_apply_K(c, cview(R), KR, nrb, m, true, false, c.snap, 0.0, ni));
+  FD_TRY(k_apply_K(c, cview(R), KR, nrb, m, ni));
   FD_TRY(k_gram_solve(c, c.w_R, c.w_KR, vi, xi, m, ni));
   // y_d = K_dd g - K_di x_i = [K_s (-x_i; g; 0)]_d
   FD_TRY(copy_cells(c, cview(xi), ua, ni, m, -1.0));
-  FD_TRY(k_apply_K(c, cview(ua), kb, 1, m, true, false, c.snap, 0.0));
+  FD_TRY(k_apply_K(c, cview(ua), kb, 1, m, n));
   FD_TRY(k_scatter_B(c, CCellVec{c.w_cell_b + ni, c.N * n, n}, z, z_rs, c.dinfo, 1.0, 0.0, m));
   return FETIDP_OK;
 }
@@ -376,7 +384,7 @@ fetidp_status local_rom(Ctx& c, CCellVec vR, CellVec xR) {
     const long long rext = (long long)m * rs;       // floats held by each buffer
     FD_TRY(tc_apply(c, c.opKinv, vR, nullptr, Rf, false, rs, nrb * nr, nr, 1.0, 0.0, m, c.N, rext));
     FD_TRY(fd_check_tc("local ROM basis (tensor cores)"));
-    FD_TRY(k_apply_K_f32(c, Rf, rs, nrb * nr, KRf, rs, nrb * nr, nrb, m, true, true, rext));
+    FD_TRY(k_krr_apply_f32(c, Rf, rs, nrb * nr, KRf, rs, nrb * nr, nrb, m, rext));
     FD_TRY(fd_check_cell("local ROM K_s products"));
     FD_TRY(k_gram_solve_f32(c, Rf, KRf, vR, xR, m, rext));
     FD_TRY(fd_check_cell("local ROM Gram solve"));
@@ -386,7 +394,7 @@ fetidp_status local_rom(Ctx& c, CCellVec vR, CellVec xR) {
   FD_TRY(k_grouped_gemm(c, c.Kinv, (long long)nr * nr, nr, nr, nr, vR, R, nullptr, 1.0, 0.0, m, true,
                         nr));
   CellVec KR{c.w_KR, c.N * nrb * nr, nrb * nr};
-  FD_TRY(k_apply_K(c, cview(R), KR, nrb, m, true, true, c.snap, 0.0));
+  FD_TRY(k_apply_K(c, cview(R), KR, nrb, m, nr));
   FD_TRY(k_gram_solve(c, c.w_R, c.w_KR, vR, xR, m));
   return FETIDP_OK;
 }
@@ -581,15 +589,14 @@ fetidp_status pcg_solve(Ctx& c, const double* b, long long b_rs, double* x, long
 
 // ------------------------------------------------------------------ Eq. 16 operator
 fetidp_status op_apply_A(Ctx& c, const double* x, double* y) {
-  const int m = c.m, n = c.n, nr = c.nr, ni = c.ni;
+  const int m = c.m, np = c.np, nr = c.nr, ni = c.ni;
   const long long nt = c.ntot, NR = c.N * nr;
-  CellVec ua{c.w_cell_a, c.N * n, n}, ub{c.w_cell_b, c.N * n, n};
-  FD_TRY(copy_cells(c, CCellVec{x, nt, nr}, ua, nr, m));
-  FD_TRY(k_primal_extract(c, x + NR, nt, CellVec{c.w_cell_a + nr, c.N * n, n}, m));
-  FD_TRY(k_apply_K(c, cview(ua), ub, 1, m, true, false, c.snap, 0.0));
-  FD_TRY(copy_cells(c, cview(ub), CellVec{y, nt, nr}, nr, m));
+  // corner values of u per cell in, corner forces per cell out; the remaining DOF straight from x to y
+  CellVec up{c.w_p1, c.N * np, np}, yp{c.w_cell_b, c.N * np, np};
+  FD_TRY(k_primal_extract(c, x + NR, nt, up, m));
+  FD_TRY(k_apply_K_split(c, CCellVec{x, nt, nr}, cview(up), CellVec{y, nt, nr}, yp, m));
   FD_TRY(k_gather_BT(c, x + NR + c.nP, nt, nullptr, CellVec{y + ni, nt, nr}, m, 1.0));
-  FD_TRY(k_primal_assemble(c, CCellVec{c.w_cell_b + nr, c.N * n, n}, y + NR, nt, 1.0, 0.0, m));
+  FD_TRY(k_primal_assemble(c, cview(yp), y + NR, nt, 1.0, 0.0, m));
   FD_TRY(k_scatter_B(c, CCellVec{x + ni, nt, nr}, y + NR + c.nP, nt, nullptr, 1.0, 0.0, m));
   return FETIDP_OK;
 }
@@ -1159,8 +1166,7 @@ fetidp_status fetidp_apply_K(fetidp_ctx* ctx, const double* u, double* y) {
   FD_TRY(enter(ctx));
   Ctx& c = ctx->c;
   FD_TRY(check_inputs(c, {{u, (long long)c.m * c.N * c.n, "u"}}, y));
-  return k_apply_K(c, CCellVec{u, c.N * c.n, c.n}, CellVec{y, c.N * c.n, c.n}, 1, c.m, false, false,
-                   c.snap, 0.0);
+  return k_apply_K_natural(c, CCellVec{u, c.N * c.n, c.n}, CellVec{y, c.N * c.n, c.n}, c.m);
 }
 
 fetidp_status fetidp_coarse_solve(fetidp_ctx* ctx, const double* b, double* x) {

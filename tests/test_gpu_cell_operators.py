@@ -96,3 +96,22 @@ def test_identical_cells_converge_in_one_outer_iteration_fp64(cells):
     s = binding.Solver(p)
     u, lam, info = s.solve()
     assert info["n_rb"] == 1 and info["outer_its"] <= 2 and info["rel_residual"] < 1e-8
+
+
+@pytest.mark.parametrize("kind", ["2d_e3", "2d_e9", "3d_e4"])
+@pytest.mark.parametrize("n_rhs", [1, 4, 8, 9, 11])
+def test_cell_stiffness_and_saddle_operator_for_every_vector_group(kind, n_rhs):
+    """1-8 vectors per thread group; 9 and 11 make uneven groups.  Natural order (apply_K) and the split
+    remaining / corner views (apply_A) against the oracle's assembled K_s: only the order of sums differs."""
+    from paper_2308_11371_gb300 import binding
+    ref = _oracle(kind)
+    s = binding.Solver(_problem(kind, n_rhs))
+    rng = np.random.default_rng(n_rhs)
+    u = rng.standard_normal((s.n_rhs, s.N, s.n_dof))
+    y = s.apply_K(_dev(u)).cpu().numpy()
+    for c in range(s.N):
+        assert _rel(y[:, c], u[:, c] @ ref.lat.stiffness(c).T) < 1e-12
+    x = rng.standard_normal((s.n_rhs, s.n_tot))
+    z = s.apply_A(_dev(x)).cpu().numpy()
+    for r in range(n_rhs):
+        assert _rel(z[r], ref.A(x[r])) < 1e-12
