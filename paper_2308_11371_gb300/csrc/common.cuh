@@ -283,11 +283,12 @@ struct Ctx {
   // [N][n_i][n_d] and [N][n_d][n_i]; larger lattices combine the principal operators at every use
   double* Uid_c = nullptr;
   double* Udi_c = nullptr;
-  // mixed path, large cells: the same operators assembled in FP32, rows padded to ld_f (16 bytes)
-  float* Fdd_f = nullptr;     // [N][nd][ld_f]
-  float* Sdd_f = nullptr;     // [N][nd][ld_f]
+  // mixed path, large cells: the same operators assembled in FP32 as blocks of at most 128 outputs
+  // (gemm_block_width), each block its n_d stored rows in sequence; ld_f entries per row over all blocks
+  float* Fdd_f = nullptr;     // [N][blocks][nd][block width]
+  float* Sdd_f = nullptr;
   // mixed path, large cells: U_id_ring = the (i, d) block of the delta-combined K_rr^{-1} (Algorithm
-  // 3), in FP32 in both orientations, [N][n_i][ld_id] and [N][n_d][ld_di]
+  // 3), in FP32 in both orientations, n_i x ld_id and n_d x ld_di entries per cell in the same blocks
   float* Uid_f = nullptr;
   float* Udi_f = nullptr;
   int ld_id = 0, ld_di = 0;
@@ -337,6 +338,11 @@ struct Ctx {
   size_t tc_xf_bytes = 0;
   float* tc_yp = nullptr;       // resident-operator combination: partial sums per principal group
   size_t tc_yp_bytes = 0;
+  // RHS-interleaved FP32 cell vectors of the FP32 cell operators: [chunk of 8][N][len][P] with P the RHS
+  // count rounded up to 1, 2, 4 or 8 (xf_P), a cell's part padded to 16 bytes (xf_cs)
+  float* xf = nullptr;
+  int xf_P = 1;
+  int xf_cs(int len) const { return (len * xf_P + 3) & ~3; }
   int* tc_err = nullptr;        // device error flag of the bounded waits
   unsigned long long wait_ns = 1000000000ull;   // budget of every device-side wait
   int* chk = nullptr;           // device flag of the input checks
@@ -386,6 +392,8 @@ fetidp_status dalloc_t(Ctx& c, T** p, size_t count) {
 // ---------------------------------------------------------------- kernels (maps, vectors)
 fetidp_status k_gather_BT(Ctx& c, const double* lam, long long lam_rs, const int* dinfo,
                           CellVec out_d, int nrhs, double beta);
+fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, float* xf, int nrhs);
+fetidp_status k_pack_f32(Ctx& c, CCellVec x, int len, float* xf, int nrhs);
 fetidp_status k_nonfinite(Ctx& c, const double* x, long long n, int* flag);
 fetidp_status wait_selfcheck(unsigned long long wait_ns, cudaStream_t stream);
 fetidp_status k_scatter_B(Ctx& c, CCellVec yd, double* out, long long out_rs, const int* dinfo,
@@ -462,9 +470,21 @@ fetidp_status k_apply_K_natural(Ctx& c, CCellVec u, CellVec y, int nrhs);
 fetidp_status k_apply_K_split(Ctx& c, CCellVec ur, CCellVec up, CellVec yr, CellVec yp, int nrhs);
 fetidp_status k_krr_f32(Ctx& c);
 fetidp_status k_rom_combine_f32(Ctx& c, const double* src, long long kstride, int ld, int r0, int c0, int rows,
-                                int cols, const double* coef, float* out, int ldo, int symT = 0);
+                                int cols, const double* coef, float* out, int ldo, int blkw = 0, int symT = 0);
+// Output blocks of an FP32 cell operator: one warp streams one block, a lane owning 4, 2 or 1 outputs --
+// the widest that gives two warps per SM (figures at cell_gemm_f32_kernel) -- and equal blocks, a
+// multiple of 4 outputs wide.
+inline int gemm_lane_outputs(int nout, long long ncell) {
+  int v = 4;
+  while (v > 1 && ncell * ((nout + 32 * v - 1) / (32 * v)) < 2 * 152) v >>= 1;
+  return v;
+}
+inline int gemm_block_width(int nout, long long ncell) {
+  const int full = 32 * gemm_lane_outputs(nout, ncell), nb = (nout + full - 1) / full;
+  return ((nout + nb - 1) / nb + 3) & ~3;
+}
 fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
-fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, CCellVec x, CellVec y,
+fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
                               double alpha, double beta, int nrhs);
 fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride, int ld, int mrows,
                                   int mcols, CCellVec x, CellVec y, double alpha, double beta,
@@ -513,7 +533,8 @@ fetidp_status tc_comb_apply(Ctx& c, const TcComb& op, CCellVec X, const double* 
 fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, const fetidp_options& o);
 fetidp_status coarse_setup(Ctx& c, const double* Spp_dev);   // per-cell S_pp_ring on the device
 fetidp_status coarse_solve_f32(Ctx& c, const double* b, long long b_rs, double* x, long long x_rs, int nrhs);
-fetidp_status k_udp_f32(Ctx& c, bool trans, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
+fetidp_status k_udp_t_f32(Ctx& c, const float* xf, CCellVec x, CellVec y, int nrhs);
+fetidp_status k_udp_n_f32(Ctx& c, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
 fetidp_status coarse_solve(Ctx& c, const double* b, long long b_rs, double* x, long long x_rs,
                            int nrhs);
 

@@ -6,6 +6,7 @@
 // * gram_solve: Eq. 46b with diagonal-pivoted Cholesky.
 // * grad: adjoint compliance gradient -w^T dK_s/dr_s u.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -309,7 +310,8 @@ __global__ void cell_gemv_narrow_kernel(const double* __restrict__ mats, long lo
 // bytes per cell, shared by the cell's m columns.  At n_d = 630 the streamed operator is the
 // cheaper of the two on GB300, and it is HBM-bound.
 
-// out[cell][r][c] (row stride ldo, FP32) = sum_k coef[cell][k] src[k][(r0 + r) * ld + c0 + c].
+// out[cell][r][c] (FP32; ldo entries per row, in blocks of blkw columns whose rows follow each other, or
+// plain rows when blkw = 0) = sum_k coef[cell][k] src[k][(r0 + r) * ld + c0 + c].
 // A thread owns one entry (r, c): its NRBM principal values sit in registers and are reused for
 // kCombCells cells, whose coefficients are staged in shared memory (FP32 arithmetic).
 constexpr int kCombCells = 32;
@@ -326,7 +328,7 @@ __global__ void __launch_bounds__(256) rom_combine_f32_kernel(const double* __re
                                                               int ld, int r0, int c0, int rows, int cols,
                                                               const double* __restrict__ coef, int nrb,
                                                               long long ncell, float* __restrict__ out, int ldo,
-                                                              int symT) {
+                                                              int blkw, int symT) {
   __shared__ float cs[kCombCells][NRBM];
   const long long per = (long long)rows * cols;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -335,7 +337,9 @@ __global__ void __launch_bounds__(256) rom_combine_f32_kernel(const double* __re
   const int r = r_, cc = c_;
   const long long cell_stride = symT ? 1024LL * symT * (symT + 1) / 2 : (long long)rows * ldo;
   const long long eoff = symT ? 1024LL * sym_tile_index(r >> 5, cc >> 5, symT) + sym_in_tile(r & 31, cc & 31)
-                              : (long long)r * ldo + cc;
+                         : blkw ? (long long)(cc / blkw) * blkw * rows +
+                                      (long long)r * min(blkw, ldo - cc / blkw * blkw) + cc % blkw
+                                : (long long)r * ldo + cc;
   float p[NRBM];
 #pragma unroll
   for (int k = 0; k < NRBM; ++k)
@@ -358,71 +362,116 @@ __global__ void __launch_bounds__(256) rom_combine_f32_kernel(const double* __re
   }
 }
 
-// y[rhs][cell][0..nout) = alpha M[cell]^T x[rhs][cell][0..nin) + beta y for per-cell FP32 matrices
-// M[cell] of nin stored rows of nout entries (row stride ldm, a multiple of 4, >= nout): row j of M
-// multiplies x_j.  For the symmetric F_dd_ring and S_dd_ring (combinations of symmetric principal
-// operators) this is M x.  One CTA per cell; a thread owns four consecutive outputs, so for each
-// stored row j it issues one 16-byte streaming load of M[j][4t..4t+3] (a warp reads 512 contiguous
-// bytes), and the row's x values for every RHS arrive as two broadcast 16-byte reads from shared
-// memory ([row][8] layout).  kAsmU rows' loads are issued before their arithmetic.
+// y[rhs][cell][0..nout) = alpha M[cell]^T x[rhs][cell][0..nin) + beta y for per-cell FP32 matrices M[cell] of
+// nin stored rows: row j of M multiplies x_j (M x for the symmetric F_dd_ring and S_dd_ring).  Bound: HBM --
+// every entry is read once and feeds MR FMAs.  The operator is stored in blocks of at most 128 outputs,
+// each block's rows in sequence, so one warp (a CTA of its own) streams one block of one cell contiguously;
+// a lane owns V outputs and copies its own 4 V bytes of every row into its own slots of a shared-memory
+// ring, kRing rows ahead of the FMAs, without any synchronisation beyond its own cp.async groups.  24 KB in
+// flight per warp (the 16-byte register loads it replaces kept 4 KB, and waited for each batch) need few
+// warps per SM, and the unit of work, a block, is a fifth of a 6^3 cell: lattices of a few hundred cells
+// fill the SMs evenly.  Copy groups of 16 rows: a wait costs a warp about as much as the FMAs of 4 rows (32
+// cells, 6 RHS: 48.6, 33.5, 28 us with groups of 4, 8, 16).  With fewer than two warps per SM the lanes own
+// 2 or 1 outputs instead of 4 (24 cells: 17 us against 24; 32 cells: 22 against 28).
+// x comes interleaved by RHS in FP32 ([j][P], gathered or packed that way), read as 16-byte broadcasts.
+// Every output is one chain of FMAs over ascending j, as before.
+// Measured, n_d = 630, before and now: 2,048 cells, 6 RHS 657 -> 502 us (6.7 TB/s of operator and vectors);
+// 864 cells, 1 RHS 249 -> 210 us; 256 cells, 6 RHS 110 -> 78 us; 50 cells, 3 RHS 100 -> 22 us.
 constexpr int kMaxRhsF32 = 8;
-constexpr int kAsmU = 8;
-constexpr int kAsmMaxThreads = 256;    // rows <= 1024
-__global__ void __launch_bounds__(kAsmMaxThreads) cell_gemm_f32_kernel(const float* __restrict__ mats, int ldm,
-                                                                       int nout, int nin,
-                                                                       const double* __restrict__ x, long long x_rs,
-                                                                       int x_cs, double* __restrict__ y,
-                                                                       long long y_rs, int y_cs, double alpha,
-                                                                       double beta, int nrhs) {
-  extern __shared__ __align__(16) float xsf[];   // [nin][kMaxRhsF32]
-  const long long cell = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int rows = nout, cols = nin;             // outputs, stored rows
-  const float* M = mats + cell * (long long)nin * ldm;
-  const int r0 = 4 * tid;                        // ldm is a multiple of 4 and >= nout: the load stays in row j
-  const bool live = r0 < rows;
-  for (int rb0 = 0; rb0 < nrhs; rb0 += kMaxRhsF32) {
-    const int rb = min(kMaxRhsF32, nrhs - rb0);
-    __syncthreads();
-    for (int t = tid; t < cols * kMaxRhsF32; t += blockDim.x) {
-      const int j = t / kMaxRhsF32, q = t - j * kMaxRhsF32;
-      xsf[t] = q < rb ? (float)x[(rb0 + q) * x_rs + cell * x_cs + j] : 0.f;
+constexpr int kRing = 48, kRingG = 16;            // rows in flight, rows per copy group
+template <int MR, int P, int V>
+__global__ void __launch_bounds__(32) cell_gemm_f32_kernel(const float* __restrict__ mats, int ldm, int nout, int nin,
+                                                           int W, int nb, const float* __restrict__ xf, int xcs,
+                                                           double* __restrict__ y, long long y_rs, int y_cs,
+                                                           double alpha, double beta, int nrhs) {
+  extern __shared__ __align__(16) float gsm[];    // x [nin][P], padded to 16 bytes; then the ring
+  constexpr int NG = kRing / kRingG;
+  const int lane = threadIdx.x;
+  const long long cell = blockIdx.x / nb;
+  const int b = (int)(blockIdx.x - cell * nb);
+  const int xn = (nin * P + 3) >> 2;              // 16-byte pieces of x
+  const int w = min(W, ldm - b * W);              // the block's row stride
+  const bool live = V * lane < w;
+  // lanes past the block's width copy and compute its first outputs again (nothing is stored for them)
+  const float* M = mats + cell * (long long)nin * ldm + (long long)b * W * nin + (live ? V * lane : 0);
+  float* ring = gsm + 4 * xn + lane * V;
+  auto copy = [](float* dst, const float* src, auto bytes) {
+    constexpr int B = decltype(bytes)::value;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"(B) : "memory");
+  };
+  for (int t = lane; t < xn; t += 32)
+    copy(gsm + 4 * t, xf + cell * xcs + 4 * t, std::integral_constant<int, 16>());
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  auto issue = [&](int j0) {                      // rows j0 .. j0 + kRingG - 1 into their slots
+    const float* src = M + (long long)j0 * w;
+    float* dst = ring + (j0 % kRing) * 32 * V;
+    if (j0 + kRingG <= nin) {
+#pragma unroll
+      for (int u = 0; u < kRingG; ++u) copy(dst + u * 32 * V, src + (long long)u * w, std::integral_constant<int, 4 * V>());
+    } else {
+      for (int u = 0; j0 + u < nin; ++u) copy(dst + u * 32 * V, src + (long long)u * w, std::integral_constant<int, 4 * V>());
     }
-    __syncthreads();
-    float acc[4][kMaxRhsF32];
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+  for (int g = 0; g < NG; ++g) issue(g * kRingG);
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(NG) : "memory");
+  __syncwarp();                                   // every lane's part of x is in place
+  float acc[V][MR];
 #pragma unroll
-      for (int q = 0; q < kMaxRhsF32; ++q) acc[a][q] = 0.f;
-    for (int j0 = 0; j0 < cols; j0 += kAsmU) {
-      float4 m[kAsmU];
+  for (int a = 0; a < V; ++a)
 #pragma unroll
-      for (int u = 0; u < kAsmU; ++u)
-        m[u] = (live && j0 + u < cols) ? __ldcs(reinterpret_cast<const float4*>(M + (long long)(j0 + u) * ldm + r0))
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < MR; ++q) acc[a][q] = 0.f;
+  auto row = [&](const float* m, const float* x) {
+    float mv[V], xv[P];
+    if constexpr (V == 4) {
+      const float4 t = *reinterpret_cast<const float4*>(m);
+      mv[0] = t.x; mv[1] = t.y; mv[2] = t.z; mv[3] = t.w;
+    } else if constexpr (V == 2) {
+      const float2 t = *reinterpret_cast<const float2*>(m);
+      mv[0] = t.x; mv[1] = t.y;
+    } else {
+      mv[0] = *m;
+    }
+    if constexpr (P >= 4) {
 #pragma unroll
-      for (int u = 0; u < kAsmU; ++u) {
-        if (j0 + u >= cols) break;
-        const float4 x0 = reinterpret_cast<const float4*>(xsf)[(j0 + u) * 2];
-        const float4 x1 = reinterpret_cast<const float4*>(xsf)[(j0 + u) * 2 + 1];
-        const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-        const float mv[4] = {m[u].x, m[u].y, m[u].z, m[u].w};
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int q = 0; q < kMaxRhsF32; ++q) acc[a][q] = fmaf(mv[a], xv[q], acc[a][q]);
+      for (int q = 0; q < P; q += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(x + q);
+        xv[q] = t.x; xv[q + 1] = t.y; xv[q + 2] = t.z; xv[q + 3] = t.w;
       }
+    } else {
+#pragma unroll
+      for (int q = 0; q < P; ++q) xv[q] = x[q];
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      if (r0 + a >= rows) continue;
+    for (int a = 0; a < V; ++a)
 #pragma unroll
-      for (int q = 0; q < kMaxRhsF32; ++q) {
-        if (q < rb) {
-          double* dst = y + (rb0 + q) * y_rs + cell * y_cs + r0 + a;
-          *dst = (beta == 0.0) ? alpha * (double)acc[a][q] : alpha * (double)acc[a][q] + beta * (*dst);
-        }
-      }
+      for (int q = 0; q < MR; ++q) acc[a][q] = fmaf(mv[a], xv[q], acc[a][q]);
+  };
+  for (int j0 = 0; j0 < nin; j0 += kRingG) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(NG - 1) : "memory");
+    const float* m = ring + (j0 % kRing) * 32 * V;
+    const float* x = gsm + j0 * P;
+    if (j0 + kRingG <= nin) {
+#pragma unroll
+      for (int u = 0; u < kRingG; ++u) row(m + u * 32 * V, x + u * P);
+    } else {
+      for (int u = 0; j0 + u < nin; ++u) row(m + u * 32 * V, x + u * P);
+    }
+    issue(j0 + kRing);                            // the slots just read
+  }
+  if (!live) return;
+  const int r0 = b * W + V * lane;
+#pragma unroll
+  for (int a = 0; a < V; ++a) {
+    if (r0 + a >= nout) continue;
+#pragma unroll
+    for (int q = 0; q < MR; ++q) {
+      if (q >= nrhs) break;
+      double* dst = y + q * y_rs + cell * y_cs + r0 + a;
+      *dst = (beta == 0.0) ? alpha * (double)acc[a][q] : alpha * (double)acc[a][q] + beta * (*dst);
     }
   }
 }
@@ -575,6 +624,7 @@ __global__ void __launch_bounds__(320, 2) cell_symv_f32_kernel(const float* __re
 // shared memory; in udp_n a thread owns a row.
 template <int NP>
 __global__ void __launch_bounds__(256, 3) udp_t_f32_kernel(const float* __restrict__ U, int nd,
+                                                        const float* __restrict__ xf, int P, int xcs, long long ncell,
                                                         const double* __restrict__ g, long long g_rs, int g_cs,
                                                         double* __restrict__ cp, long long c_rs, int c_cs,
                                                         int nrhs) {
@@ -590,9 +640,17 @@ __global__ void __launch_bounds__(256, 3) udp_t_f32_kernel(const float* __restri
   for (int rb0 = 0; rb0 < nrhs; rb0 += 8) {
     const int rb = min(8, nrhs - rb0);
     __syncthreads();
-    for (int t = tid; t < nd * 8; t += blockDim.x) {
-      const int q = t / nd, d = t - q * nd;
-      gs[d * 8 + q] = q < rb ? (float)g[(rb0 + q) * g_rs + cell * g_cs + d] : 0.f;
+    if (xf) {                                     // already FP32 and interleaved
+      const float* xc = xf + ((rb0 >> 3) * ncell + cell) * xcs;
+      for (int t = tid; t < nd * 8; t += blockDim.x) {
+        const int d = t >> 3, q = t & 7;
+        gs[t] = q < rb ? xc[d * P + q] : 0.f;
+      }
+    } else {
+      for (int t = tid; t < nd * 8; t += blockDim.x) {
+        const int q = t / nd, d = t - q * nd;
+        gs[d * 8 + q] = q < rb ? (float)g[(rb0 + q) * g_rs + cell * g_cs + d] : 0.f;
+      }
     }
     __syncthreads();
     float acc[4][8];
@@ -1448,7 +1506,7 @@ fetidp_status k_krr_apply_f32(Ctx& c, const float* u, long long u_rs, int u_cs, 
 }
 
 fetidp_status k_rom_combine_f32(Ctx& c, const double* src, long long kstride, int ld, int r0, int c0, int rows,
-                                int cols, const double* coef, float* out, int ldo, int symT) {
+                                int cols, const double* coef, float* out, int ldo, int blkw, int symT) {
   if (c.nrb > 64) { set_error("n_rb above 64"); return FETIDP_EINVAL; }
   const long long per = (long long)rows * cols;
   long long gy = (c.N + kCombCells - 1) / kCombCells;
@@ -1457,33 +1515,59 @@ fetidp_status k_rom_combine_f32(Ctx& c, const double* src, long long kstride, in
   ProfScope ps(c, FETIDP_K_SETUP, 2.0 * c.nrb * per * (double)c.N, 4.0 * per * (double)c.N);
   if (c.nrb <= 16)
     rom_combine_f32_kernel<16><<<grid, 256, 0, c.stream>>>(src, kstride, ld, r0, c0, rows, cols, coef, c.nrb, c.N, out, ldo,
-                                                             symT);
+                                                             blkw, symT);
   else if (c.nrb <= 32)
     rom_combine_f32_kernel<32><<<grid, 256, 0, c.stream>>>(src, kstride, ld, r0, c0, rows, cols, coef, c.nrb, c.N, out, ldo,
-                                                             symT);
+                                                             blkw, symT);
   else
     rom_combine_f32_kernel<64><<<grid, 256, 0, c.stream>>>(src, kstride, ld, r0, c0, rows, cols, coef, c.nrb, c.N, out, ldo,
-                                                             symT);
+                                                             blkw, symT);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
 
-fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, CCellVec x, CellVec y,
+template <int MR, int P, int V>
+static fetidp_status gemm_f32_launch(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
+                                     double alpha, double beta, int nrhs) {
+  const int W = gemm_block_width(nout, c.N), nb = ceil_div(nout, W);
+  const size_t smem = 16 * ((size_t)(nin * P + 3) / 4) + 4 * (size_t)kRing * 32 * V;
+  cudaFuncSetAttribute(cell_gemm_f32_kernel<MR, P, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cell_gemm_f32_kernel<MR, P, V><<<(unsigned)(c.N * nb), 32, smem, c.stream>>>(
+      mats, ldm, nout, nin, W, nb, xf, c.xf_cs(nin), y.p, y.rs, y.cs, alpha, beta, nrhs);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
                               double alpha, double beta, int nrhs) {
-  // algorithmic bytes: the operators once (padded rows as stored), the FP64 vectors in and out
+  // algorithmic bytes: the operators once (padded rows as stored), the vectors in (FP32) and out (FP64)
   ProfScope ps(c, FETIDP_K_ASM_OP, 2.0 * nout * nin * (double)c.N * nrhs,
-               4.0 * c.N * (double)nin * ldm + 8.0 * c.N * (double)nrhs * (nout + nin));
-  if (nout < 1 || nin < 1 || nout > 4 * kAsmMaxThreads || ldm % 4 != 0 || ldm < nout ||
+               4.0 * c.N * (double)nin * ldm + c.N * (double)nrhs * (8.0 * nout + 4.0 * nin));
+  if (nout < 1 || nin < 1 || nout > 1024 || ldm % 4 != 0 || ldm < nout ||
       (size_t)nin * kMaxRhsF32 * sizeof(float) > 200 * 1024 || (reinterpret_cast<uintptr_t>(mats) & 15) != 0) {
     set_error("FP32 cell operators: at most 1024 outputs, rows padded to 16 bytes");
     return FETIDP_EINVAL;
   }
-  const size_t smem = (size_t)nin * kMaxRhsF32 * sizeof(float);
-  const int threads = ((nout + 3) / 4 + 31) / 32 * 32;
-  cudaFuncSetAttribute(cell_gemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cell_gemm_f32_kernel<<<(unsigned)c.N, threads, smem, c.stream>>>(mats, ldm, nout, nin, x.p, x.rs, x.cs, y.p,
-                                                                   y.rs, y.cs, alpha, beta, nrhs);
-  FD_CHECK_LAUNCH();
+  for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsF32) {
+    const float* x = xf + (r0 / kMaxRhsF32) * (long long)c.N * c.xf_cs(nin);
+    const CellVec yr{y.p + r0 * y.rs, y.rs, y.cs};
+    const int mr = std::min(kMaxRhsF32, nrhs - r0);
+    fetidp_status st = FETIDP_EINVAL;
+    // P: the interleave of the context's RHS count; MR: RHS computed (>= those of this chunk)
+    const int V = gemm_lane_outputs(nout, c.N);
+#define FD_GEMM(MR, P)                                                                              \
+  st = V == 4   ? gemm_f32_launch<MR, P, 4>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr) \
+       : V == 2 ? gemm_f32_launch<MR, P, 2>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr) \
+                : gemm_f32_launch<MR, P, 1>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr)
+    if (c.xf_P == 1) FD_GEMM(1, 1);
+    else if (c.xf_P == 2) FD_GEMM(2, 2);
+    else if (c.xf_P == 4) { if (mr == 3) FD_GEMM(3, 4); else FD_GEMM(4, 4); }
+    else if (mr <= 5) FD_GEMM(5, 8);
+    else if (mr == 6) FD_GEMM(6, 8);
+    else FD_GEMM(8, 8);
+#undef FD_GEMM
+    FD_TRY(st);
+  }
   return FETIDP_OK;
 }
 
@@ -1507,31 +1591,40 @@ fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, 
   return FETIDP_OK;
 }
 
-fetidp_status k_udp_f32(Ctx& c, bool trans, CCellVec x, CellVec y, double alpha, double beta, int nrhs) {
+// x: the FP32 layout (xf) where the gather wrote it, else FP64 cell vectors
+fetidp_status k_udp_t_f32(Ctx& c, const float* xf, CCellVec x, CellVec y, int nrhs) {
+  const int nd = c.nd, np = c.np;
+  if (!c.Udp_f || (np != 8 && np != 24) || nd < 1) { set_error("FP32 U_dp needs n_p of 8 or 24"); return FETIDP_EINVAL; }
+  ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nd * np * (double)c.N * nrhs,
+               4.0 * c.N * nd * np + 8.0 * c.N * nrhs * np + (xf ? 4.0 : 8.0) * c.N * nrhs * nd);
+  const int G = np / 4, RG = 256 / G;
+  const size_t smem = sizeof(float) * ((size_t)nd * 8 + (size_t)RG * G * 32);
+  if (smem > 227 * 1024) { set_error("FP32 U_dp: n_d too large"); return FETIDP_EINVAL; }
+  if (np == 8) {
+    cudaFuncSetAttribute(udp_t_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    udp_t_f32_kernel<8><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, xf, c.xf_P, c.xf_cs(nd), c.N, x.p, x.rs,
+                                                                x.cs, y.p, y.rs, y.cs, nrhs);
+  } else {
+    cudaFuncSetAttribute(udp_t_f32_kernel<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    udp_t_f32_kernel<24><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, xf, c.xf_P, c.xf_cs(nd), c.N, x.p, x.rs,
+                                                                 x.cs, y.p, y.rs, y.cs, nrhs);
+  }
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_udp_n_f32(Ctx& c, CCellVec x, CellVec y, double alpha, double beta, int nrhs) {
   const int nd = c.nd, np = c.np;
   if (!c.Udp_f || (np != 8 && np != 24) || nd < 1) { set_error("FP32 U_dp needs n_p of 8 or 24"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nd * np * (double)c.N * nrhs,
                4.0 * c.N * nd * np + 8.0 * c.N * nrhs * (nd + np + (beta != 0.0 ? nd : 0)));
-  if (trans) {
-    const int G = np / 4, RG = 256 / G;
-    const size_t smem = sizeof(float) * ((size_t)nd * 8 + (size_t)RG * G * 32);
-    if (smem > 227 * 1024) { set_error("FP32 U_dp: n_d too large"); return FETIDP_EINVAL; }
-    if (np == 8) {
-      cudaFuncSetAttribute(udp_t_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      udp_t_f32_kernel<8><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs, nrhs);
-    } else {
-      cudaFuncSetAttribute(udp_t_f32_kernel<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      udp_t_f32_kernel<24><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs, nrhs);
-    }
-  } else {
-    const int threads = std::min(1024, (nd + 31) / 32 * 32);
-    if (np == 8)
-      udp_n_f32_kernel<8><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
-                                                                   alpha, beta, nrhs);
-    else
-      udp_n_f32_kernel<24><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
-                                                                    alpha, beta, nrhs);
-  }
+  const int threads = std::min(1024, (nd + 31) / 32 * 32);
+  if (np == 8)
+    udp_n_f32_kernel<8><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
+                                                                 alpha, beta, nrhs);
+  else
+    udp_n_f32_kernel<24><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
+                                                                  alpha, beta, nrhs);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

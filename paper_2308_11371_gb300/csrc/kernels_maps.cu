@@ -44,10 +44,13 @@ __device__ __forceinline__ double flip_sign(double x, int neg) {
 // at most three rows by the D block -- are decoded once, then applied to every RHS.  Entries whose
 // terms all have weight +-1 (every entry of the unscaled map) take one FP64 addition per RHS, the
 // signs applied to the bits.
+// XF: the values go to the RHS-interleaved FP32 layout of the FP32 cell operators (outf, P entries per
+// dual DOF, xcs per cell) in groups of min(P, 4), rounded once, instead of to FP64 cell vectors.
+template <bool XF>
 __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __restrict__ lam,
                                  long long lam_rs, const int* __restrict__ dinfo, int d,
                                  double* __restrict__ out, long long out_rs, int out_cs, int nd,
-                                 long long ncell, int nrhs, double beta) {
+                                 long long ncell, int nrhs, double beta, float* __restrict__ outf, int P, int xcs) {
   const int total = (int)(ncell * nd);               // < 2^31, checked by the host
   const bool overwrite = beta == 0.0;
   for (int cj = blockIdx.x * blockDim.x + threadIdx.x; cj < total; cj += gridDim.x * blockDim.x) {
@@ -88,7 +91,7 @@ __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __r
         }
       }
     }
-    for (int rhs = 0; rhs < nrhs; ++rhs) {
+    auto value = [&](int rhs) {
       const double* l = lam + rhs * lam_rs;
       double v;
       if (unit) {
@@ -100,8 +103,45 @@ __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __r
         for (int k = 0; k < 6; ++k)
           if ((live >> k) & 1) v = fma(w[k], l[idx[k]], v);
       }
+      return v;
+    };
+    if (XF) {
+      for (int r0 = 0; r0 < nrhs; r0 += 4) {
+        float* o = outf + (r0 >> 3) * ncell * xcs + (long long)cell * xcs + j * P + (r0 & 7);
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? (float)value(r0 + q) : 0.f;
+        if (P >= 4) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+        else if (P == 2) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+        else *o = v[0];
+      }
+      continue;
+    }
+    for (int rhs = 0; rhs < nrhs; ++rhs) {
+      const double v = value(rhs);
       double* o = out + rhs * out_rs + (long long)cell * out_cs + j;
       *o = overwrite ? v : v + beta * (*o);
+    }
+  }
+}
+
+// FP64 cell vectors rounded into the RHS-interleaved FP32 layout (len entries per cell).
+__global__ void pack_f32_kernel(const double* __restrict__ x, long long x_rs, int x_cs, int len, long long ncell,
+                                int nrhs, float* __restrict__ xf, int P, int xcs) {
+  const long long per = ncell * len;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < per;
+       t += (long long)gridDim.x * blockDim.x) {
+    const long long cell = t / len;
+    const int j = (int)(t - cell * len);
+    const double* xc = x + cell * x_cs + j;
+    for (int r0 = 0; r0 < nrhs; r0 += 4) {
+      float* o = xf + (r0 >> 3) * ncell * xcs + cell * xcs + j * P + (r0 & 7);
+      float v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? (float)xc[(r0 + q) * x_rs] : 0.f;
+      if (P >= 4) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+      else if (P == 2) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+      else *o = v[0];
     }
   }
 }
@@ -325,8 +365,26 @@ fetidp_status k_gather_BT(Ctx& c, const double* lam, long long lam_rs, const int
   const long long work = c.N * c.nd;
   if (work >= (1LL << 31) || c.L >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 8.0) + c.N * c.nd * 8.0);
-  gather_BT_kernel<<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, out.p, out.rs,
-                                                          out.cs, c.nd, c.N, nrhs, beta);
+  gather_BT_kernel<false><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, out.p, out.rs,
+                                                                out.cs, c.nd, c.N, nrhs, beta, nullptr, 1, 0);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+// B_d^T lambda (or B_d^T D lambda) rounded into the FP32 cell operators' input layout.
+fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, float* xf, int nrhs) {
+  const long long work = c.N * c.nd;
+  if (work >= (1LL << 31) || c.L >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
+  ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 4.0) + c.N * c.nd * 8.0);
+  gather_BT_kernel<true><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, nullptr, 0, 0, c.nd,
+                                                               c.N, nrhs, 0.0, xf, c.xf_P, c.xf_cs(c.nd));
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_pack_f32(Ctx& c, CCellVec x, int len, float* xf, int nrhs) {
+  ProfScope ps(c, FETIDP_K_MAPS, 0.0, 12.0 * nrhs * c.N * len);
+  pack_f32_kernel<<<grid_for(c.N * len), 256, 0, c.stream>>>(x.p, x.rs, x.cs, len, c.N, nrhs, xf, c.xf_P, c.xf_cs(len));
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

@@ -816,6 +816,8 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
     // HBM-bound), principal form on the tensor cores otherwise
     c.asm_f32 = o.mixed_assembled > 0 || (o.mixed_assembled < 0 && nd > 128);
     if (c.asm_f32) {
+      c.xf_P = c.m >= 5 ? 8 : c.m >= 3 ? 4 : c.m;
+      FD_TRY(dalloc_t(c, &c.xf, (size_t)((c.m + 7) / 8) * c.N * c.xf_cs(std::max(nd, ni))));
       // dense rows padded to 16 bytes (streamed at the HBM rate), or with mixed_assembled = 2 the
       // packed upper-triangle 32 x 32 tiles of these symmetric operators (about half the bytes, up to
       // 20 tile rows; on GB300 that kernel is bound by its shared-memory traffic and is not faster)
@@ -824,12 +826,13 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
       c.ld_f = c.sym_T ? 0 : (nd + 3) & ~3;
       const size_t fbytes = c.sym_T ? sizeof(float) * (size_t)c.N * 1024 * T * (T + 1) / 2
                                     : sizeof(float) * (size_t)c.N * nd * c.ld_f;
+      const int bw = c.sym_T ? 0 : gemm_block_width(nd, c.N);
       FD_TRY(dalloc(c, reinterpret_cast<void**>(&c.Fdd_f), fbytes));
       FD_TRY(dalloc(c, reinterpret_cast<void**>(&c.Sdd_f), fbytes));
       FD_CUDA(cudaMemsetAsync(c.Fdd_f, 0, fbytes, c.stream));   // padding stays zero
       FD_CUDA(cudaMemsetAsync(c.Sdd_f, 0, fbytes, c.stream));
-      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nd, c.delta, c.Fdd_f, c.ld_f, c.sym_T));
-      FD_TRY(k_rom_combine_f32(c, c.Sdd, (long long)nd * nd, nd, 0, 0, nd, nd, c.alpha, c.Sdd_f, c.ld_f, c.sym_T));
+      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nd, c.delta, c.Fdd_f, c.ld_f, bw, c.sym_T));
+      FD_TRY(k_rom_combine_f32(c, c.Sdd, (long long)nd * nd, nd, 0, 0, nd, nd, c.alpha, c.Sdd_f, c.ld_f, bw, c.sym_T));
       // Algorithm 3's U_rd_ring = [U_id_ring; F_dd_ring]: the (i, d) block in FP32, stored once per
       // orientation so that both of its products stream rows (K_rr^{-1} is symmetric, so the (d, i)
       // block is its transpose)
@@ -839,8 +842,10 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
       FD_TRY(dalloc_t(c, &c.Udi_f, (size_t)c.N * nd * c.ld_di));
       FD_CUDA(cudaMemsetAsync(c.Uid_f, 0, sizeof(float) * (size_t)c.N * ni * c.ld_id, c.stream));
       FD_CUDA(cudaMemsetAsync(c.Udi_f, 0, sizeof(float) * (size_t)c.N * nd * c.ld_di, c.stream));
-      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, 0, ni, ni, nd, c.delta, c.Uid_f, c.ld_id));
-      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, ni, 0, nd, ni, c.delta, c.Udi_f, c.ld_di));
+      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, 0, ni, ni, nd, c.delta, c.Uid_f, c.ld_id,
+                               gemm_block_width(nd, c.N)));
+      FD_TRY(k_rom_combine_f32(c, c.Kinv, (long long)nr * nr, nr, ni, 0, nd, ni, c.delta, c.Udi_f, c.ld_di,
+                               gemm_block_width(ni, c.N)));
     }
     FD_TRY(tc_comb_pack(c, c.cFdd, c.Kinv, (long long)nr * nr, nr, ni, ni, nd, nullptr, 0, 0, 0, 0, 0, nd, nrb,
                         split));

@@ -262,11 +262,15 @@ fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, in
 fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y, long long y_rs) {
   const int m = c.m, nd = c.nd, np = c.np, nr = c.nr, ni = c.ni;
   CellVec g{c.w_d1, c.N * nd, nd}, yd{c.w_d2, c.N * nd, nd}, cp{c.w_p1, c.N * np, np};
-  FD_TRY(k_gather_BT(c, lam, lam_rs, nullptr, g, m, 0.0));
-  if (c.asm_f32 && c.sym_T)
-    FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, 1.0, 0.0, m));
+  const bool xf = c.asm_f32 && !c.sym_T;   // the FP32 operators read the interleaved FP32 gather
+  if (xf)
+    FD_TRY(k_gather_BT_f32(c, lam, lam_rs, nullptr, c.xf, m));
+  else
+    FD_TRY(k_gather_BT(c, lam, lam_rs, nullptr, g, m, 0.0));
+  if (xf)
+    FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
   else if (c.asm_f32)
-    FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, cview(g), yd, 1.0, 0.0, m));
+    FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, 1.0, 0.0, m));
   else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cFdd, cview(g), c.delta, c.delta, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
   else
@@ -275,7 +279,7 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
   // applies it with FP32 copies of U_dp_ring and of the S_PP factor (a fixed perturbation of the
   // operator of the inner iterations, well inside their 1e-6 tolerance; the outer FGMRES is FP64).
   if (c.Udp_f)
-    FD_TRY(k_udp_f32(c, true, cview(g), cp, 1.0, 0.0, m));
+    FD_TRY(k_udp_t_f32(c, xf ? c.xf : nullptr, cview(g), cp, m));
   else
     FD_TRY(cell_opt(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, np, nd, cview(g), cp, 1.0, 0.0));
   FD_TRY(k_primal_assemble(c, cview(cp), c.w_P1, c.nP, 1.0, 0.0, m));
@@ -285,7 +289,7 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
     FD_TRY(coarse_solve(c, c.w_P1, c.nP, c.w_P2, c.nP, m));
   FD_TRY(k_primal_extract(c, c.w_P2, c.nP, cp, m));
   if (c.Udp_f)
-    FD_TRY(k_udp_f32(c, false, cview(cp), yd, 1.0, 1.0, m));
+    FD_TRY(k_udp_n_f32(c, cview(cp), yd, 1.0, 1.0, m));
   else
     FD_TRY(cell_op(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, nd, np, cview(cp), yd, 1.0, 1.0));
   FD_TRY(k_scatter_B(c, cview(yd), y, y_rs, nullptr, 1.0, 0.0, m));
@@ -296,11 +300,15 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
 fetidp_status op_apply_MD(Ctx& c, const double* r, long long r_rs, double* z, long long z_rs) {
   const int m = c.m, nd = c.nd;
   CellVec g{c.w_d1, c.N * nd, nd}, yd{c.w_d2, c.N * nd, nd};
-  FD_TRY(k_gather_BT(c, r, r_rs, c.dinfo, g, m, 0.0));
-  if (c.asm_f32 && c.sym_T)
-    FD_TRY(k_cell_symv_f32(c, c.Sdd_f, cview(g), yd, 1.0, 0.0, m));
+  const bool xf = c.asm_f32 && !c.sym_T;
+  if (xf)
+    FD_TRY(k_gather_BT_f32(c, r, r_rs, c.dinfo, c.xf, m));
+  else
+    FD_TRY(k_gather_BT(c, r, r_rs, c.dinfo, g, m, 0.0));
+  if (xf)
+    FD_TRY(k_cell_gemm_f32(c, c.Sdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
   else if (c.asm_f32)
-    FD_TRY(k_cell_gemm_f32(c, c.Sdd_f, c.ld_f, nd, nd, cview(g), yd, 1.0, 0.0, m));
+    FD_TRY(k_cell_symv_f32(c, c.Sdd_f, cview(g), yd, 1.0, 0.0, m));
   else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cSdd, cview(g), c.alpha, c.alpha, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
   else
@@ -352,12 +360,15 @@ fetidp_status U_apply(Ctx& c, CCellVec vR, const double* vP, long long vP_rs, do
   if (c.exact)   // standard FETI-DP: columns d of each cell's own K_rr^{-1} (symmetric)
     FD_TRY(cell_opt(c, c.Kinv + ni, (long long)nr * nr, nr, nd, nr, vR, td, 1.0, 0.0));
   else if (c.Uid_f) {   // assembled FP32 blocks: U_id^T v_i + F_dd v_d
-    FD_TRY(k_cell_gemm_f32(c, c.Uid_f, c.ld_id, nd, ni, vR, td, 1.0, 0.0, m));
+    FD_TRY(k_pack_f32(c, vR, ni, c.xf, m));
+    FD_TRY(k_cell_gemm_f32(c, c.Uid_f, c.ld_id, nd, ni, c.xf, td, 1.0, 0.0, m));
     const CCellVec vd{vR.p + ni, vR.rs, vR.cs};
     if (c.sym_T)
       FD_TRY(k_cell_symv_f32(c, c.Fdd_f, vd, td, 1.0, 1.0, m));
-    else
-      FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, vd, td, 1.0, 1.0, m));
+    else {
+      FD_TRY(k_pack_f32(c, vd, nd, c.xf, m));
+      FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, td, 1.0, 1.0, m));
+    }
   } else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cUrdT, vR, c.delta, c.delta, td.p, true, td.rs, td.cs, 1.0, 0.0, m, c.N));
   else if (c.Uid_c) {   // assembled blocks: U_id^T v_i + F_dd v_d
@@ -635,12 +646,13 @@ fetidp_status op_precondition(Ctx& c, const double* x, double* y) {
   if (c.exact)   // rows d of each cell's own K_rr^{-1}, applied transposed (symmetric)
     FD_TRY(cell_opt(c, c.Kinv + (size_t)ni * nr, (long long)nr * nr, nr, nr, nd, cview(g), yR, -1.0, 1.0));
   else if (c.Uid_f) {   // assembled FP32 blocks: y_i -= U_id g, y_d -= F_dd g
-    FD_TRY(k_cell_gemm_f32(c, c.Udi_f, c.ld_di, ni, nd, cview(g), yR, -1.0, 1.0, m));
+    FD_TRY(k_pack_f32(c, cview(g), nd, c.xf, m));
+    FD_TRY(k_cell_gemm_f32(c, c.Udi_f, c.ld_di, ni, nd, c.xf, yR, -1.0, 1.0, m));
     const CellVec yd{yR.p + ni, yR.rs, yR.cs};
     if (c.sym_T)
       FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, -1.0, 1.0, m));
     else
-      FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, cview(g), yd, -1.0, 1.0, m));
+      FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yd, -1.0, 1.0, m));
   } else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cUrd, cview(g), c.delta, c.delta, yR.p, true, yR.rs, yR.cs, -1.0, 1.0, m, c.N));
   else if (c.Uid_c) {   // assembled blocks: y_i -= U_id g, y_d -= F_dd g

@@ -115,3 +115,35 @@ def test_cell_stiffness_and_saddle_operator_for_every_vector_group(kind, n_rhs):
     z = s.apply_A(_dev(x)).cpu().numpy()
     for r in range(n_rhs):
         assert _rel(z[r], ref.A(x[r])) < 1e-12
+
+
+@pytest.mark.parametrize("kind,copies", [("3d_e4", 1), ("3d_e4", 3), ("3d_e4", 5)])
+@pytest.mark.parametrize("n_rhs", [1, 2, 3, 4, 5, 6, 7, 8, 11])
+def test_fp32_cell_operators_for_every_rhs_count_and_block_width(kind, copies, n_rhs):
+    """Mixed path on 2 x 2 x 1 lattices batched 1, 3 and 5 times (4 to 20 cells with n_d = 270: lanes of 1,
+    and lanes of 4 with a lattice of 216 cells below), every interleave of the right-hand sides.  The FP32
+    operators carry ~6e-8 per entry and an FP32 sum of 270 terms: 1e-5 relative covers both."""
+    from paper_2308_11371_gb300 import binding
+    ref = _oracle(kind)
+    probs = [_problem(kind, n_rhs) for _ in range(copies)]
+    s = binding.Solver(probs, precision=binding.FETIDP_MIXED_BF16)
+    f = binding.Solver(probs)
+    rng = np.random.default_rng(n_rhs)
+    lam = _dev(rng.standard_normal((s.n_rhs, s.L)))
+    assert _rel(s.apply_F(lam).cpu(), f.apply_F(lam).cpu()) < 1e-5
+    assert _rel(s.precond(lam).cpu(), f.precond(lam).cpu()) < 1e-5
+    if copies == 1:
+        y = s.apply_F(lam).cpu().numpy()
+        assert max(_rel(y[r], ref.apply_F(lam[r].cpu().numpy())) for r in range(n_rhs)) < 1e-5
+
+
+@pytest.mark.parametrize("cells,n_rhs", [((6, 6, 6), 3), ((7, 5, 4), 1), ((5, 3, 5), 6)])
+def test_fp32_cell_operators_on_wider_blocks(cells, n_rhs):
+    """216, 140 and 75 cells of n_d = 270: blocks of 4, 4 and 2 outputs per lane against the FP64 path."""
+    from paper_2308_11371_gb300 import binding
+    p = W.lattice_3d(*cells, e=4, r=0.2, r_spread=0.05, seed=3, n_rb=3, mask_kind=W.MASK_BCC_SIGMOID,
+                     loads=_loads(3, n_rhs))
+    s, f = binding.Solver(p, precision=binding.FETIDP_MIXED_BF16), binding.Solver(p)
+    lam = _dev(np.random.default_rng(2).standard_normal((s.n_rhs, s.L)))
+    assert _rel(s.apply_F(lam).cpu(), f.apply_F(lam).cpu()) < 1e-5
+    assert _rel(s.precond(lam).cpu(), f.precond(lam).cpu()) < 1e-5
