@@ -229,6 +229,10 @@ struct Ctx {
   unsigned pcg_graph_mask = 0;           // profiled kernel classes when the graph was captured
   cudaStream_t ws = nullptr;             // the context's own stream for graph capture and replay
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  // streams of the branches that run beside the main one (SideBranch): 0 the coarse correction of
+  // F_ring (high priority), 1 the local ROM solve; made in setup, so a use inside a capture makes none
+  cudaStream_t side[2] = {nullptr, nullptr};
+  cudaEvent_t ev_fork[2] = {nullptr, nullptr}, ev_join[2] = {nullptr, nullptr};
   // per RHS: min over lattices of ||f_b|| / ||f||; the outer solve targets tol * this so that
   // every lattice meets tol relative to its own load
   std::vector<double> tol_scale;

@@ -956,6 +956,13 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   FD_TRY(dalloc_t(c, &c.red, (size_t)m * (c.kry + 2) * 304));
   FD_TRY(dalloc_t(c, &c.scal, 64 * m + (size_t)m * (c.kry + 2) * 2));
   FD_CUDA(cudaMallocHost(&c.h_scal, sizeof(double) * (64 * m + (size_t)m * (c.kry + 2) * 2)));
+  int prio_low = 0, prio_high = 0;
+  FD_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
+  for (int k = 0; k < 2; ++k) {
+    FD_CUDA(cudaStreamCreateWithPriority(&c.side[k], cudaStreamNonBlocking, k == 0 ? prio_high : prio_low));
+    FD_CUDA(cudaEventCreateWithFlags(&c.ev_fork[k], cudaEventDisableTiming));
+    FD_CUDA(cudaEventCreateWithFlags(&c.ev_join[k], cudaEventDisableTiming));
+  }
   FD_CUDA(cudaStreamSynchronize(c.stream));
   phase("workspace");
   c.t_setup_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

