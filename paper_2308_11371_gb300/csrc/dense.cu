@@ -505,9 +505,15 @@ __global__ void coarse_assemble_kernel(const double* __restrict__ Spp, long long
 // float planes hi = fl(v), lo = fl(v - hi) (48 significant bits), zero-padded to whole tiles.  A
 // term is hi*hi, made exact by an FMA residual, plus the two cross products; the sum is kept as
 // an unevaluated pair (s, c) with TwoSum on the leading part: 12 FP32 instructions per term.
-// Relative error ~K * 2^-46 of the largest term, against K * 2^-53 for FP64.  64 x 64 output
-// tile per block, 4 x 4 per thread, K chunks of 16 staged by cp.async in two buffers.
-constexpr int DF_T = 64, DF_K = 16, DF_LD = 20;   // smem rows of 16 floats + 4 pad (16-byte aligned)
+// Relative error ~K * 2^-46 of the largest term, against K * 2^-53 for FP64.  256 threads of E x E
+// outputs, K chunks of 16 staged by cp.async in two buffers.
+// Bound: FP32 issue, and with few outputs the K = 77,760 steps of one output's chain (K is not split: the
+// Gram solves behind the traces amplify a change of summation order).  E = 2 leaves registers for enough
+// warps to hide the chains (4,096 cells of 16^2 elements, 32 principals: 18.0 ms against 20.2 with E = 4);
+// E = 1 is taken while E = 2 gives less than a block per SM: 46 cells of 6^3 elements and 37 principals
+// 20.1 (E = 4), 5.5 (2), 3.4 ms (1); 256 cells and 32 principals 20.2, 10.1, 12.2; 864 and 15 20.2, 10.1, 9.2.
+constexpr int DF_K = 16, DF_LD = 20;   // smem rows of 16 floats + 4 pad (16-byte aligned)
+constexpr int DF_T = 32;               // rows and columns of the planes are padded to the wider tile
 
 __global__ void df_split_kernel(const double* __restrict__ src, long long rows, int cols, long long src_ld,
                                 long long rows_p, int ld_p, float* __restrict__ hi, float* __restrict__ lo) {
@@ -528,22 +534,24 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 
-__global__ void __launch_bounds__(256, 2) df_gemm_kernel(const float* __restrict__ Ah, const float* __restrict__ Al,
+template <int E>
+__global__ void __launch_bounds__(256, 4) df_gemm_kernel(const float* __restrict__ Ah, const float* __restrict__ Al,
                                                       const float* __restrict__ Xh, const float* __restrict__ Xl,
                                                       int ldk, int nkc, int M, long long ncols,
                                                       double* __restrict__ Y, int y_cs) {
-  __shared__ __align__(16) float sA[2][2][DF_T][DF_LD];   // [buffer][hi, lo][row m][k]
-  __shared__ __align__(16) float sX[2][2][DF_T][DF_LD];   // [buffer][hi, lo][column][k]
+  constexpr int T = 16 * E;
+  __shared__ __align__(16) float sA[2][2][T][DF_LD];   // [buffer][hi, lo][row m][k]
+  __shared__ __align__(16) float sX[2][2][T][DF_LD];   // [buffer][hi, lo][column][k]
   // row tiles fastest: the blocks resident together share their X (snapshot) tiles, which are
   // then read from DRAM about once, while the table planes stay in L2
-  const long long m0 = (long long)blockIdx.x * DF_T;
-  const long long col0 = (long long)blockIdx.y * DF_T;
+  const long long m0 = (long long)blockIdx.x * T;
+  const long long col0 = (long long)blockIdx.y * T;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  // one chunk: 4 planes x 64 rows x 4 quads of 16 bytes = 1024 copies, 4 per thread
+  // one chunk: 4 planes x T rows x 4 quads of 16 bytes, E copies per thread
   auto load = [&](int buf, int kc) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = tid + 256 * u, plane = e >> 8, row = (e >> 2) & 63, quad = e & 3;
+    for (int u = 0; u < E; ++u) {
+      const int e = tid + 256 * u, plane = e / (4 * T), row = (e >> 2) % T, quad = e & 3;
       const long long off = (long long)kc * DF_K + quad * 4;
       switch (plane) {
         case 0: cp_async16(&sA[buf][0][row][quad * 4], Ah + (m0 + row) * ldk + off); break;
@@ -554,11 +562,11 @@ __global__ void __launch_bounds__(256, 2) df_gemm_kernel(const float* __restrict
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  float s[4][4], cl[4][4];
+  float s[E][E], cl[E][E];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < E; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { s[i][j] = 0.f; cl[i][j] = 0.f; }
+    for (int j = 0; j < E; ++j) { s[i][j] = 0.f; cl[i][j] = 0.f; }
   load(0, 0);
   for (int kc = 0; kc < nkc; ++kc) {
     const int buf = kc & 1;
@@ -571,19 +579,19 @@ __global__ void __launch_bounds__(256, 2) df_gemm_kernel(const float* __restrict
     __syncthreads();
 #pragma unroll
     for (int q4 = 0; q4 < DF_K; q4 += 4) {
-      float4 bh[4], bl[4];
+      float4 bh[E], bl[E];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < E; ++j) {
         bh[j] = *reinterpret_cast<const float4*>(&sX[buf][0][tx + 16 * j][q4]);
         bl[j] = *reinterpret_cast<const float4*>(&sX[buf][1][tx + 16 * j][q4]);
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < E; ++i) {
         const float4 ah4 = *reinterpret_cast<const float4*>(&sA[buf][0][ty + 16 * i][q4]);
         const float4 al4 = *reinterpret_cast<const float4*>(&sA[buf][1][ty + 16 * i][q4]);
         const float ah[4] = {ah4.x, ah4.y, ah4.z, ah4.w}, al[4] = {al4.x, al4.y, al4.z, al4.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < E; ++j) {
           const float xh[4] = {bh[j].x, bh[j].y, bh[j].z, bh[j].w}, xl[4] = {bl[j].x, bl[j].y, bl[j].z, bl[j].w};
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
@@ -603,11 +611,11 @@ __global__ void __launch_bounds__(256, 2) df_gemm_kernel(const float* __restrict
     __syncthreads();
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < E; ++j) {
     const long long gc = col0 + tx + 16 * j;
     if (gc >= ncols) continue;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < E; ++i) {
       const long long gm = m0 + ty + 16 * i;
       if (gm < M) Y[gc * y_cs + gm] = (double)s[i][j] + (double)cl[i][j];
     }
@@ -724,8 +732,11 @@ fetidp_status k_df_gemm_planes(Ctx& c, const float* Ah, const float* Al, int M, 
   }
   {
     ProfScope ps(c, FETIDP_K_TRACES, 2.0 * M * (double)K * ncols, 8.0 * ((double)M * K + (double)ncols * (K + M)));
-    const dim3 grid((unsigned)(Mp / DF_T), (unsigned)(Np / DF_T));
-    df_gemm_kernel<<<grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs);
+    const bool wide = (Mp / DF_T) * (Np / DF_T) >= 152;
+    const int t = wide ? 32 : 16;
+    const dim3 grid((unsigned)((M + t - 1) / t), (unsigned)((ncols + t - 1) / t));
+    if (wide) df_gemm_kernel<2><<<grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs);
+    else df_gemm_kernel<1><<<grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs);
     count_launch();
   }
   if (cudaPeekAtLastError() != cudaSuccess) {
