@@ -230,7 +230,7 @@ struct Ctx {
   cudaStream_t ws = nullptr;             // the context's own stream for graph capture and replay
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   // streams of the branches that run beside the main one (SideBranch): 0 the coarse correction of
-  // F_ring (high priority), 1 the local ROM solve; made in setup, so a use inside a capture makes none
+  // F_ring (high priority), 1 the local ROM solve; made first in setup, so a use inside a capture makes none
   cudaStream_t side[2] = {nullptr, nullptr};
   cudaEvent_t ev_fork[2] = {nullptr, nullptr}, ev_join[2] = {nullptr, nullptr};
   // per RHS: min over lattices of ||f_b|| / ||f||; the outer solve targets tol * this so that
@@ -393,6 +393,39 @@ fetidp_status dalloc_t(Ctx& c, T** p, size_t count) {
   return dalloc(c, reinterpret_cast<void**>(p), count * sizeof(T));
 }
 
+// A branch of an operator on its own stream: work issued between the constructor and leave() starts after
+// what the main stream holds at that point and runs beside what the main stream gets next, until join().
+// Both ends are events, so the branch becomes a parallel path of a graph when the main stream is being
+// captured.  The destructor joins whatever happened in between (an error return too): nothing of a branch
+// outlives the call on the context's buffers.
+struct SideBranch {
+  Ctx& c;
+  const int k;
+  cudaStream_t main;
+  bool inside = false, open = false;
+  SideBranch(Ctx& ctx, int which) : c(ctx), k(which), main(ctx.stream) {}
+  fetidp_status enter() {
+    FD_CUDA(cudaEventRecord(c.ev_fork[k], main));
+    FD_CUDA(cudaStreamWaitEvent(c.side[k], c.ev_fork[k], 0));
+    c.stream = c.side[k];
+    inside = open = true;
+    return FETIDP_OK;
+  }
+  void leave() {
+    if (inside) c.stream = main;
+    inside = false;
+  }
+  fetidp_status join() {
+    leave();
+    if (!open) return FETIDP_OK;
+    open = false;
+    FD_CUDA(cudaEventRecord(c.ev_join[k], c.side[k]));
+    FD_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join[k], 0));
+    return FETIDP_OK;
+  }
+  ~SideBranch() { join(); }
+};
+
 // ---------------------------------------------------------------- kernels (maps, vectors)
 fetidp_status k_gather_BT(Ctx& c, const double* lam, long long lam_rs, const int* dinfo,
                           CellVec out_d, int nrhs, double beta);
@@ -445,7 +478,8 @@ fetidp_status k_greedy_alpha(Ctx& c, const double* Z, const double* nrm, const d
                              const GreedyState* st, double* T, double* alpha);
 // dense batched setup kernels (principal blocks, SPD inverses by sweeps)
 fetidp_status k_assemble_principal(Ctx& c, const int* sigma_dev, int nrb, double* Krr, double* Krp, double* Kpp);
-fetidp_status k_spd_inverse_batched(Ctx& c, double* A, long long stride, int n, int lda, int batch, int* status);
+fetidp_status k_spd_inverse_batched(Ctx& c, double* A, long long stride, int n, int lda, int batch, int* status,
+                                    int ns = 0, double* schur = nullptr);
 fetidp_status k_batched_gemm_nn(Ctx& c, const double* A, long long sa, int lda, const double* B, long long sb,
                                 int ldb, double* C, long long sc, int ldc, int M, int N, int K, int batch);
 fetidp_status k_batched_block_copy(Ctx& c, const double* in, long long si, int ldi, int r0, int c0, double* out,

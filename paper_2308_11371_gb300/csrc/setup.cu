@@ -260,6 +260,13 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
     set_error("gram_drop_mixed must lie in [0, 1)");
     return FETIDP_EINVAL;
   }
+  int prio_low = 0, prio_high = 0;
+  FD_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
+  for (int k = 0; k < 2; ++k) {
+    FD_CUDA(cudaStreamCreateWithPriority(&c.side[k], cudaStreamNonBlocking, k == 0 ? prio_high : prio_low));
+    FD_CUDA(cudaEventCreateWithFlags(&c.ev_fork[k], cudaEventDisableTiming));
+    FD_CUDA(cudaEventCreateWithFlags(&c.ev_join[k], cudaEventDisableTiming));
+  }
   const int d = p.dim, e = p.elems;
   c.lat.assign(nprob, LatticeSpan{});
   c.N = 0;
@@ -664,16 +671,14 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
       FD_TRY(k_spd_inverse_batched(c, c.Kii_inv, (long long)ni * ni, ni, ni, nrb, st_dev));
     }
     phase("  principal assembly");
-    FD_TRY(k_spd_inverse_batched(c, c.Kinv, (long long)nr * nr, nr, nr, nrb, st_dev));
+    // K_rr^{-1}, and S_dd = F_dd^{-1} as the Schur complement of the interior DOF on the way
+    FD_TRY(k_spd_inverse_batched(c, c.Kinv, (long long)nr * nr, nr, nr, nrb, st_dev, ni, c.Sdd));
     phase("  principal K_rr inverse");
     FD_TRY(k_batched_gemm_nn(c, c.Kinv, (long long)nr * nr, nr, Krp_d, (long long)nr * np, np, c.Urp,
                              (long long)nr * np, np, nr, np, nr, nrb));
     FD_TRY(k_batched_block_copy(c, c.Urp, (long long)nr * np, np, 0, 0, c.UrpT, (long long)np * nr, nr, nr, np,
                                 nrb, true));
     FD_TRY(k_batched_diag_sum(c, c.Kinv, (long long)nr * nr, nr, ni, nd, nrb, dvec_d));
-    FD_TRY(k_batched_block_copy(c, c.Kinv, (long long)nr * nr, nr, ni, ni, c.Sdd, (long long)nd * nd, nd, nd, nd,
-                                nrb, false));
-    FD_TRY(k_spd_inverse_batched(c, c.Sdd, (long long)nd * nd, nd, nd, nrb, st_dev));
     int hst = 0;
     FD_CUDA(cudaMemcpyAsync(dvec.data(), dvec_d, sizeof(double) * nrb, cudaMemcpyDeviceToHost, c.stream));
     FD_CUDA(cudaMemcpyAsync(&hst, st_dev, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
@@ -956,13 +961,6 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   FD_TRY(dalloc_t(c, &c.red, (size_t)m * (c.kry + 2) * 304));
   FD_TRY(dalloc_t(c, &c.scal, 64 * m + (size_t)m * (c.kry + 2) * 2));
   FD_CUDA(cudaMallocHost(&c.h_scal, sizeof(double) * (64 * m + (size_t)m * (c.kry + 2) * 2)));
-  int prio_low = 0, prio_high = 0;
-  FD_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
-  for (int k = 0; k < 2; ++k) {
-    FD_CUDA(cudaStreamCreateWithPriority(&c.side[k], cudaStreamNonBlocking, k == 0 ? prio_high : prio_low));
-    FD_CUDA(cudaEventCreateWithFlags(&c.ev_fork[k], cudaEventDisableTiming));
-    FD_CUDA(cudaEventCreateWithFlags(&c.ev_join[k], cudaEventDisableTiming));
-  }
   FD_CUDA(cudaStreamSynchronize(c.stream));
   phase("workspace");
   c.t_setup_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

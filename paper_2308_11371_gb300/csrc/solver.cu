@@ -256,39 +256,6 @@ fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, in
   return k_cell_gemvt(c, mats, mstride, ld, nout, nin, x, y, alpha, beta, c.m);
 }
 
-// A branch of an operator on its own stream: work issued between the constructor and leave() starts after
-// what the main stream holds at that point and runs beside what the main stream gets next, until join().
-// Both ends are events, so the branch becomes a parallel path of a graph when the main stream is being
-// captured.  The destructor joins whatever happened in between (an error return too): nothing of a branch
-// outlives the call on the context's buffers.
-struct SideBranch {
-  Ctx& c;
-  const int k;
-  cudaStream_t main;
-  bool inside = false, open = false;
-  SideBranch(Ctx& ctx, int which) : c(ctx), k(which), main(ctx.stream) {}
-  fetidp_status enter() {
-    FD_CUDA(cudaEventRecord(c.ev_fork[k], main));
-    FD_CUDA(cudaStreamWaitEvent(c.side[k], c.ev_fork[k], 0));
-    c.stream = c.side[k];
-    inside = open = true;
-    return FETIDP_OK;
-  }
-  void leave() {
-    if (inside) c.stream = main;
-    inside = false;
-  }
-  fetidp_status join() {
-    leave();
-    if (!open) return FETIDP_OK;
-    open = false;
-    FD_CUDA(cudaEventRecord(c.ev_join[k], c.side[k]));
-    FD_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join[k], 0));
-    return FETIDP_OK;
-  }
-  ~SideBranch() { join(); }
-};
-
 }  // namespace
 
 // ------------------------------------------------------------------ Eq. 48
