@@ -325,7 +325,7 @@ struct Ctx {
   double* Z = nullptr;          // [max_outer][m][ntot]
   double* pcg = nullptr;        // [6][m][L]: x, r, z, p, q, right-hand side
   double* red = nullptr;        // reduction scratch (partials + scalars)
-  unsigned int* red_count = nullptr;
+  unsigned int* red_count = nullptr;   // arrivals per reduced vector, zero between launches
   double* scal = nullptr;       // device scalars [64][m]
   double* h_scal = nullptr;     // pinned host mirror
   int inner_total = 0;
@@ -440,6 +440,11 @@ fetidp_status k_primal_assemble(Ctx& c, CCellVec cp, double* out, long long out_
 fetidp_status k_primal_extract(Ctx& c, const double* uP, long long uP_rs, CellVec cp, int nrhs);
 fetidp_status k_dot(Ctx& c, const double* x, long long xs, const double* y, long long ys,
                     long long len, int nrhs, double* out);
+// rows of c.scal (one value per RHS) that a PCG iteration reads and writes
+struct PcgSlots { int rz, pq, rr, act, r0, err, its; };
+fetidp_status k_pcg_update(Ctx& c, double* X, double* R, const double* P, const double* Q, const PcgSlots& S,
+                           double tol);
+fetidp_status k_pcg_p(Ctx& c, double* P, const double* Z, const PcgSlots& S, int rz_new);
 fetidp_status k_multi_dot(Ctx& c, const double* Vb, long long vstride, int nv, const double* w,
                           long long len, int nrhs, double* out);
 fetidp_status k_multi_axpy(Ctx& c, const double* Vb, long long vstride, int nv, const double* coef,

@@ -262,21 +262,47 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;
 }
 
-// partial[(rhs*nv + i)*kRedBlocks + blk] = sum over this block's fixed slice of V_i . w
-__global__ void multi_dot_partial(const double* __restrict__ Vb, long long vstride, long long vrs,
-                                  const double* __restrict__ w, long long wrs, long long len,
-                                  int nv, double* __restrict__ partial) {
+// Sum of one value per block over the blocks blockIdx.x of a launch (deterministic, one launch): every block
+// leaves its value in part[blockIdx.x]; the last one to arrive (a counter that it leaves at zero) adds them
+// in a fixed order and tree.  True in thread 0 of that block, with the total in `total`.
+__device__ __forceinline__ bool grid_sum(double v, double* __restrict__ part, unsigned* __restrict__ count,
+                                         double* sh, double& total) {
+  __shared__ bool last;
+  v = block_sum(v, sh);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(count, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double s = 0.0;
+  for (int t = threadIdx.x; t < (int)gridDim.x; t += blockDim.x) s += __ldcg(part + t);
+  total = block_sum(s, sh);
+  if (threadIdx.x == 0) *count = 0u;
+  return threadIdx.x == 0;
+}
+
+// out[rhs*nv + i] = V_i[rhs] . w[rhs], V_i at Vb + i*vstride + rhs*vrs: blockIdx.x a fixed slice, y the RHS,
+// z the vector.
+__global__ void multi_dot_kernel(const double* __restrict__ Vb, long long vstride, long long vrs,
+                                 const double* __restrict__ w, long long wrs, long long len,
+                                 int nv, double* __restrict__ partial, unsigned* __restrict__ count,
+                                 double* __restrict__ out) {
   __shared__ double sh[32];
   const int i = blockIdx.z, rhs = blockIdx.y, blk = blockIdx.x;
   const double* v = Vb + i * vstride + rhs * vrs;
   const double* x = w + rhs * wrs;
-  const long long chunk = (len + kRedBlocks - 1) / kRedBlocks;
+  const long long chunk = (len + gridDim.x - 1) / gridDim.x;
   const long long beg = blk * chunk;
   const long long end = beg + chunk < len ? beg + chunk : len;
   double s = 0.0;
+#pragma unroll 4
   for (long long t = beg + threadIdx.x; t < end; t += blockDim.x) s += v[t] * x[t];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) partial[((long long)rhs * nv + i) * kRedBlocks + blk] = s;
+  const long long k = (long long)rhs * nv + i;
+  double total;
+  if (grid_sum(s, partial + k * kRedBlocks, count + k, sh, total)) out[k] = total;
 }
 
 __global__ void reduce_partials(const double* __restrict__ partial, int count,
@@ -289,6 +315,55 @@ __global__ void reduce_partials(const double* __restrict__ partial, int count,
   s = block_sum(s, sh);
   if (threadIdx.x == 0) out[k] = s;
   (void)count;
+}
+
+// One PCG update: x += alpha p, r -= alpha q, alpha = rz / pq, and r . r of the new residual; blockIdx.y is the
+// RHS (converged ones leave at once).  With tol >= 0 the last block of an RHS also makes the convergence
+// test: counts the iteration, flags a breakdown (p^T F p <= 0 or a non-finite residual) and clears the
+// active flag when ||r|| / ||r_0|| <= tol or r = 0, so whole iterations run without a host round trip.
+__global__ void pcg_update_kernel(double* __restrict__ X, double* __restrict__ R, const double* __restrict__ P,
+                                  const double* __restrict__ Q, double* __restrict__ scal, PcgSlots S, long long L,
+                                  int nrhs, double tol, double* __restrict__ partial, unsigned* __restrict__ count) {
+  __shared__ double sh[32];
+  const int rhs = blockIdx.y;
+  if (scal[S.act * nrhs + rhs] == 0.0) return;
+  const double pq = scal[S.pq * nrhs + rhs];
+  const double alpha = scal[S.rz * nrhs + rhs] / pq;
+  const long long chunk = (L + gridDim.x - 1) / gridDim.x, beg = blockIdx.x * chunk, o = rhs * L;
+  const long long end = beg + chunk < L ? beg + chunk : L;
+  double s = 0.0;
+#pragma unroll 2
+  for (long long t = beg + threadIdx.x; t < end; t += blockDim.x) {
+    X[o + t] += alpha * P[o + t];
+    const double r = R[o + t] - alpha * Q[o + t];
+    R[o + t] = r;
+    s += r * r;
+  }
+  double rr;
+  if (!grid_sum(s, partial + (long long)rhs * kRedBlocks, count + rhs, sh, rr)) return;
+  scal[S.rr * nrhs + rhs] = rr;
+  if (tol < 0.0) return;
+  scal[S.its * nrhs + rhs] += 1.0;
+  if (!(pq > 0.0) || !isfinite(rr)) {
+    scal[S.err * nrhs + rhs] = 1.0;
+    scal[S.act * nrhs + rhs] = 0.0;
+  } else if (sqrt(rr / scal[S.r0 * nrhs + rhs]) <= tol || rr == 0.0) {
+    scal[S.act * nrhs + rhs] = 0.0;
+  }
+}
+
+// p = z + beta p, beta = rz_new / rz_old, for the active RHS (blockIdx.y)
+__global__ void pcg_p_kernel(double* __restrict__ P, const double* __restrict__ Zv,
+                             const double* __restrict__ scal, int act, int new_slot, int old_slot, long long L,
+                             int nrhs) {
+  const int rhs = blockIdx.y;
+  if (scal[act * nrhs + rhs] == 0.0) return;
+  const double beta = scal[new_slot * nrhs + rhs] / scal[old_slot * nrhs + rhs];
+  double* p = P + rhs * L;
+  const double* z = Zv + rhs * L;
+#pragma unroll 4
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L; t += (long long)gridDim.x * blockDim.x)
+    p[t] = z[t] + beta * p[t];
 }
 
 // Compliance partial sums: sum over (cell, local dof) of f . u for one load case, with f the
@@ -349,6 +424,12 @@ __global__ void nonfinite_kernel(const double* __restrict__ x, long long n, int*
       atomicOr(flag, 1);
       return;
     }
+}
+
+// blocks per reduced vector: at least four entries per thread, at most two blocks per SM
+inline int red_blocks(long long len) {
+  const long long b = (len + 4 * kRedThreads - 1) / (4 * kRedThreads);
+  return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
 }
 
 inline int grid_for(long long work, int threads = 256) {
@@ -421,10 +502,8 @@ static fetidp_status multi_dot_impl(Ctx& c, const double* Vb, long long vstride,
                                     int nv, const double* w, long long wrs, long long len,
                                     int nrhs, double* out) {
   ProfScope ps(c, FETIDP_K_VECTOR, 2.0 * nv * len * nrhs, 8.0 * (nv + 1) * len * nrhs);
-  dim3 grid(kRedBlocks, nrhs, nv);
-  multi_dot_partial<<<grid, kRedThreads, 0, c.stream>>>(Vb, vstride, vrs, w, wrs, len, nv, c.red);
-  FD_CHECK_LAUNCH();
-  reduce_partials<<<nrhs * nv, kRedThreads, 0, c.stream>>>(c.red, nrhs * nv, out);
+  multi_dot_kernel<<<dim3(red_blocks(len), nrhs, nv), kRedThreads, 0, c.stream>>>(Vb, vstride, vrs, w, wrs, len, nv,
+                                                                                  c.red, c.red_count, out);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
@@ -432,6 +511,22 @@ static fetidp_status multi_dot_impl(Ctx& c, const double* Vb, long long vstride,
 fetidp_status k_dot(Ctx& c, const double* x, long long xs, const double* y, long long ys,
                     long long len, int nrhs, double* out) {
   return multi_dot_impl(c, x, 0, xs, 1, y, ys, len, nrhs, out);
+}
+
+fetidp_status k_pcg_update(Ctx& c, double* X, double* R, const double* P, const double* Q, const PcgSlots& S,
+                           double tol) {
+  ProfScope ps(c, FETIDP_K_VECTOR, 6.0 * c.L * c.m, 48.0 * c.L * c.m);
+  pcg_update_kernel<<<dim3(red_blocks(c.L), c.m), kRedThreads, 0, c.stream>>>(X, R, P, Q, c.scal, S, c.L, c.m, tol,
+                                                                             c.red, c.red_count);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_pcg_p(Ctx& c, double* P, const double* Z, const PcgSlots& S, int rz_new) {
+  ProfScope ps(c, FETIDP_K_VECTOR, 2.0 * c.L * c.m, 24.0 * c.L * c.m);
+  pcg_p_kernel<<<dim3(grid_for((c.L + 3) / 4), c.m), 256, 0, c.stream>>>(P, Z, c.scal, S.act, rz_new, S.rz, c.L, c.m);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
 }
 
 fetidp_status k_multi_dot(Ctx& c, const double* Vb, long long vstride, int nv, const double* w,

@@ -68,50 +68,6 @@ __global__ void permute_out_kernel(const int* __restrict__ perm, const double* _
   }
 }
 
-// x += alpha p, r -= alpha q with alpha = rz / pq per active RHS
-__global__ void pcg_xr_kernel(double* __restrict__ X, double* __restrict__ R,
-                              const double* __restrict__ P, const double* __restrict__ Q,
-                              const double* __restrict__ scal, int rz_slot, long long L, int nrhs) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L * nrhs;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int rhs = (int)(t / L);
-    const double act = scal[S_ACT * nrhs + rhs];
-    if (act == 0.0) continue;
-    const double alpha = scal[rz_slot * nrhs + rhs] / scal[S_PQ * nrhs + rhs];
-    X[t] += alpha * P[t];
-    R[t] -= alpha * Q[t];
-  }
-}
-
-// Convergence test of one PCG iteration on the device (one thread per RHS): counts the iteration,
-// flags a breakdown (p^T F p <= 0 or a non-finite residual) and clears the RHS's active flag when
-// ||r|| / ||r_0|| <= tol or r = 0.  Lets whole iterations run without a host round trip.
-__global__ void pcg_check_kernel(double* __restrict__ scal, int nrhs, double tol) {
-  const int r = threadIdx.x;
-  if (r >= nrhs || scal[S_ACT * nrhs + r] == 0.0) return;
-  const double pq = scal[S_PQ * nrhs + r], rr = scal[S_RR * nrhs + r];
-  scal[S_ITS * nrhs + r] += 1.0;
-  if (!(pq > 0.0) || !isfinite(rr)) {
-    scal[S_ERR * nrhs + r] = 1.0;
-    scal[S_ACT * nrhs + r] = 0.0;
-    return;
-  }
-  if (sqrt(rr / scal[S_R0 * nrhs + r]) <= tol || rr == 0.0) scal[S_ACT * nrhs + r] = 0.0;
-}
-
-// p = z + beta p, beta = rz_new / rz_old per active RHS
-__global__ void pcg_p_kernel(double* __restrict__ P, const double* __restrict__ Zv,
-                             const double* __restrict__ scal, int new_slot, int old_slot, long long L,
-                             int nrhs) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L * nrhs;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int rhs = (int)(t / L);
-    if (scal[S_ACT * nrhs + rhs] == 0.0) continue;
-    const double beta = scal[new_slot * nrhs + rhs] / scal[old_slot * nrhs + rhs];
-    P[t] = Zv[t] + beta * P[t];
-  }
-}
-
 inline int gridn(long long work) {
   long long g = (work + 255) / 256;
   if (g > 152LL * 16) g = 152LL * 16;
@@ -427,6 +383,7 @@ fetidp_status pcg_solve(Ctx& c, const double* b, long long b_rs, double* x, long
   double *X = c.pcg, *R = c.pcg + mL, *Zv = c.pcg + 2 * mL, *P = c.pcg + 3 * mL, *Q = c.pcg + 4 * mL;
   double* sc = c.scal;
   double* hs = c.h_scal;
+  auto slots = [](int rz) { return PcgSlots{rz, S_PQ, S_RR, S_ACT, S_R0, S_ERR, S_ITS}; };
   FD_TRY(k_copy_scale(c, b, R, L, m, b_rs, L, nullptr, 1.0));
   FD_CUDA(cudaMemsetAsync(X, 0, sizeof(double) * mL, c.stream));
   FD_TRY(k_dot(c, R, L, R, L, L, m, sc + S_R0 * m));
@@ -502,21 +459,10 @@ fetidp_status pcg_solve(Ctx& c, const double* b, long long b_rs, double* x, long
         const int rz = half == 0 ? S_RZ0 : S_RZ1, rzn = half == 0 ? S_RZ1 : S_RZ0;
         cap = op_apply_F(c, P, L, Q, L);
         if (cap == FETIDP_OK) cap = k_dot(c, P, L, Q, L, L, m, sc + S_PQ * m);
-        if (cap == FETIDP_OK) {
-          pcg_xr_kernel<<<gridn(mL), 256, 0, c.stream>>>(X, R, P, Q, sc, rz, L, m);
-          count_launch();
-          cap = k_dot(c, R, L, R, L, L, m, sc + S_RR * m);
-        }
-        if (cap == FETIDP_OK) {
-          pcg_check_kernel<<<1, 32, 0, c.stream>>>(sc, m, tol);
-          count_launch();
-          cap = op_apply_MD(c, R, L, Zv, L);
-        }
+        if (cap == FETIDP_OK) cap = k_pcg_update(c, X, R, P, Q, slots(rz), tol);
+        if (cap == FETIDP_OK) cap = op_apply_MD(c, R, L, Zv, L);
         if (cap == FETIDP_OK) cap = k_dot(c, R, L, Zv, L, L, m, sc + rzn * m);
-        if (cap == FETIDP_OK) {
-          pcg_p_kernel<<<gridn(mL), 256, 0, c.stream>>>(P, Zv, sc, rzn, rz, L, m);
-          count_launch();
-        }
+        if (cap == FETIDP_OK) cap = k_pcg_p(c, P, Zv, slots(rz), rzn);
       }
       cudaGraph_t graph = nullptr;
       const cudaError_t ce = cudaStreamEndCapture(c.stream, &graph);
@@ -572,9 +518,7 @@ fetidp_status pcg_solve(Ctx& c, const double* b, long long b_rs, double* x, long
   while (nact > 0 && it < max_it) {
     FD_TRY(op_apply_F(c, P, L, Q, L));
     FD_TRY(k_dot(c, P, L, Q, L, L, m, sc + S_PQ * m));
-    pcg_xr_kernel<<<gridn(mL), 256, 0, c.stream>>>(X, R, P, Q, sc, cur, L, m);
-    FD_CHECK_LAUNCH();
-    FD_TRY(k_dot(c, R, L, R, L, L, m, sc + S_RR * m));
+    FD_TRY(k_pcg_update(c, X, R, P, Q, slots(cur), -1.0));   // the host makes the test
     FD_CUDA(cudaMemcpyAsync(hs, sc, sizeof(double) * S_NSLOT * m, cudaMemcpyDeviceToHost, c.stream));
     FD_CUDA(cudaStreamSynchronize(c.stream));
     ++it;
@@ -597,8 +541,7 @@ fetidp_status pcg_solve(Ctx& c, const double* b, long long b_rs, double* x, long
     FD_TRY(op_apply_MD(c, R, L, Zv, L));
     const int nxt = cur == S_RZ0 ? S_RZ1 : S_RZ0;
     FD_TRY(k_dot(c, R, L, Zv, L, L, m, sc + nxt * m));
-    pcg_p_kernel<<<gridn(mL), 256, 0, c.stream>>>(P, Zv, sc, nxt, cur, L, m);
-    FD_CHECK_LAUNCH();
+    FD_TRY(k_pcg_p(c, P, Zv, slots(cur), nxt));
     cur = nxt;
   }
   c.inner_total += it;
