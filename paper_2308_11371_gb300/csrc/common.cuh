@@ -111,6 +111,37 @@ fetidp_status fd_check_tc(const char* where);
   fetidp_status fname(const char*) { return FETIDP_OK; }
 #endif
 
+// ---------------------------------------------------------------- conversions off the FP64 pipe
+// GB300's FP64 pipe takes two lanes per clock and SM, conversions between FP32 and FP64 included: a kernel
+// that rounds or widens one value per few bytes is bound by it, not by memory.  These give the bits of the
+// hardware conversions from integer instructions; values outside the normal range take the hardware path.
+__device__ __forceinline__ double fd_widen(float f) {
+  const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u) return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+  if (a == 0u) return __hiloint2double((int)b, 0);
+  return (double)f;
+}
+__device__ __forceinline__ float fd_round(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u < 254u) {                              // normal in FP32 before rounding
+    const unsigned m = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rest = lo & 0x1fffffffu;           // round to nearest even; a carry may reach infinity
+    return __uint_as_float(m + (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))));
+  }
+  if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(hi);
+  return (float)d;
+}
+// x / 2 (exact for normal results)
+__device__ __forceinline__ double fd_half(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), e = (hi >> 20) & 0x7ffu;
+  if (e - 2u < 0x7fdu) return __hiloint2double((int)(hi - 0x00100000u), __double2loint(x));
+  return 0.5 * x;
+}
+__device__ __forceinline__ bool fd_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
+__device__ __forceinline__ double fd_load(double v) { return v; }
+__device__ __forceinline__ double fd_load(float v) { return fd_widen(v); }
+
 // Per-cell vector view: element (rhs, cell, i) at p[rhs*rs + cell*cs + i].
 struct CellVec {
   double* p;
@@ -300,6 +331,7 @@ struct Ctx {
   int sym_T = 0;
   bool asm_f32 = false;
   bool exact = false;         // standard FETI-DP: every cell's own K_rr^{-1} (nrb = N, no ROM)
+  float* cpf = nullptr;       // [chunk of 8 RHS][N][np][8] mixed path: corner values for U_dp in FP32
   float* Udp_f = nullptr;     // [N][nd][np] mixed path: the dual rows of U_rp_ring in FP32
   double* Urp_c = nullptr;    // [N][nr][np]
   // coarse solve
@@ -347,6 +379,10 @@ struct Ctx {
   float* xf = nullptr;
   int xf_P = 1;
   int xf_cs(int len) const { return (len * xf_P + 3) & ~3; }
+  // dual DOF of a cell with the face nodes' first, and multiplier rows with those whose D block is not a
+  // matrix last: warps of the D-scaled maps then take one of their two paths
+  int* dual_order = nullptr;    // [nd]
+  int* row_order = nullptr;     // [L]
   int* tc_err = nullptr;        // device error flag of the bounded waits
   unsigned long long wait_ns = 1000000000ull;   // budget of every device-side wait
   int* chk = nullptr;           // device flag of the input checks
@@ -429,7 +465,21 @@ struct SideBranch {
 // ---------------------------------------------------------------- kernels (maps, vectors)
 fetidp_status k_gather_BT(Ctx& c, const double* lam, long long lam_rs, const int* dinfo,
                           CellVec out_d, int nrhs, double beta);
-fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, float* xf, int nrhs);
+// Where an FP32 gather puts entry (rhs, cell, j): chunk rhs / 8 at chs, then rs, cs, ds strides; entries
+// nd <= j < width are zero.
+struct XfLayout {
+  float* p;
+  long long chs, rs, cs;
+  int ds, width, P;             // P > 1: the rhs of a chunk are adjacent (ds = P), written in groups
+};
+fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, const XfLayout& xf,
+                              int nrhs);
+struct FCellVec {               // FP32 cell vectors
+  float* p;
+  long long rs;
+  int cs;
+};
+fetidp_status k_scatter_B_f32(Ctx& c, const FCellVec& yd, double* out, long long out_rs, const int* dinfo, int nrhs);
 fetidp_status k_pack_f32(Ctx& c, CCellVec x, int len, float* xf, int nrhs);
 fetidp_status k_nonfinite(Ctx& c, const double* x, long long n, int* flag);
 fetidp_status wait_selfcheck(unsigned long long wait_ns, cudaStream_t stream);
@@ -438,6 +488,8 @@ fetidp_status k_scatter_B(Ctx& c, CCellVec yd, double* out, long long out_rs, co
 fetidp_status k_primal_assemble(Ctx& c, CCellVec cp, double* out, long long out_rs, double alpha,
                                 double beta, int nrhs);
 fetidp_status k_primal_extract(Ctx& c, const double* uP, long long uP_rs, CellVec cp, int nrhs);
+// rounded to FP32, [chunk of 8 RHS][cell][n_p][8]
+fetidp_status k_primal_extract_f32(Ctx& c, const double* uP, long long uP_rs, float* cpf, int nrhs);
 fetidp_status k_dot(Ctx& c, const double* x, long long xs, const double* y, long long ys,
                     long long len, int nrhs, double* out);
 // rows of c.scal (one value per RHS) that a PCG iteration reads and writes
@@ -529,6 +581,8 @@ inline int gemm_block_width(int nout, long long ncell) {
 fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
 fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
                               double alpha, double beta, int nrhs);
+fetidp_status k_cell_gemm_f32_out(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf,
+                                  const FCellVec& y, int nrhs);
 fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride, int ld, int mrows,
                                   int mcols, CCellVec x, CellVec y, double alpha, double beta,
                                   int nrhs);
@@ -566,6 +620,9 @@ fetidp_status tc_comb_pack(Ctx& c, TcComb& op, const double* src0, long long st0
 size_t tc_comb_staging_bytes(const TcComb& op, long long ncols);
 bool tc_comb2_ok(const TcComb& op);
 size_t tc_comb2_xf_bytes(const TcComb& op, long long ncols);
+// the resident-operator combination with x already in c.tc_xf ([col][tc_comb2_width]), FP32 results
+int tc_comb2_width(const TcComb& op);
+fetidp_status tc_comb2_apply_f32(Ctx& c, const TcComb& op, const double* coef, const FCellVec& y, int nrhs);
 size_t tc_comb2_yp_bytes(const TcComb& op, long long ncols);
 fetidp_status tc_comb_selfcheck(Ctx& c, int M0, int M1, int K, int N, int nops, double* rel_err);
 fetidp_status tc_comb_apply(Ctx& c, const TcComb& op, CCellVec X, const double* coef0, const double* coef1,
@@ -576,8 +633,8 @@ fetidp_status tc_comb_apply(Ctx& c, const TcComb& op, CCellVec X, const double* 
 fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, const fetidp_options& o);
 fetidp_status coarse_setup(Ctx& c, const double* Spp_dev);   // per-cell S_pp_ring on the device
 fetidp_status coarse_solve_f32(Ctx& c, const double* b, long long b_rs, double* x, long long x_rs, int nrhs);
-fetidp_status k_udp_t_f32(Ctx& c, const float* xf, CCellVec x, CellVec y, int nrhs);
-fetidp_status k_udp_n_f32(Ctx& c, CCellVec x, CellVec y, double alpha, double beta, int nrhs);
+fetidp_status k_udp_t_f32(Ctx& c, const XfLayout& xf, CellVec y, int nrhs);
+fetidp_status k_udp_n_f32(Ctx& c, const float* cpf, const FCellVec* yf, CellVec y, int nrhs);
 fetidp_status coarse_solve(Ctx& c, const double* b, long long b_rs, double* x, long long x_rs,
                            int nrhs);
 

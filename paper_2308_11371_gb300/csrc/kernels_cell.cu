@@ -379,10 +379,10 @@ __global__ void __launch_bounds__(256) rom_combine_f32_kernel(const double* __re
 // 864 cells, 1 RHS 249 -> 210 us; 256 cells, 6 RHS 110 -> 78 us; 50 cells, 3 RHS 100 -> 22 us.
 constexpr int kMaxRhsF32 = 8;
 constexpr int kRing = 48, kRingG = 16;            // rows in flight, rows per copy group
-template <int MR, int P, int V>
+template <int MR, int P, int V, typename TO>
 __global__ void __launch_bounds__(32) cell_gemm_f32_kernel(const float* __restrict__ mats, int ldm, int nout, int nin,
                                                            int W, int nb, const float* __restrict__ xf, int xcs,
-                                                           double* __restrict__ y, long long y_rs, int y_cs,
+                                                           TO* __restrict__ y, long long y_rs, int y_cs,
                                                            double alpha, double beta, int nrhs) {
   extern __shared__ __align__(16) float gsm[];    // x [nin][P], padded to 16 bytes; then the ring
   constexpr int NG = kRing / kRingG;
@@ -470,8 +470,9 @@ __global__ void __launch_bounds__(32) cell_gemm_f32_kernel(const float* __restri
 #pragma unroll
     for (int q = 0; q < MR; ++q) {
       if (q >= nrhs) break;
-      double* dst = y + q * y_rs + cell * y_cs + r0 + a;
-      *dst = (beta == 0.0) ? alpha * (double)acc[a][q] : alpha * (double)acc[a][q] + beta * (*dst);
+      TO* dst = y + q * y_rs + cell * y_cs + r0 + a;
+      if constexpr (sizeof(TO) == 4) *dst = acc[a][q];   // alpha = 1, beta = 0
+      else *dst = (beta == 0.0) ? alpha * (double)acc[a][q] : alpha * (double)acc[a][q] + beta * (*dst);
     }
   }
 }
@@ -618,124 +619,148 @@ __global__ void __launch_bounds__(320, 2) cell_symv_f32_kernel(const float* __re
 // Coarse restriction and prolongation of the inner iterations (the coarse term of Eq. 48) with the
 // FP32 copy of U_dp_ring (the dual rows of U_rp_ring), [cell][n_d][NP] row-major:
 //   udp_t:  cp[rhs][cell][p] = sum_d U[d][p] g[rhs][cell][d]
-//   udp_n:  y[rhs][cell][d]  = alpha sum_p U[d][p] cp[rhs][cell][p] + beta y
-// One CTA per cell.  In udp_t a thread owns four consecutive p of every RG-th row (one 16-byte
-// load per row), accumulates them for up to eight RHS in FP32 and the RG row groups are summed in
-// shared memory; in udp_n a thread owns a row.
-template <int NP>
-__global__ void __launch_bounds__(256, 3) udp_t_f32_kernel(const float* __restrict__ U, int nd,
-                                                        const float* __restrict__ xf, int P, int xcs, long long ncell,
-                                                        const double* __restrict__ g, long long g_rs, int g_cs,
+//   udp_n:  y[rhs][cell][d]  = y[rhs][cell][d] + sum_p U[d][p] cp[rhs][cell][p]
+// Bound: HBM (U once, the vectors).  The sum over d keeps its order: RG = 256 / (NP / 4) interleaved chains of
+// FMAs, then their sums in sequence.  udp_t runs one CTA per cell, a thread four consecutive p of one chain
+// (its first rows loaded before x is staged), MR sums each, the chains added through shared memory; where
+// every chain has one row (n_d <= RG, 2D cells up to 17^2 elements) it is one thread per (cell, p) and no
+// barrier.  udp_n is one thread per (cell, d) for the RHS of a chunk.
+// 2,048 cells of n_d = 630 and 6 RHS: udp_t 100 -> 32 us, udp_n 100 -> 49; 864 cells, 1 RHS: 37 -> 12 and 41 -> 13;
+// 4,096 cells of n_d = 120, 1 RHS: 58 -> 20 and 23 -> 6.5 us.
+template <int NP, int MR, int P>
+__global__ void __launch_bounds__(256) udp_t_f32_kernel(const float* __restrict__ U, int nd, XfLayout xf,
                                                         double* __restrict__ cp, long long c_rs, int c_cs,
                                                         int nrhs) {
   constexpr int G = NP / 4;          // 16-byte groups per row
   constexpr int RG = 256 / G;        // row groups
-  extern __shared__ __align__(16) float smu[];   // gs[nd][8], red[RG * G][32]
+  constexpr int UB = 8;              // rows loaded ahead of their FMAs, the first batch ahead of the staging
+  extern __shared__ __align__(16) float smu[];   // gs[nd][P] (16-byte padded), red[RG * G][4 MR]
   float* gs = smu;
-  float* red = smu + (size_t)nd * 8;
+  float* red = smu + (((size_t)nd * P + 3) & ~(size_t)3);
   const long long cell = blockIdx.x;
   const int tid = threadIdx.x;
   const int grp = tid % G, rg = tid / G;
-  const float4* Uc = reinterpret_cast<const float4*>(U + cell * (long long)nd * NP);
-  for (int rb0 = 0; rb0 < nrhs; rb0 += 8) {
-    const int rb = min(8, nrhs - rb0);
-    __syncthreads();
-    if (xf) {                                     // already FP32 and interleaved
-      const float* xc = xf + ((rb0 >> 3) * ncell + cell) * xcs;
-      for (int t = tid; t < nd * 8; t += blockDim.x) {
-        const int d = t >> 3, q = t & 7;
-        gs[t] = q < rb ? xc[d * P + q] : 0.f;
-      }
-    } else {
-      for (int t = tid; t < nd * 8; t += blockDim.x) {
-        const int q = t / nd, d = t - q * nd;
-        gs[d * 8 + q] = q < rb ? (float)g[(rb0 + q) * g_rs + cell * g_cs + d] : 0.f;
+  const float4* Uc = reinterpret_cast<const float4*>(U + cell * (long long)nd * NP) + grp;
+  float4 u[UB];
+#pragma unroll
+  for (int k = 0; k < UB; ++k)
+    u[k] = rg < RG && rg + k * RG < nd ? __ldcs(Uc + (long long)(rg + k * RG) * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* xc = xf.p + cell * xf.cs;
+  if (xf.ds == P) {
+#pragma unroll 4
+    for (int t = tid; t < (nd * P + 3) / 4; t += blockDim.x)
+      reinterpret_cast<float4*>(gs)[t] = __ldg(reinterpret_cast<const float4*>(xc) + t);
+  } else {
+    for (int t = tid; t < nd * P; t += blockDim.x) gs[t] = t % P < nrhs ? xc[t / P * xf.ds + t % P * xf.rs] : 0.f;
+  }
+  __syncthreads();
+  float acc[4][MR];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int q = 0; q < MR; ++q) acc[a][q] = 0.f;
+  if (rg < RG) {
+    for (int d0 = rg; d0 < nd; d0 += UB * RG) {
+      if (d0 != rg)
+#pragma unroll
+        for (int k = 0; k < UB; ++k)
+          u[k] = d0 + k * RG < nd ? __ldcs(Uc + (long long)(d0 + k * RG) * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < UB; ++k) {
+        const int d = d0 + k * RG;
+        if (d >= nd) break;
+        const float uv[4] = {u[k].x, u[k].y, u[k].z, u[k].w};
+        const float* x = gs + d * P;
+#pragma unroll
+        for (int q = 0; q < MR; ++q) {
+          const float xq = x[q];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) acc[a][q] = fmaf(uv[a], xq, acc[a][q]);
+        }
       }
     }
-    __syncthreads();
-    float acc[4][8];
+    float* rd = red + (size_t)(rg * G + grp) * 4 * MR;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc[a][q] = 0.f;
-    if (rg < RG) {
-#pragma unroll 4
-      for (int d = rg; d < nd; d += RG) {
-        const float4 u = __ldcs(Uc + (long long)d * G + grp);
-        const float4 x0 = reinterpret_cast<const float4*>(gs)[d * 2];
-        const float4 x1 = reinterpret_cast<const float4*>(gs)[d * 2 + 1];
-        const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-        const float uv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int q = 0; q < 8; ++q) acc[a][q] = fmaf(uv[a], xv[q], acc[a][q]);
-      }
-      float4* rd = reinterpret_cast<float4*>(red + (size_t)(rg * G + grp) * 32);
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        rd[2 * a] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-        rd[2 * a + 1] = make_float4(acc[a][4], acc[a][5], acc[a][6], acc[a][7]);
-      }
-    }
-    __syncthreads();
-    for (int o = tid; o < NP * 8; o += blockDim.x) {
-      const int p = o >> 3, q = o & 7;
-      const int gp = p >> 2, a = p & 3;
-      float sum = 0.f;
-      for (int k = 0; k < RG; ++k) sum += red[(size_t)(k * G + gp) * 32 + a * 8 + q];
-      if (q < rb) cp[(rb0 + q) * c_rs + cell * c_cs + p] = (double)sum;
-    }
+      for (int q = 0; q < MR; ++q) rd[a * MR + q] = acc[a][q];
+  }
+  __syncthreads();
+  for (int o = tid; o < NP * MR; o += blockDim.x) {
+    const int p = o / MR, q = o - p * MR;
+    float sum = 0.f;
+#pragma unroll 14
+    for (int k = 0; k < RG; ++k) sum += red[(size_t)(k * G + (p >> 2)) * 4 * MR + (p & 3) * MR + q];
+    if (q < nrhs) cp[q * c_rs + cell * c_cs + p] = fd_widen(sum);
   }
 }
 
 template <int NP>
-__global__ void __launch_bounds__(1024) udp_n_f32_kernel(const float* __restrict__ U, int nd,
-                                                         const double* __restrict__ cp, long long c_rs, int c_cs,
-                                                         double* __restrict__ y, long long y_rs, int y_cs,
-                                                         double alpha, double beta, int nrhs) {
-  constexpr int G = NP / 4;
-  __shared__ __align__(16) float cs[NP][8];
-  const long long cell = blockIdx.x;
-  const int tid = threadIdx.x;
-  const float4* Uc = reinterpret_cast<const float4*>(U + cell * (long long)nd * NP);
-  for (int rb0 = 0; rb0 < nrhs; rb0 += 8) {
-    const int rb = min(8, nrhs - rb0);
-    __syncthreads();
-    for (int t = tid; t < NP * 8; t += blockDim.x) {
-      const int p = t >> 3, q = t & 7;
-      cs[p][q] = q < rb ? (float)cp[(rb0 + q) * c_rs + cell * c_cs + p] : 0.f;
+__global__ void __launch_bounds__(128) udp_t_short_f32_kernel(const float* __restrict__ U, int nd, XfLayout xf,
+                                                              double* __restrict__ cp, long long c_rs, int c_cs,
+                                                              int nrhs, long long ncell) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long cell = t / NP;
+  const int p = (int)(t - cell * NP);
+  if (cell >= ncell) return;
+  const float* Uc = U + cell * (long long)nd * NP + p;
+  for (int q = 0; q < nrhs; ++q) {
+    const float* x = xf.p + cell * xf.cs + q * xf.rs;
+    float tot = 0.f;
+    int d = 0;
+    for (; d + 8 <= nd; d += 8) {
+      float u[8], v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        u[k] = __ldg(Uc + (d + k) * NP);
+        v[k] = __ldg(x + (d + k) * xf.ds);
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) tot = __fadd_rn(tot, __fmul_rn(u[k], v[k]));   // a chain's sum is its one product
     }
-    __syncthreads();
-    for (int d = tid; d < nd; d += blockDim.x) {
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (; d < nd; ++d) tot = __fadd_rn(tot, __fmul_rn(__ldg(Uc + d * NP), __ldg(x + d * xf.ds)));
+    cp[q * c_rs + cell * c_cs + p] = fd_widen(tot);
+  }
+}
+
+// With cvt, mul and fma on the FP64 pipe the epilogue bound the kernel (111 of 101-120 us at 2,048 cells and 6
+// RHS): the sums are widened by integer instructions and one FP64 addition is left.  cp comes rounded to
+// FP32, [cell][NP][8] (broadcast reads); yin is the FP32 or FP64 vector the product is added to.
+template <int NP, int MR, typename TI>
+__global__ void __launch_bounds__(128) udp_n_f32_kernel(const float* __restrict__ U, int nd,
+                                                        const float* __restrict__ cpf, const TI* yin,
+                                                        long long yi_rs, int yi_cs, double* y, long long y_rs,
+                                                        int y_cs, int nrhs, long long ncell) {
+  constexpr int G = NP / 4;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long cell = t / nd;
+  const int d = (int)(t - cell * nd);
+  if (cell >= ncell) return;
+  const float4* Uc = reinterpret_cast<const float4*>(U + t * NP);
+  float4 u[G];
 #pragma unroll
-      for (int gq = 0; gq < G; ++gq) {
-        const float4 u = __ldcs(Uc + (long long)d * G + gq);
-        const float uv[4] = {u.x, u.y, u.z, u.w};
+  for (int gq = 0; gq < G; ++gq) u[gq] = __ldcs(Uc + gq);
+  TI y0[MR];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const float4 x0 = reinterpret_cast<const float4*>(cs[4 * gq + a])[0];
-          const float4 x1 = reinterpret_cast<const float4*>(cs[4 * gq + a])[1];
-          acc[0] = fmaf(uv[a], x0.x, acc[0]);
-          acc[1] = fmaf(uv[a], x0.y, acc[1]);
-          acc[2] = fmaf(uv[a], x0.z, acc[2]);
-          acc[3] = fmaf(uv[a], x0.w, acc[3]);
-          acc[4] = fmaf(uv[a], x1.x, acc[4]);
-          acc[5] = fmaf(uv[a], x1.y, acc[5]);
-          acc[6] = fmaf(uv[a], x1.z, acc[6]);
-          acc[7] = fmaf(uv[a], x1.w, acc[7]);
-        }
-      }
+  for (int q = 0; q < MR; ++q) y0[q] = yin[min(q, nrhs - 1) * yi_rs + cell * yi_cs + d];
+  const float4* cc = reinterpret_cast<const float4*>(cpf + cell * NP * 8);
+  float acc[MR];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (q < rb) {
-          double* dst = y + (rb0 + q) * y_rs + cell * y_cs + d;
-          *dst = (beta == 0.0) ? alpha * (double)acc[q] : alpha * (double)acc[q] + beta * (*dst);
-        }
-      }
+  for (int q = 0; q < MR; ++q) acc[q] = 0.f;
+#pragma unroll
+  for (int gq = 0; gq < G; ++gq) {
+    const float uv[4] = {u[gq].x, u[gq].y, u[gq].z, u[gq].w};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const float4 x0 = __ldg(cc + 2 * (4 * gq + a)), x1 = MR > 4 ? __ldg(cc + 2 * (4 * gq + a) + 1) : x0;
+      const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+      for (int q = 0; q < MR; ++q) acc[q] = fmaf(uv[a], xv[q], acc[q]);
     }
   }
+#pragma unroll
+  for (int q = 0; q < MR; ++q)
+    if (q < nrhs) y[q * y_rs + cell * y_cs + d] = fd_widen(acc[q]) + fd_load(y0[q]);
 }
 
 // Grouped FP64 GEMM, 64 x TN output tile per block (256 threads, 4 x TN/16 per thread), K chunks of 16.
@@ -1526,23 +1551,24 @@ fetidp_status k_rom_combine_f32(Ctx& c, const double* src, long long kstride, in
   return FETIDP_OK;
 }
 
-template <int MR, int P, int V>
-static fetidp_status gemm_f32_launch(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
-                                     double alpha, double beta, int nrhs) {
+template <int MR, int P, int V, typename TO>
+static fetidp_status gemm_f32_launch(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, TO* y,
+                                     long long y_rs, int y_cs, double alpha, double beta, int nrhs) {
   const int W = gemm_block_width(nout, c.N), nb = ceil_div(nout, W);
   const size_t smem = 16 * ((size_t)(nin * P + 3) / 4) + 4 * (size_t)kRing * 32 * V;
-  cudaFuncSetAttribute(cell_gemm_f32_kernel<MR, P, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cell_gemm_f32_kernel<MR, P, V><<<(unsigned)(c.N * nb), 32, smem, c.stream>>>(
-      mats, ldm, nout, nin, W, nb, xf, c.xf_cs(nin), y.p, y.rs, y.cs, alpha, beta, nrhs);
+  cudaFuncSetAttribute(cell_gemm_f32_kernel<MR, P, V, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cell_gemm_f32_kernel<MR, P, V, TO><<<(unsigned)(c.N * nb), 32, smem, c.stream>>>(
+      mats, ldm, nout, nin, W, nb, xf, c.xf_cs(nin), y, y_rs, y_cs, alpha, beta, nrhs);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
 
-fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
-                              double alpha, double beta, int nrhs) {
-  // algorithmic bytes: the operators once (padded rows as stored), the vectors in (FP32) and out (FP64)
+template <typename TO>
+static fetidp_status cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, TO* y,
+                                   long long y_rs, int y_cs, double alpha, double beta, int nrhs) {
+  // algorithmic bytes: the operators once (padded rows as stored), the vectors in (FP32) and out
   ProfScope ps(c, FETIDP_K_ASM_OP, 2.0 * nout * nin * (double)c.N * nrhs,
-               4.0 * c.N * (double)nin * ldm + c.N * (double)nrhs * (8.0 * nout + 4.0 * nin));
+               4.0 * c.N * (double)nin * ldm + c.N * (double)nrhs * ((double)sizeof(TO) * nout + 4.0 * nin));
   if (nout < 1 || nin < 1 || nout > 1024 || ldm % 4 != 0 || ldm < nout ||
       (size_t)nin * kMaxRhsF32 * sizeof(float) > 200 * 1024 || (reinterpret_cast<uintptr_t>(mats) & 15) != 0) {
     set_error("FP32 cell operators: at most 1024 outputs, rows padded to 16 bytes");
@@ -1550,15 +1576,15 @@ fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int 
   }
   for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsF32) {
     const float* x = xf + (r0 / kMaxRhsF32) * (long long)c.N * c.xf_cs(nin);
-    const CellVec yr{y.p + r0 * y.rs, y.rs, y.cs};
+    TO* yr = y + r0 * y_rs;
     const int mr = std::min(kMaxRhsF32, nrhs - r0);
     fetidp_status st = FETIDP_EINVAL;
     // P: the interleave of the context's RHS count; MR: RHS computed (>= those of this chunk)
     const int V = gemm_lane_outputs(nout, c.N);
 #define FD_GEMM(MR, P)                                                                              \
-  st = V == 4   ? gemm_f32_launch<MR, P, 4>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr) \
-       : V == 2 ? gemm_f32_launch<MR, P, 2>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr) \
-                : gemm_f32_launch<MR, P, 1>(c, mats, ldm, nout, nin, x, yr, alpha, beta, mr)
+  st = V == 4   ? gemm_f32_launch<MR, P, 4>(c, mats, ldm, nout, nin, x, yr, y_rs, y_cs, alpha, beta, mr) \
+       : V == 2 ? gemm_f32_launch<MR, P, 2>(c, mats, ldm, nout, nin, x, yr, y_rs, y_cs, alpha, beta, mr) \
+                : gemm_f32_launch<MR, P, 1>(c, mats, ldm, nout, nin, x, yr, y_rs, y_cs, alpha, beta, mr)
     if (c.xf_P == 1) FD_GEMM(1, 1);
     else if (c.xf_P == 2) FD_GEMM(2, 2);
     else if (c.xf_P == 4) { if (mr == 3) FD_GEMM(3, 4); else FD_GEMM(4, 4); }
@@ -1569,6 +1595,17 @@ fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int 
     FD_TRY(st);
   }
   return FETIDP_OK;
+}
+
+fetidp_status k_cell_gemm_f32(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf, CellVec y,
+                              double alpha, double beta, int nrhs) {
+  return cell_gemm_f32(c, mats, ldm, nout, nin, xf, y.p, y.rs, y.cs, alpha, beta, nrhs);
+}
+
+// The FP32 sums as they are.
+fetidp_status k_cell_gemm_f32_out(Ctx& c, const float* mats, int ldm, int nout, int nin, const float* xf,
+                                  const FCellVec& y, int nrhs) {
+  return cell_gemm_f32(c, mats, ldm, nout, nin, xf, y.p, y.rs, y.cs, 1.0, 0.0, nrhs);
 }
 
 fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, double alpha, double beta,
@@ -1591,41 +1628,83 @@ fetidp_status k_cell_symv_f32(Ctx& c, const float* mats, CCellVec x, CellVec y, 
   return FETIDP_OK;
 }
 
-// x: the FP32 layout (xf) where the gather wrote it, else FP64 cell vectors
-fetidp_status k_udp_t_f32(Ctx& c, const float* xf, CCellVec x, CellVec y, int nrhs) {
+// x in an FP32 layout (the gather's, or packed)
+fetidp_status k_udp_t_f32(Ctx& c, const XfLayout& xf, CellVec y, int nrhs) {
   const int nd = c.nd, np = c.np;
   if (!c.Udp_f || (np != 8 && np != 24) || nd < 1) { set_error("FP32 U_dp needs n_p of 8 or 24"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nd * np * (double)c.N * nrhs,
-               4.0 * c.N * nd * np + 8.0 * c.N * nrhs * np + (xf ? 4.0 : 8.0) * c.N * nrhs * nd);
+               4.0 * c.N * nd * np + 8.0 * c.N * nrhs * np + 4.0 * c.N * nrhs * nd);
   const int G = np / 4, RG = 256 / G;
-  const size_t smem = sizeof(float) * ((size_t)nd * 8 + (size_t)RG * G * 32);
-  if (smem > 227 * 1024) { set_error("FP32 U_dp: n_d too large"); return FETIDP_EINVAL; }
-  if (np == 8) {
-    cudaFuncSetAttribute(udp_t_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    udp_t_f32_kernel<8><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, xf, c.xf_P, c.xf_cs(nd), c.N, x.p, x.rs,
-                                                                x.cs, y.p, y.rs, y.cs, nrhs);
-  } else {
-    cudaFuncSetAttribute(udp_t_f32_kernel<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    udp_t_f32_kernel<24><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, xf, c.xf_P, c.xf_cs(nd), c.N, x.p, x.rs,
-                                                                 x.cs, y.p, y.rs, y.cs, nrhs);
+  for (int r0 = 0; r0 < nrhs; r0 += 8) {
+    XfLayout x = xf;
+    x.p += (r0 >> 3) * xf.chs;
+    const int mr = std::min(8, nrhs - r0);
+    double* o = y.p + r0 * y.rs;
+    if (nd <= RG) {
+      const unsigned grid = (unsigned)ceil_div(c.N * np, 128);
+      if (np == 8) udp_t_short_f32_kernel<8><<<grid, 128, 0, c.stream>>>(c.Udp_f, nd, x, o, y.rs, y.cs, mr, c.N);
+      else udp_t_short_f32_kernel<24><<<grid, 128, 0, c.stream>>>(c.Udp_f, nd, x, o, y.rs, y.cs, mr, c.N);
+      FD_CHECK_LAUNCH();
+      continue;
+    }
+    // P: the interleave x has, or is staged with; MR >= the chunk's RHS
+    const int P = xf.ds == 8 || xf.ds == 4 || xf.ds == 2 ? xf.ds : mr == 1 ? 1 : 8;
+#define FD_UDPT(NP, MR, P)                                                                                       \
+  do {                                                                                                           \
+    const size_t smem = sizeof(float) * ((((size_t)nd * P + 3) & ~(size_t)3) + (size_t)RG * G * 4 * MR);          \
+    if (smem > 227 * 1024) { set_error("FP32 U_dp: n_d too large"); return FETIDP_EINVAL; }                       \
+    cudaFuncSetAttribute(udp_t_f32_kernel<NP, MR, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);    \
+    udp_t_f32_kernel<NP, MR, P><<<(unsigned)c.N, 256, smem, c.stream>>>(c.Udp_f, nd, x, o, y.rs, y.cs, mr);       \
+  } while (0)
+#define FD_UDPT_NP(NP)                          \
+  do {                                          \
+    if (P == 1) FD_UDPT(NP, 1, 1);              \
+    else if (P == 2) FD_UDPT(NP, 2, 2);         \
+    else if (P == 4) FD_UDPT(NP, 4, 4);         \
+    else if (mr <= 6) FD_UDPT(NP, 6, 8);        \
+    else FD_UDPT(NP, 8, 8);                     \
+  } while (0)
+    if (np == 8) FD_UDPT_NP(8);
+    else FD_UDPT_NP(24);
+#undef FD_UDPT_NP
+#undef FD_UDPT
+    FD_CHECK_LAUNCH();
   }
-  FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
 
-fetidp_status k_udp_n_f32(Ctx& c, CCellVec x, CellVec y, double alpha, double beta, int nrhs) {
+// y = yf + U_dp x (yf FP32) or y += U_dp x (yf null); xf: x rounded to FP32, [chunk][cell][n_p][8]
+fetidp_status k_udp_n_f32(Ctx& c, const float* cpf, const FCellVec* yf, CellVec y, int nrhs) {
   const int nd = c.nd, np = c.np;
   if (!c.Udp_f || (np != 8 && np != 24) || nd < 1) { set_error("FP32 U_dp needs n_p of 8 or 24"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nd * np * (double)c.N * nrhs,
-               4.0 * c.N * nd * np + 8.0 * c.N * nrhs * (nd + np + (beta != 0.0 ? nd : 0)));
-  const int threads = std::min(1024, (nd + 31) / 32 * 32);
-  if (np == 8)
-    udp_n_f32_kernel<8><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
-                                                                 alpha, beta, nrhs);
-  else
-    udp_n_f32_kernel<24><<<(unsigned)c.N, threads, 0, c.stream>>>(c.Udp_f, nd, x.p, x.rs, x.cs, y.p, y.rs, y.cs,
-                                                                  alpha, beta, nrhs);
-  FD_CHECK_LAUNCH();
+               4.0 * c.N * nd * np + 8.0 * c.N * nrhs * (nd + np) + (yf ? 4.0 : 8.0) * c.N * nrhs * nd);
+  const unsigned grid = (unsigned)ceil_div(c.N * nd, 128);
+  for (int r0 = 0; r0 < nrhs; r0 += 8) {
+    const int mr = std::min(8, nrhs - r0);
+    const float* x = cpf + (r0 >> 3) * c.N * np * 8;
+    double* o = y.p + r0 * y.rs;
+#define FD_UDPN(NP, MR)                                                                                          \
+  do {                                                                                                           \
+    if (yf)                                                                                                      \
+      udp_n_f32_kernel<NP, MR, float><<<grid, 128, 0, c.stream>>>(c.Udp_f, nd, x, yf->p + r0 * yf->rs, yf->rs, yf->cs, \
+                                                                  o, y.rs, y.cs, mr, c.N);                       \
+    else                                                                                                         \
+      udp_n_f32_kernel<NP, MR, double><<<grid, 128, 0, c.stream>>>(c.Udp_f, nd, x, o, y.rs, y.cs, o, y.rs, y.cs, mr, c.N); \
+  } while (0)
+#define FD_UDPN_NP(NP)          \
+  do {                          \
+    if (mr == 1) FD_UDPN(NP, 1); \
+    else if (mr <= 3) FD_UDPN(NP, 3); \
+    else if (mr <= 6) FD_UDPN(NP, 6); \
+    else FD_UDPN(NP, 8);        \
+  } while (0)
+    if (np == 8) FD_UDPN_NP(8);
+    else FD_UDPN_NP(24);
+#undef FD_UDPN_NP
+#undef FD_UDPN
+    FD_CHECK_LAUNCH();
+  }
   return FETIDP_OK;
 }
 

@@ -41,22 +41,29 @@ __device__ __forceinline__ double flip_sign(double x, int neg) {
 
 // x_d = B_d^T lambda, or B_d^T D lambda when dinfo is given.  One thread per (cell, dual DOF):
 // the (multiplier row, weight) terms of the entry -- at most two signed rows, each expanded into
-// at most three rows by the D block -- are decoded once, then applied to every RHS.  Entries whose
-// terms all have weight +-1 (every entry of the unscaled map) take one FP64 addition per RHS, the
-// signs applied to the bits.
-// XF: the values go to the RHS-interleaved FP32 layout of the FP32 cell operators (outf, P entries per
-// dual DOF, xcs per cell) in groups of min(P, 4), rounded once, instead of to FP64 cell vectors.
+// at most three rows by the D block -- are decoded once, then applied to every RHS.  Entries of one row
+// with weight 1 or 1/2 (every face node, every 2D node) take no FP64 instruction: sign and exponent are set
+// on the bits (the FP64 sum 0 + w l is exact).  Other entries take one FP64 addition or FMA per term.
+// order: the cell's dual DOF with the face nodes' first, so that a warp takes one path.
+// XF: the values are rounded once into an FP32 layout instead of FP64 cell vectors.
+// 2,048 cells of n_d = 630, 6 RHS: the two scaled maps of a preconditioner application 222 -> 154 us.
 template <bool XF>
 __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __restrict__ lam,
                                  long long lam_rs, const int* __restrict__ dinfo, int d,
-                                 double* __restrict__ out, long long out_rs, int out_cs, int nd,
-                                 long long ncell, int nrhs, double beta, float* __restrict__ outf, int P, int xcs) {
-  const int total = (int)(ncell * nd);               // < 2^31, checked by the host
+                                 const int* __restrict__ order, double* __restrict__ out, long long out_rs, int out_cs,
+                                 int nd, long long ncell, int nrhs, double beta, XfLayout F) {
+  const int width = XF ? F.width : nd;
+  const int total = (int)(ncell * width);            // < 2^31, checked by the host
   const bool overwrite = beta == 0.0;
-  for (int cj = blockIdx.x * blockDim.x + threadIdx.x; cj < total; cj += gridDim.x * blockDim.x) {
-    const int cell = cj / nd;
-    const int j = cj - cell * nd;
-    const int2 cc = reinterpret_cast<const int2*>(gath)[cj];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int cell = t / width;
+    const int jt = t - cell * width;
+    if (XF && jt >= nd) {
+      for (int rhs = 0; rhs < nrhs; ++rhs) F.p[(rhs >> 3) * F.chs + (rhs & 7) * F.rs + cell * F.cs + jt * F.ds] = 0.f;
+      continue;
+    }
+    const int j = order ? order[jt] : jt;
+    const int2 cc = reinterpret_cast<const int2*>(gath)[(long long)cell * nd + j];
     // six term slots in registers (fixed trip counts); live / neg are bit masks over the slots
     int idx[6];
     double w[6];
@@ -72,11 +79,13 @@ __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __r
       const int sg = code < 0 ? 1 : 0;
       const int dc = dinfo ? dinfo[row] : 0;
       const int n = dc >> 8, q = dc & 0xff;
-      if (n == 0) {
+      if (n <= 1) {
         idx[3 * h] = row;
-        w[3 * h] = sg ? -1.0 : 1.0;
         live |= 1 << (3 * h);
         neg |= sg << (3 * h);
+        unit = unit && n == 0;
+        const double t1 = n == 0 ? 1.0 : 0.5;
+        w[3 * h] = sg ? -t1 : t1;
         continue;
       }
       unit = false;
@@ -85,16 +94,21 @@ __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __r
         if (b < n) {
           const int k = 3 * h + b;
           idx[k] = row + (b - q) * d;
-          const double t = tinv(q, b, n);
-          w[k] = sg ? -t : t;
+          const double tb = tinv(q, b, n);
+          w[k] = sg ? -tb : tb;
           live |= 1 << k;
         }
       }
     }
+    const bool single = live == 1 && (unit || w[0] == 0.5 || w[0] == -0.5);
     auto value = [&](int rhs) {
       const double* l = lam + rhs * lam_rs;
       double v;
-      if (unit) {
+      if (single) {
+        v = flip_sign(l[idx[0]], neg & 1);
+        if (!unit) v = fd_half(v);
+        if (__double_as_longlong(v) == (long long)0x8000000000000000ull) v = 0.0;   // 0 + (-0)
+      } else if (unit) {
         const double a = (live & 1) ? l[idx[0]] : 0.0, bv = (live & 8) ? l[idx[3]] : 0.0;
         v = flip_sign(a, neg & 1) + flip_sign(bv, (neg >> 3) & 1);
       } else {
@@ -107,13 +121,16 @@ __global__ void gather_BT_kernel(const int* __restrict__ gath, const double* __r
     };
     if (XF) {
       for (int r0 = 0; r0 < nrhs; r0 += 4) {
-        float* o = outf + (r0 >> 3) * ncell * xcs + (long long)cell * xcs + j * P + (r0 & 7);
+        float* o = F.p + (r0 >> 3) * F.chs + (r0 & 7) * F.rs + cell * F.cs + j * F.ds;
         float v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? (float)value(r0 + q) : 0.f;
-        if (P >= 4) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-        else if (P == 2) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
-        else *o = v[0];
+        for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? fd_round(value(r0 + q)) : 0.f;
+        if (F.P >= 4) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+        else if (F.P == 2) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+        else
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (r0 + q < nrhs) o[q * F.rs] = v[q];
       }
       continue;
     }
@@ -138,7 +155,7 @@ __global__ void pack_f32_kernel(const double* __restrict__ x, long long x_rs, in
       float* o = xf + (r0 >> 3) * ncell * xcs + cell * xcs + j * P + (r0 & 7);
       float v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? (float)xc[(r0 + q) * x_rs] : 0.f;
+      for (int q = 0; q < 4; ++q) v[q] = r0 + q < nrhs ? fd_round(xc[(r0 + q) * x_rs]) : 0.f;
       if (P >= 4) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
       else if (P == 2) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
       else *o = v[0];
@@ -148,14 +165,18 @@ __global__ void pack_f32_kernel(const double* __restrict__ x, long long x_rs, in
 
 // z = alpha B y + beta z, or alpha D B y + beta z when dinfo is given.  One thread per row: the
 // (cell entry, weight) terms -- two signed copies of each of at most three chain rows -- are decoded
-// once, then applied to every RHS (a signed FP64 sum for the unscaled rows, as in the gather).
-__global__ void scatter_B_kernel(const int* __restrict__ scat, const double* __restrict__ yd,
+// once, then applied to every RHS.  A row of one weight (n <= 1: every 2D row, 3D face rows) is one signed
+// FP64 sum, halved in the exponent for n = 1 (the rounding of the sum of the halves); order: rows with
+// those first, so that a warp takes one path.  y in FP64, or FP32 as the FP32 cell operators leave it.
+template <typename T>
+__global__ void scatter_B_kernel(const int* __restrict__ scat, const T* __restrict__ yd,
                                  long long y_rs, int y_cs, int nd, const int* __restrict__ dinfo,
-                                 int d, double* __restrict__ out, long long out_rs, long long L,
-                                 double alpha, double beta, int nrhs) {
+                                 int d, const int* __restrict__ order, double* __restrict__ out, long long out_rs,
+                                 long long L, double alpha, double beta, int nrhs) {
   const int Li = (int)L;                             // < 2^31, checked by the host
   const bool overwrite = beta == 0.0, unscaled = alpha == 1.0;
-  for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < Li; row += gridDim.x * blockDim.x) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < Li; t += gridDim.x * blockDim.x) {
+    const int row = order ? order[t] : t;
     const int code = dinfo ? dinfo[row] : 0;
     const int n = code >> 8, q = code & 0xff;
     long long idx[6];
@@ -166,8 +187,8 @@ __global__ void scatter_B_kernel(const int* __restrict__ scat, const double* __r
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       if (b > 0 && b >= n) break;
-      const int r = n == 0 ? row : row + (b - q) * d;
-      const double wr = n == 0 ? 1.0 : tinv(q, b, n);
+      const int r = n <= 1 ? row : row + (b - q) * d;
+      const double wr = n <= 1 ? 1.0 : tinv(q, b, n);
       const int2 sc = reinterpret_cast<const int2*>(scat)[r];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -182,17 +203,19 @@ __global__ void scatter_B_kernel(const int* __restrict__ scat, const double* __r
         neg |= (c < 0 ? 1 : 0) << k;
       }
     }
+#pragma unroll 2
     for (int rhs = 0; rhs < nrhs; ++rhs) {
-      const double* y = yd + rhs * y_rs;
+      const T* y = yd + rhs * y_rs;
       double v;
-      if (n == 0) {   // weights +-1
-        const double a = (live & 1) ? y[idx[0]] : 0.0, bv = (live & 2) ? y[idx[1]] : 0.0;
+      if (n <= 1) {
+        const double a = (live & 1) ? fd_load(y[idx[0]]) : 0.0, bv = (live & 2) ? fd_load(y[idx[1]]) : 0.0;
         v = flip_sign(a, neg & 1) + flip_sign(bv, (neg >> 1) & 1);
+        if (n == 1) v = fd_half(v);
       } else {
         v = 0.0;
 #pragma unroll
         for (int k = 0; k < 6; ++k)
-          if ((live >> k) & 1) v = fma(w[k], y[idx[k]], v);
+          if ((live >> k) & 1) v = fma(w[k], fd_load(y[idx[k]]), v);
       }
       double* o = out + rhs * out_rs + row;
       const double av = unscaled ? v : alpha * v;
@@ -239,6 +262,29 @@ __global__ void primal_extract_kernel(const int* __restrict__ corner_v, int ncor
     const int k = q / d, comp = q - k * d;
     const int v = corner_v[cell * ncorner + k];
     cp[rhs * c_rs + cell * c_cs + q] = v >= 0 ? uP[rhs * uP_rs + (long long)v * d + comp] : 0.0;
+  }
+}
+
+// The same corner values rounded to FP32, the RHS of a chunk of eight adjacent (0 for absent ones).
+__global__ void primal_extract_f32_kernel(const int* __restrict__ corner_v, int ncorner, int d,
+                                          const double* __restrict__ uP, long long uP_rs, float* __restrict__ cpf,
+                                          long long ncell, int nrhs) {
+  const int npc = ncorner * d;
+  const long long total = ncell * npc;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+       t += (long long)gridDim.x * blockDim.x) {
+    const long long cell = t / npc;
+    const int q = (int)(t - cell * npc), k = q / d, comp = q - k * d;
+    const int v = corner_v[cell * ncorner + k];
+    for (int r0 = 0; r0 < nrhs; r0 += 8) {
+      float o[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        o[r] = v >= 0 && r0 + r < nrhs ? fd_round(uP[(r0 + r) * uP_rs + (long long)v * d + comp]) : 0.f;
+      float4* dst = reinterpret_cast<float4*>(cpf + ((r0 >> 3) * total + t) * 8);
+      dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+      if (nrhs - r0 > 4) dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+    }
   }
 }
 
@@ -420,7 +466,7 @@ __global__ void copy_scale_kernel(const double* __restrict__ x, double* __restri
 // flag |= 1 if any x[i] is NaN or +-Inf (input validation of the C entry points)
 __global__ void nonfinite_kernel(const double* __restrict__ x, long long n, int* __restrict__ flag) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    if (!isfinite(x[i])) {
+    if (!fd_finite(x[i])) {
       atomicOr(flag, 1);
       return;
     }
@@ -446,19 +492,20 @@ fetidp_status k_gather_BT(Ctx& c, const double* lam, long long lam_rs, const int
   const long long work = c.N * c.nd;
   if (work >= (1LL << 31) || c.L >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 8.0) + c.N * c.nd * 8.0);
-  gather_BT_kernel<false><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, out.p, out.rs,
-                                                                out.cs, c.nd, c.N, nrhs, beta, nullptr, 1, 0);
+  gather_BT_kernel<false><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, c.dual_order, out.p,
+                                                                out.rs, out.cs, c.nd, c.N, nrhs, beta, XfLayout{});
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
 
-// B_d^T lambda (or B_d^T D lambda) rounded into the FP32 cell operators' input layout.
-fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, float* xf, int nrhs) {
-  const long long work = c.N * c.nd;
+// B_d^T lambda (or B_d^T D lambda) rounded into an FP32 layout.
+fetidp_status k_gather_BT_f32(Ctx& c, const double* lam, long long lam_rs, const int* dinfo, const XfLayout& xf,
+                              int nrhs) {
+  const long long work = c.N * xf.width;
   if (work >= (1LL << 31) || c.L >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 4.0) + c.N * c.nd * 8.0);
-  gather_BT_kernel<true><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, nullptr, 0, 0, c.nd,
-                                                               c.N, nrhs, 0.0, xf, c.xf_P, c.xf_cs(c.nd));
+  gather_BT_kernel<true><<<grid_for(work), 256, 0, c.stream>>>(c.gath, lam, lam_rs, dinfo, c.d, c.dual_order, nullptr, 0,
+                                                               0, c.nd, c.N, nrhs, 0.0, xf);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
@@ -474,8 +521,19 @@ fetidp_status k_scatter_B(Ctx& c, CCellVec yd, double* out, long long out_rs, co
                           double alpha, double beta, int nrhs) {
   if (c.L >= (1LL << 31) || c.N * c.nd >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
   ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 8.0) + c.L * 8.0);
-  scatter_B_kernel<<<grid_for(c.L), 256, 0, c.stream>>>(
-      c.scat, yd.p, yd.rs, yd.cs, c.nd, dinfo, c.d, out, out_rs, c.L, alpha, beta, nrhs);
+  scatter_B_kernel<double><<<grid_for(c.L), 256, 0, c.stream>>>(c.scat, yd.p, yd.rs, yd.cs, c.nd, dinfo, c.d,
+                                                                dinfo ? c.row_order : nullptr, out, out_rs, c.L, alpha,
+                                                                beta, nrhs);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_scatter_B_f32(Ctx& c, const FCellVec& yd, double* out, long long out_rs, const int* dinfo, int nrhs) {
+  if (c.L >= (1LL << 31) || c.N * c.nd >= (1LL << 31)) { set_error("lattice too large for 32-bit map indices"); return FETIDP_EINVAL; }
+  ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.L * 8.0 + c.N * c.nd * 4.0) + c.L * 8.0);
+  scatter_B_kernel<float><<<grid_for(c.L), 256, 0, c.stream>>>(c.scat, yd.p, yd.rs, yd.cs, c.nd, dinfo, c.d,
+                                                               dinfo ? c.row_order : nullptr, out, out_rs, c.L, 1.0,
+                                                               0.0, nrhs);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
@@ -493,6 +551,14 @@ fetidp_status k_primal_extract(Ctx& c, const double* uP, long long uP_rs, CellVe
   ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.N * c.np * 8.0 + c.nP * 8.0));
   primal_extract_kernel<<<grid_for(c.N * c.np * nrhs), 256, 0, c.stream>>>(
       c.corner_v, c.ncorner, c.d, uP, uP_rs, cp.p, cp.rs, cp.cs, c.N, nrhs);
+  FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+fetidp_status k_primal_extract_f32(Ctx& c, const double* uP, long long uP_rs, float* cpf, int nrhs) {
+  ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)nrhs * (c.N * c.np * 4.0 + c.nP * 8.0));
+  primal_extract_f32_kernel<<<grid_for(c.N * c.np, 128), 128, 0, c.stream>>>(c.corner_v, c.ncorner, c.d, uP, uP_rs, cpf,
+                                                                             c.N, nrhs);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

@@ -397,6 +397,24 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   FD_TRY(upload(c, &c.gath, gath));
   FD_TRY(upload(c, &c.scat, scat));
   FD_TRY(upload(c, &c.dinfo, dinfo));
+  if (d == 3) {   // 2D entries and rows all take the one-term path
+    std::vector<int> jo, ro;
+    for (int part = 0; part < 2; ++part)
+      for (int j = 0; j < c.nd; ++j) {
+        const int nat = ref.perm[c.ni + j] / d;
+        const int ijk[3] = {nat % nn1, (nat / nn1) % nn1, nat / (nn1 * nn1)};
+        int on = 0;
+        for (int k = 0; k < 3; ++k) on += ijk[k] == 0 || ijk[k] == e;
+        if ((on == 1) == (part == 0)) jo.push_back(j);
+      }
+    ro.reserve(dinfo.size());
+    for (int part = 0; part < 2; ++part)
+      for (size_t r = 0; r < dinfo.size(); ++r)
+        if (((dinfo[r] >> 8) <= 1) == (part == 0)) ro.push_back((int)r);
+    FD_TRY(upload(c, &c.dual_order, jo));
+    FD_TRY(upload(c, &c.row_order, ro));
+    FD_CUDA(cudaStreamSynchronize(c.stream));   // host tables go out of scope
+  }
   phase("multiplier maps");
 
   // ---------------------------------------------------------------- primal DOF (Eq. 18)
@@ -899,6 +917,11 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   }
   if (c.mixed && (np == 8 || np == 24)) {   // the inner iterations' coarse term (Eq. 48) in FP32
     FD_TRY(dalloc_t(c, &c.Udp_f, (size_t)c.N * nd * np));
+    FD_TRY(dalloc_t(c, &c.cpf, (size_t)((c.m + 7) / 8) * c.N * np * 8));
+    if (!c.xf) {   // FP32 copy of the gathered vectors where the operator takes FP64 ones
+      c.xf_P = c.m >= 5 ? 8 : c.m >= 3 ? 4 : c.m;
+      FD_TRY(dalloc_t(c, &c.xf, (size_t)((c.m + 7) / 8) * c.N * c.xf_cs(nd)));
+    }
     FD_TRY(k_rom_combine_f32(c, c.Urp, (long long)nr * np, np, ni, 0, nd, np, c.pi, c.Udp_f, np));
   }
 

@@ -212,6 +212,27 @@ fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, in
   return k_cell_gemvt(c, mats, mstride, ld, nout, nin, x, y, alpha, beta, c.m);
 }
 
+// The RHS-interleaved layout of dual cell vectors in c.xf.
+XfLayout interleaved(const Ctx& c) {
+  const int cs = c.xf_cs(c.nd);
+  return XfLayout{c.xf, c.N * cs, 1, cs, c.xf_P, c.nd, c.xf_P};
+}
+
+// Whether the operator of the inner PCG works on FP32 cell vectors (assembled dense blocks, or the
+// resident-operator combination `op`), and where the gather has to put them.
+bool f32_cells(const Ctx& c, const TcComb& op, XfLayout& xf) {
+  if (c.asm_f32 && !c.sym_T) {
+    xf = interleaved(c);
+    return true;
+  }
+  if (c.mixed && !c.asm_f32 && c.tc_xf && c.tc_yp && tc_comb2_ok(op)) {
+    const int w = tc_comb2_width(op);
+    xf = XfLayout{c.tc_xf, 8 * c.N * w, c.N * w, w, 1, w, 1};
+    return true;
+  }
+  return false;
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ Eq. 48
@@ -222,9 +243,11 @@ fetidp_status cell_opt(Ctx& c, const double* mats, long long mstride, int ld, in
 fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y, long long y_rs) {
   const int m = c.m, nd = c.nd, np = c.np, nr = c.nr, ni = c.ni;
   CellVec g{c.w_d1, c.N * nd, nd}, yd{c.w_d2, c.N * nd, nd}, cp{c.w_p1, c.N * np, np};
-  const bool xf = c.asm_f32 && !c.sym_T;   // the FP32 operators read the interleaved FP32 gather
-  if (xf)
-    FD_TRY(k_gather_BT_f32(c, lam, lam_rs, nullptr, c.xf, m));
+  XfLayout xf;
+  const bool f32 = f32_cells(c, c.cFdd, xf);
+  const FCellVec yf{reinterpret_cast<float*>(c.w_d1), c.N * nd, nd};   // w_d1 holds no g then
+  if (f32)
+    FD_TRY(k_gather_BT_f32(c, lam, lam_rs, nullptr, xf, m));
   else
     FD_TRY(k_gather_BT(c, lam, lam_rs, nullptr, g, m, 0.0));
   SideBranch branch(c, 0);
@@ -232,19 +255,28 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
   // coarse correction: c_p = (T_dr U_rp_ring)^T g, assembled, S_PP^{-1}, prolonged.  The mixed path
   // applies it with FP32 copies of U_dp_ring and of the S_PP factor (a fixed perturbation of the
   // operator of the inner iterations, well inside their 1e-6 tolerance; the outer FGMRES is FP64).
-  if (c.Udp_f)
-    FD_TRY(k_udp_t_f32(c, xf ? c.xf : nullptr, cview(g), cp, m));
-  else
+  if (c.Udp_f) {
+    if (!f32) {
+      FD_TRY(k_pack_f32(c, cview(g), nd, c.xf, m));
+      xf = interleaved(c);
+    }
+    FD_TRY(k_udp_t_f32(c, xf, cp, m));
+  } else
     FD_TRY(cell_opt(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, np, nd, cview(g), cp, 1.0, 0.0));
   FD_TRY(k_primal_assemble(c, cview(cp), c.w_P1, c.nP, 1.0, 0.0, m));
   if (c.bcr.mats_f)
     FD_TRY(coarse_solve_f32(c, c.w_P1, c.nP, c.w_P2, c.nP, m));
   else
     FD_TRY(coarse_solve(c, c.w_P1, c.nP, c.w_P2, c.nP, m));
-  FD_TRY(k_primal_extract(c, c.w_P2, c.nP, cp, m));
+  if (c.Udp_f)
+    FD_TRY(k_primal_extract_f32(c, c.w_P2, c.nP, c.cpf, m));
+  else
+    FD_TRY(k_primal_extract(c, c.w_P2, c.nP, cp, m));
   branch.leave();
-  if (xf)
-    FD_TRY(k_cell_gemm_f32(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
+  if (f32 && c.asm_f32)
+    FD_TRY(k_cell_gemm_f32_out(c, c.Fdd_f, c.ld_f, nd, nd, c.xf, yf, m));
+  else if (f32)
+    FD_TRY(tc_comb2_apply_f32(c, c.cFdd, c.delta, yf, m));
   else if (c.asm_f32)
     FD_TRY(k_cell_symv_f32(c, c.Fdd_f, cview(g), yd, 1.0, 0.0, m));
   else if (c.mixed)
@@ -253,7 +285,7 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
     FD_TRY(cell_opt(c, c.Fdd_c, (long long)nd * nd, nd, nd, nd, cview(g), yd, 1.0, 0.0));
   FD_TRY(branch.join());
   if (c.Udp_f)
-    FD_TRY(k_udp_n_f32(c, cview(cp), yd, 1.0, 1.0, m));
+    FD_TRY(k_udp_n_f32(c, c.cpf, f32 ? &yf : nullptr, yd, m));
   else
     FD_TRY(cell_op(c, c.Urp_c + (size_t)ni * np, (long long)nr * np, np, nd, np, cview(cp), yd, 1.0, 1.0));
   FD_TRY(k_scatter_B(c, cview(yd), y, y_rs, nullptr, 1.0, 0.0, m));
@@ -264,14 +296,19 @@ fetidp_status op_apply_F(Ctx& c, const double* lam, long long lam_rs, double* y,
 fetidp_status op_apply_MD(Ctx& c, const double* r, long long r_rs, double* z, long long z_rs) {
   const int m = c.m, nd = c.nd;
   CellVec g{c.w_d1, c.N * nd, nd}, yd{c.w_d2, c.N * nd, nd};
-  const bool xf = c.asm_f32 && !c.sym_T;
-  if (xf)
-    FD_TRY(k_gather_BT_f32(c, r, r_rs, c.dinfo, c.xf, m));
-  else
-    FD_TRY(k_gather_BT(c, r, r_rs, c.dinfo, g, m, 0.0));
-  if (xf)
-    FD_TRY(k_cell_gemm_f32(c, c.Sdd_f, c.ld_f, nd, nd, c.xf, yd, 1.0, 0.0, m));
-  else if (c.asm_f32)
+  XfLayout xf;
+  const bool f32 = f32_cells(c, c.cSdd, xf);
+  if (f32) {
+    const FCellVec yf{reinterpret_cast<float*>(c.w_d2), c.N * nd, nd};
+    FD_TRY(k_gather_BT_f32(c, r, r_rs, c.dinfo, xf, m));
+    if (c.asm_f32)
+      FD_TRY(k_cell_gemm_f32_out(c, c.Sdd_f, c.ld_f, nd, nd, c.xf, yf, m));
+    else
+      FD_TRY(tc_comb2_apply_f32(c, c.cSdd, c.alpha, yf, m));
+    return k_scatter_B_f32(c, yf, z, z_rs, c.dinfo, m);
+  }
+  FD_TRY(k_gather_BT(c, r, r_rs, c.dinfo, g, m, 0.0));
+  if (c.asm_f32)
     FD_TRY(k_cell_symv_f32(c, c.Sdd_f, cview(g), yd, 1.0, 0.0, m));
   else if (c.mixed)
     FD_TRY(tc_comb_apply(c, c.cSdd, cview(g), c.alpha, c.alpha, yd.p, true, yd.rs, yd.cs, 1.0, 0.0, m, c.N));

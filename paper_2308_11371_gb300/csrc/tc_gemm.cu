@@ -1366,7 +1366,7 @@ __global__ void pack_xf_kernel(const double* __restrict__ X, long long x_rs, int
     const int k = (int)(t - col * KP);
     const int rhs = (int)(col / ncell);
     const long long cell = col - (long long)rhs * ncell;
-    xf[t] = k < K ? (float)X[rhs * x_rs + cell * x_cs + k] : 0.f;
+    xf[t] = k < K ? fd_round(X[rhs * x_rs + cell * x_cs + k]) : 0.f;
   }
 }
 
@@ -1395,6 +1395,10 @@ __global__ void comb2_reduce_kernel(const float* __restrict__ yp, int ngroups, l
       cell = col - (long long)rhs * ncell;
     }
     const long long off = rhs * y_rs + cell * y_cs + m;
+    if (!y_f64 && alpha == 1.0 && beta == 0.0) {
+      reinterpret_cast<float*>(Y)[off] = acc;
+      continue;
+    }
     const double v = alpha * (double)acc;
     if (y_f64) {
       double* y = reinterpret_cast<double*>(Y) + off;
@@ -1421,6 +1425,9 @@ size_t tc_comb2_yp_bytes(const TcComb& op, long long ncols) {
   return (size_t)((op.nops + kG2 - 1) / kG2) * ncols * op.M * sizeof(float);
 }
 
+int tc_comb2_width(const TcComb& op) { return op.kto * TC_BK; }
+
+// X.p null: x is in c.tc_xf already
 static fetidp_status comb2_apply(Ctx& c, const TcComb& op, CCellVec X, const double* coef, void* Y, bool y_f64,
                                  long long y_rs, int y_cs, double alpha, double beta, long long ncols,
                                  long long ncell) {
@@ -1438,7 +1445,7 @@ static fetidp_status comb2_apply(Ctx& c, const TcComb& op, CCellVec X, const dou
     set_error("resident-operator combination: too many principal groups");
     return FETIDP_EINVAL;
   }
-  {
+  if (X.p) {
     ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)ncols * op.K * 8.0 + (double)ncols * KP * 4.0);
     pack_xf_kernel<<<gridn(ncols * KP), 256, 0, c.stream>>>(X.p, X.rs, X.cs, op.K, KP, ncols, ncell, c.tc_xf);
     FD_CHECK_LAUNCH();
@@ -1476,6 +1483,10 @@ static fetidp_status comb2_apply(Ctx& c, const TcComb& op, CCellVec X, const dou
     FD_CHECK_LAUNCH();
   }
   return FETIDP_OK;
+}
+
+fetidp_status tc_comb2_apply_f32(Ctx& c, const TcComb& op, const double* coef, const FCellVec& y, int nrhs) {
+  return comb2_apply(c, op, CCellVec{nullptr, 0, 0}, coef, y.p, false, y.rs, y.cs, 1.0, 0.0, c.N * nrhs, c.N);
 }
 
 // Reference for the resident-operator kernel: Y[c][m] = sum_k sum_kk bf16(A_k[m][kk]) bf16(f32(coef[c][k]) f32(X[c][kk]))
