@@ -9,6 +9,12 @@
 // solve is 2 log2(slabs) + 1 level-parallel sweeps of dense b x b FP64
 // matrix-vector products (one warp per output row, all RHS per row) instead
 // of a sequential sparse triangular substitution.
+//
+// Small coarse problems of the FP64 path (n_P <= kDenseP) keep S_PP^{-1} itself: a solve is one launch over
+// all SMs instead of 2 log2(slabs) + 3 dependent ones of a few microseconds each.  The line: a product
+// of 1,024 columns costs about 10 us for up to eight RHS (FP64 pipe), a cyclic reduction of such a problem 46-170 us;
+// the inverse costs a sweep of n_P pivots at setup (2-3 ms at 1,024, as much as the factorisation it
+// replaces at 400).  n_P = 864, 1 RHS: 67 -> 11 us; 972, 6 RHS: 163 -> 28 us.
 #include <cstring>
 
 #include "common.cuh"
@@ -385,6 +391,24 @@ __global__ void bcr_convert_blocks_kernel(const double* __restrict__ src, const 
     d[e] = (float)s[e];
 }
 
+// Dense S_PP from the slab blocks: D[i][j], i and j primal DOF with slab and position.
+__global__ void bcr_dense_kernel(const double* __restrict__ A, const double* __restrict__ C, int b,
+                                 const int* __restrict__ slab, const int* __restrict__ pos, int n,
+                                 double* __restrict__ D) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)n * n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(t / n), j = (int)(t - (long long)i * n);
+    const int si = slab[i], sj = slab[j];
+    const long long bb = (long long)b * b;
+    double v = 0.0;
+    if (si == sj) v = A[si * bb + (long long)pos[i] * b + pos[j]];
+    else if (sj == si + 1) v = C[si * bb + (long long)pos[i] * b + pos[j]];
+    else if (si == sj + 1) v = C[sj * bb + (long long)pos[j] * b + pos[i]];
+    D[t] = v;
+  }
+}
+constexpr int kDenseP = 1024;
+
 // grid-stride kernels may cap the grid; the warp-per-row kernels may not
 inline int gridn(long long work, int threads = 256) {
   long long g = (work + threads - 1) / threads;
@@ -467,10 +491,16 @@ fetidp_status coarse_setup(Ctx& c, const double* Spp_dev) {
   const int levels = (int)nl.size();
   std::vector<long long> base(levels + 1, 0);
   for (int l = 0; l < levels; ++l) base[l + 1] = base[l] + 5LL * nl[l] * bb;
+  const bool dense = !c.mixed && c.nP <= kDenseP;
   const long long pool = base[levels] + bb;
-  FD_TRY(dalloc_t(c, &B.mats, (size_t)pool));
-  B.mat_bytes = (size_t)pool * sizeof(double);
-  double* P = B.mats;
+  double* P = nullptr;
+  if (dense) {
+    FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&P), sizeof(double) * (size_t)nb * bb));
+  } else {
+    FD_TRY(dalloc_t(c, &B.mats, (size_t)pool));
+    B.mat_bytes = (size_t)pool * sizeof(double);
+    P = B.mats;
+  }
   double* Cbuf[2] = {nullptr, nullptr};
   int *vslab_d = nullptr, *vpos_d = nullptr, *st_d = nullptr;
   const long long cmax = nb > 1 ? (long long)(nb - 1) * bb : bb;
@@ -501,6 +531,36 @@ fetidp_status coarse_setup(Ctx& c, const double* Spp_dev) {
                              vpos_d + voff[bl], b, P + base[0], Cbuf[0]));
   bcr_pad_identity_kernel<<<gridn((long long)nb * b), 256, 0, c.stream>>>(P + base[0], bb, b, real_d, nb);
   FD_CHECK_LAUNCH();
+  if (dense) {
+    std::vector<int> where(2 * (size_t)c.nP);   // slab and position of every primal DOF
+    for (int sl = 0; sl < nb; ++sl)
+      for (size_t q = 0; q < slab_dofs[sl].size(); ++q) {
+        where[slab_dofs[sl][q]] = sl;
+        where[(size_t)c.nP + slab_dofs[sl][q]] = (int)q;
+      }
+    int* where_d = nullptr;
+    const int n = (int)c.nP;
+    FD_TRY(dalloc_t(c, &B.dense, (size_t)n * n));
+    FD_TRY(dalloc_t(c, &B.bl, (size_t)c.m * n));
+    B.mat_bytes = sizeof(double) * (size_t)n * n;
+    FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&where_d), sizeof(int) * where.size()));
+    FD_CUDA(cudaMemcpyAsync(where_d, where.data(), sizeof(int) * where.size(), cudaMemcpyHostToDevice, c.stream));
+    bcr_dense_kernel<<<gridn((long long)n * n), 256, 0, c.stream>>>(P, Cbuf[0], b, where_d, where_d + n, n, B.dense);
+    FD_CHECK_LAUNCH();
+    const fetidp_status sd = k_spd_inverse_batched(c, B.dense, (long long)n * n, n, n, 1, st_d);
+    int bad = 0;
+    if (sd == FETIDP_OK) FD_CUDA(cudaMemcpyAsync(&bad, st_d, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    FD_CUDA(cudaStreamSynchronize(c.stream));
+    for (void* p : {(void*)P, (void*)Cbuf[0], (void*)Cbuf[1], (void*)vslab_d, (void*)vpos_d, (void*)real_d, (void*)st_d,
+                    (void*)where_d})
+      tmp_free(c, p);
+    FD_TRY(sd);
+    if (bad) {
+      set_error("coarse S_PP is not positive definite");
+      return FETIDP_ESINGULAR;
+    }
+    return FETIDP_OK;
+  }
   // ---- block cyclic reduction on the device
   B.off_Ainv.assign(levels, {}); B.off_U.assign(levels, {}); B.off_UT.assign(levels, {});
   B.off_V.assign(levels, {}); B.off_VT.assign(levels, {});
@@ -645,6 +705,15 @@ fetidp_status coarse_setup(Ctx& c, const double* Spp_dev) {
 fetidp_status coarse_solve(Ctx& c, const double* b, long long b_rs, double* x, long long x_rs,
                            int nrhs) {
   CoarseBCR& B = c.bcr;
+  if (B.dense) {
+    ProfScope ps(c, FETIDP_K_COARSE, 2.0 * (B.mat_bytes / 8.0) * nrhs, (double)B.mat_bytes + 16.0 * nrhs * c.nP);
+    if (b == x) {   // the product reads all of b for every output
+      FD_TRY(k_copy_scale(c, b, B.bl, c.nP, nrhs, b_rs, c.nP, nullptr, 1.0));
+      b = B.bl;
+      b_rs = c.nP;
+    }
+    return k_dense_symv(c, B.dense, (int)c.nP, b, b_rs, x, x_rs, nrhs);
+  }
   const long long len0 = (long long)B.nb * B.b;
   const long long rs = B.vec_len;
   ProfScope ps(c, FETIDP_K_COARSE, 2.0 * (B.mat_bytes / 8.0) * nrhs,

@@ -175,6 +175,7 @@ struct CoarseBCR {
   double* bl = nullptr;            // device [m][vec_len] right-hand sides per level
   double* xl = nullptr;            // device [m][vec_len] solutions per level
   size_t mat_bytes = 0;
+  double* dense = nullptr;         // FP64 path, n_P <= kDenseP: S_PP^{-1} itself, row-major (no blocks then)
   // mixed path: an FP32 copy of the used blocks (compact pool, same per-level table layout) and
   // level vectors [rhs chunk of 8][vec_len][8] for the inner iterations' coarse correction
   float* mats_f = nullptr;
@@ -385,7 +386,9 @@ struct Ctx {
   int* row_order = nullptr;     // [L]
   int* tc_err = nullptr;        // device error flag of the bounded waits
   unsigned long long wait_ns = 1000000000ull;   // budget of every device-side wait
-  int* chk = nullptr;           // device flag of the input checks
+  // host-mapped flags: [0] set by the input check's kernel itself, [1] copy of tc_err (a check is then one
+  // kernel and a stream synchronisation, without a memset and a copy through pageable memory)
+  int* h_flag = nullptr;
 };
 
 // RAII timing of one launch (or one multi-kernel step) of a kernel class.
@@ -586,6 +589,9 @@ fetidp_status k_cell_gemm_f32_out(Ctx& c, const float* mats, int ldm, int nout, 
 fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride, int ld, int mrows,
                                   int mcols, CCellVec x, CellVec y, double alpha, double beta,
                                   int nrhs);
+// x = S b for one symmetric n x n matrix and every RHS (b, x: [rhs][n], not aliased)
+fetidp_status k_dense_symv(Ctx& c, const double* S, int n, const double* b, long long b_rs, double* x, long long x_rs,
+                           int nrhs);
 fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin,
                            CCellVec x, CellVec y, double alpha, double beta, int nrhs);
 fetidp_status k_grouped_gemm(Ctx& c, const double* A, long long a_stride_k, int lda, int M, int K,

@@ -1742,14 +1742,35 @@ fetidp_status k_cell_gemv_strided(Ctx& c, const double* mats, long long mstride,
 
 template <int MR>
 static fetidp_status gemvt_launch(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin, CCellVec x,
-                                  CellVec y, double alpha, double beta) {
-  const int TI = std::min(nout, 32), S = kGemvThreads / TI, ntile = ceil_div(nout, TI);
+                                  CellVec y, double alpha, double beta, long long ncell, int tile) {
+  const int TI = std::min(nout, tile), S = kGemvThreads / TI, ntile = ceil_div(nout, TI);
   const size_t smem = sizeof(double) * MR * (size_t)std::max(nin, S * TI);
   if (smem > 227 * 1024) { set_error("per-cell operators: too many columns for shared memory"); return FETIDP_EINVAL; }
   cudaFuncSetAttribute(cell_gemvt_kernel<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cell_gemvt_kernel<MR><<<(unsigned)(c.N * ntile), kGemvThreads, smem, c.stream>>>(
+  cell_gemvt_kernel<MR><<<(unsigned)(ncell * ntile), kGemvThreads, smem, c.stream>>>(
       mats, mstride, ld, nout, nin, TI, S, x.p, x.rs, x.cs, y.p, y.rs, y.cs, alpha, beta, ntile);
   FD_CHECK_LAUNCH();
+  return FETIDP_OK;
+}
+
+static fetidp_status gemvt(Ctx& c, const double* mats, long long mstride, int ld, int nout, int nin, CCellVec x,
+                           CellVec y, double alpha, double beta, int nrhs, long long ncell, int tile) {
+  // RHS per launch: eight, fewer where their x would not fit shared memory
+  const int most = (int)std::max<long long>(1, std::min<long long>(kMaxRhsGemv, 227 * 1024 / (8LL * nin)));
+  for (int r0 = 0; r0 < nrhs; r0 += most) {
+    const CCellVec xr{x.p + r0 * x.rs, x.rs, x.cs};
+    const CellVec yr{y.p + r0 * y.rs, y.rs, y.cs};
+    switch (std::min(most, nrhs - r0)) {
+      case 1: FD_TRY(gemvt_launch<1>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 2: FD_TRY(gemvt_launch<2>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 3: FD_TRY(gemvt_launch<3>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 4: FD_TRY(gemvt_launch<4>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 5: FD_TRY(gemvt_launch<5>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 6: FD_TRY(gemvt_launch<6>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      case 7: FD_TRY(gemvt_launch<7>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+      default: FD_TRY(gemvt_launch<8>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta, ncell, tile)); break;
+    }
+  }
   return FETIDP_OK;
 }
 
@@ -1757,23 +1778,14 @@ fetidp_status k_cell_gemvt(Ctx& c, const double* mats, long long mstride, int ld
                            CellVec y, double alpha, double beta, int nrhs) {
   ProfScope ps(c, FETIDP_K_CELL_GEMV, 2.0 * nout * nin * (double)c.N * nrhs,
                8.0 * c.N * ((double)nout * nin + (double)nrhs * (nout + nin)));
-  // RHS per launch: eight, fewer where their x would not fit shared memory
-  const int most = (int)std::max<long long>(1, std::min<long long>(kMaxRhsGemv, 227 * 1024 / (8LL * nin)));
-  for (int r0 = 0; r0 < nrhs; r0 += most) {
-    const CCellVec xr{x.p + r0 * x.rs, x.rs, x.cs};
-    const CellVec yr{y.p + r0 * y.rs, y.rs, y.cs};
-    switch (std::min(most, nrhs - r0)) {
-      case 1: FD_TRY(gemvt_launch<1>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 2: FD_TRY(gemvt_launch<2>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 3: FD_TRY(gemvt_launch<3>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 4: FD_TRY(gemvt_launch<4>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 5: FD_TRY(gemvt_launch<5>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 6: FD_TRY(gemvt_launch<6>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      case 7: FD_TRY(gemvt_launch<7>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-      default: FD_TRY(gemvt_launch<8>(c, mats, mstride, ld, nout, nin, xr, yr, alpha, beta)); break;
-    }
-  }
-  return FETIDP_OK;
+  return gemvt(c, mats, mstride, ld, nout, nin, x, y, alpha, beta, nrhs, c.N, 32);
+}
+
+// Tiles of 8 outputs: one matrix of at most 1,024 columns then spreads over up to 128 SMs, each thread with a
+// chain of at most 32 loads.
+fetidp_status k_dense_symv(Ctx& c, const double* S, int n, const double* b, long long b_rs, double* x, long long x_rs,
+                           int nrhs) {
+  return gemvt(c, S, 0, n, n, n, CCellVec{b, b_rs, 0}, CellVec{x, x_rs, 0}, 1.0, 0.0, nrhs, 1, 8);
 }
 
 fetidp_status k_grouped_gemm(Ctx& c, const double* A, long long a_stride_k, int lda, int M, int K,

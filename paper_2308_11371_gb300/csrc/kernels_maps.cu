@@ -463,11 +463,11 @@ __global__ void copy_scale_kernel(const double* __restrict__ x, double* __restri
   }
 }
 
-// flag |= 1 if any x[i] is NaN or +-Inf (input validation of the C entry points)
+// *flag = 1 (host-mapped) if any x[i] is NaN or +-Inf (input validation of the C entry points)
 __global__ void nonfinite_kernel(const double* __restrict__ x, long long n, int* __restrict__ flag) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     if (!fd_finite(x[i])) {
-      atomicOr(flag, 1);
+      *reinterpret_cast<volatile int*>(flag) = 1;
       return;
     }
 }

@@ -979,13 +979,14 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   FD_TRY(dalloc_t(c, &c.V, (size_t)(c.kry + 1) * m * c.ntot));
   FD_TRY(dalloc_t(c, &c.Z, (size_t)c.kry * m * c.ntot));
   FD_TRY(dalloc_t(c, &c.pcg, 6 * m * c.L + 1));
-  FD_TRY(dalloc(c, reinterpret_cast<void**>(&c.chk), sizeof(int)));
   if (o.interface == 1) FD_TRY(dalloc_t(c, &c.w_i, m * c.N * c.ni));
   FD_TRY(dalloc_t(c, &c.red, (size_t)m * (c.kry + 2) * 304));
   FD_TRY(dalloc_t(c, &c.red_count, (size_t)m * (c.kry + 2)));
   FD_CUDA(cudaMemsetAsync(c.red_count, 0, sizeof(unsigned) * m * (c.kry + 2), c.stream));
   FD_TRY(dalloc_t(c, &c.scal, 64 * m + (size_t)m * (c.kry + 2) * 2));
-  FD_CUDA(cudaMallocHost(&c.h_scal, sizeof(double) * (64 * m + (size_t)m * (c.kry + 2) * 2)));
+  const size_t nscal = 64 * m + (size_t)m * (c.kry + 2) * 2;
+  FD_CUDA(cudaMallocHost(&c.h_scal, sizeof(double) * (nscal + 1)));   // host-mapped: kernels may write the flags
+  c.h_flag = reinterpret_cast<int*>(c.h_scal + nscal);
   FD_CUDA(cudaStreamSynchronize(c.stream));
   phase("workspace");
   c.t_setup_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

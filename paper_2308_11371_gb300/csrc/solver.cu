@@ -856,12 +856,10 @@ static fetidp_status check_inputs(Ctx& c, std::initializer_list<InVec> ins, cons
   if (!out) { set_error("null output"); return FETIDP_EINVAL; }
   if (!c.opt.check_inputs) return FETIDP_OK;
   for (const InVec& v : ins) {
-    FD_CUDA(cudaMemsetAsync(c.chk, 0, sizeof(int), c.stream));
-    FD_TRY(k_nonfinite(c, v.p, v.n, c.chk));
-    int h = 0;
-    FD_CUDA(cudaMemcpyAsync(&h, c.chk, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    *c.h_flag = 0;   // no check is in flight: each ends with a synchronisation
+    FD_TRY(k_nonfinite(c, v.p, v.n, c.h_flag));
     FD_CUDA(cudaStreamSynchronize(c.stream));
-    if (h) { set_error(std::string("non-finite value in ") + v.name); return FETIDP_EINVAL; }
+    if (*const_cast<volatile int*>(c.h_flag)) { set_error(std::string("non-finite value in ") + v.name); return FETIDP_EINVAL; }
   }
   return FETIDP_OK;
 }
@@ -870,9 +868,9 @@ static fetidp_status check_inputs(Ctx& c, std::initializer_list<InVec> ins, cons
 // cleared, so the context stays usable).  Only with check_inputs, which already synchronises.
 static fetidp_status check_waits(Ctx& c, fetidp_status st) {
   if (!c.mixed || !c.tc_err || !c.opt.check_inputs) return st;
-  int h = 0;
-  FD_CUDA(cudaMemcpyAsync(&h, c.tc_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+  FD_CUDA(cudaMemcpyAsync(c.h_flag + 1, c.tc_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   FD_CUDA(cudaStreamSynchronize(c.stream));
+  const int h = c.h_flag[1];
   if (h) {
     FD_CUDA(cudaMemsetAsync(c.tc_err, 0, sizeof(int), c.stream));
     set_error("a device wait (tensor-core pipeline or coarse-solve barrier) exceeded wait_budget_ns (code " + std::to_string(h) + ")");

@@ -184,3 +184,24 @@ def test_unsynchronised_calls_on_a_stream_and_in_a_graph_match_checked_calls(pre
     torch.cuda.synchronize()
     for (y, z), (yw, zw) in zip(outs, want):
         assert torch.equal(y, yw) and torch.equal(z, zw)
+
+
+@pytest.mark.parametrize("n_rhs", [1, 3, 9])
+@pytest.mark.parametrize("kind,copies", [("2d_e9", 1), ("3d_e4", 1), ("3d_e4", 3)])
+def test_dense_and_block_coarse_solves_agree(kind, copies, n_rhs):
+    """The FP64 context keeps S_PP^{-1} (n_P <= 1,024), the mixed one the FP64 block factors of the same
+    matrix up to its own projections (pi agrees to 1e-7): both against each other, in place and not, and
+    the dense one against the oracle."""
+    from paper_2308_11371_gb300 import binding
+    probs = [_problem(kind, n_rhs) for _ in range(copies)]
+    f, s = binding.Solver(probs), binding.Solver(probs, precision=binding.FETIDP_MIXED_BF16)
+    b = np.random.default_rng(4).standard_normal((f.n_rhs, f.n_P))
+    x = f.coarse_solve(_dev(b))
+    y = _dev(b)
+    f.coarse_solve(y, y)
+    assert torch.equal(x, y)
+    assert _rel(s.coarse_solve(_dev(b)).cpu(), x.cpu()) < 1e-6
+    if copies == 1:
+        ref = _oracle(kind)
+        for r in range(n_rhs):
+            assert _rel(x[r].cpu(), ref.rom.coarse_solve(b[r])) < 1e-9
