@@ -573,6 +573,7 @@ inline int gridn(long long work) {
 // every (element, Gauss point) in shared memory, then each node's sum of w detJ N_a over its
 // elements, then every local DOF (natural index perm[li]) of every body load written into the
 // remaining-DOF right-hand side (li < nr) or the cell's corner loads (li >= nr).
+template <bool TAB>
 __global__ void body_loads_kernel(Geo g, int nelem, const int* __restrict__ perm, int n, int nr, int np,
                                   const double* __restrict__ dirs, const int* __restrict__ body, int m,
                                   double* __restrict__ rhs, long long rhs_rs, double* __restrict__ fpc,
@@ -587,9 +588,7 @@ __global__ void body_loads_kernel(Geo g, int nelem, const int* __restrict__ perm
   const double h = 1.0 / e;
   double hw = 1.0;
   for (int k = 0; k < d; ++k) hw *= 0.5 * h;
-  for (int t = threadIdx.x; t < nelem * NA; t += blockDim.x) {
-    const int el = t / NA, gp = t - el * NA;
-    const int ex = el % e, ey = (el / e) % e, ez = el / (e * e);
+  auto weight = [&](int ex, int ey, int ez, int gp) {
     double eta[3], xi[3], J[3][3];
     gauss_point(g, cx, cy, cz, ex, ey, ez, gp, eta, xi);
     macro_jacobian(g, xi, J);
@@ -597,8 +596,13 @@ __global__ void body_loads_kernel(Geo g, int nelem, const int* __restrict__ perm
                               : J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
                                     J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
                                     J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-    wq[t] = hw * det;
-  }
+    return hw * det;
+  };
+  if (TAB)
+    for (int t = threadIdx.x; t < nelem * NA; t += blockDim.x) {
+      const int el = t / NA;
+      wq[t] = weight(el % e, (el / e) % e, el / (e * e), t - el * NA);
+    }
   __syncthreads();
   const int nnode = d == 2 ? nn1 * nn1 : nn1 * nn1 * nn1;
   for (int node = threadIdx.x; node < nnode; node += blockDim.x) {
@@ -614,11 +618,22 @@ __global__ void body_loads_kernel(Geo g, int nelem, const int* __restrict__ perm
           const double tk = gauss_t((gp >> k) & 1);
           Nv *= ((A >> k) & 1) ? tk : 1.0 - tk;
         }
-        acc += wq[el * NA + gp] * Nv;
+        acc += (TAB ? wq[el * NA + gp] : weight(ex, ey, ez, gp)) * Nv;
       }
     }
-    mn[node] = acc;
+    if (TAB) {
+      mn[node] = acc;
+      continue;
+    }
+    for (int l = 0; l < m; ++l)
+      for (int i = 0; i < d && body[l]; ++i) {
+        const int li = perm[n + node * d + i];
+        const double v = acc * dirs[l * d + i];
+        if (li < nr) rhs[l * rhs_rs + s * nr + li] += v;
+        else fpc[((long long)l * ncell + s) * np + (li - nr)] += v;
+      }
   }
+  if (!TAB) return;
   __syncthreads();
   for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
     const int l = t / n, li = t - l * n;
@@ -782,15 +797,18 @@ fetidp_status k_rom_combine(Ctx& c, const double* src, long long kstride, int ld
   return FETIDP_OK;
 }
 
-fetidp_status k_body_loads(Ctx& c, const Geo& g, const int* perm_dev, const double* dirs_dev, const int* body_dev,
-                           double* rhs, long long rhs_rs, double* fpc) {
+fetidp_status k_body_loads(Ctx& c, const LatticeSpan& ls, const int* perm_dev, const double* dirs_dev,
+                           const int* body_dev, double* rhs, long long rhs_rs, double* fpc) {
   const int NA = 1 << c.d;
   const int nnode = c.d == 2 ? (c.e + 1) * (c.e + 1) : (c.e + 1) * (c.e + 1) * (c.e + 1);
   const size_t smem = sizeof(double) * ((size_t)c.nelem * NA + nnode);
-  ProfScope ps(c, FETIDP_K_SETUP, 0.0, 8.0 * (double)c.N * c.m * c.n);
-  cudaFuncSetAttribute(body_loads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  body_loads_kernel<<<(unsigned)c.N, 256, smem, c.stream>>>(g, c.nelem, perm_dev, c.n, c.nr, c.np, dirs_dev,
-                                                             body_dev, c.m, rhs, rhs_rs, fpc, c.N);
+  ProfScope ps(c, FETIDP_K_SETUP, 0.0, 8.0 * (double)ls.ncell * c.m * c.n);
+  const bool tab = smem <= 227 * 1024;   // larger cells: weights recomputed per node
+  const auto kern = tab ? body_loads_kernel<true> : body_loads_kernel<false>;
+  if (tab) FD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<(unsigned)ls.ncell, 256, tab ? smem : 0, c.stream>>>(ls.geo, c.nelem, perm_dev, c.n, c.nr, c.np, dirs_dev,
+                                                              body_dev, c.m, rhs + ls.cell0 * c.nr, rhs_rs,
+                                                              fpc + ls.cell0 * c.np, c.N);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

@@ -1,17 +1,16 @@
 // Setup phase of the ROM-based inexact FETI-DP solver.
 //
-// Host C++ builds the integer maps (Eqs. 12-18), the loads (Eq. 5b) and the
-// O(N_rb) principal work (Eq. 39 factorisations); the O(N) work runs on the
-// GPU: snapshots (Eq. 52), the greedy passes of Algorithm 4, the projection
-// traces of Eq. 42 (one GEMM against the snapshot matrix) and the ROM local
-// operators of Eq. 43.
+// The host validates the problem and builds the reference cell's tables; the
+// O(N) work runs on the GPU: the integer maps (Eqs. 12-18) and the loads (Eq.
+// 5b), snapshots (Eq. 52), the greedy passes of Algorithm 4, the principal
+// factorisations (Eq. 39), the projection traces of Eq. 42 (one GEMM against
+// the snapshot matrix) and the ROM local operators of Eq. 43.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <thread>
 
 #include "common.cuh"
 #include "host_linalg.h"
@@ -82,81 +81,6 @@ RefCell build_ref(int d, int e, int& ni, int& nd, int& np) {
   nd = cnt[1] * d;
   np = cnt[2] * d;
   return R;
-}
-
-// f^(s) of one load case for one cell (natural order), Eq. 5b.
-void cell_load(const Ctx& c, const Geo& g, const fetidp_problem& p, int load, int cx, int cy, int cz,
-               std::vector<double>& f) {
-  const int d = c.d, e = c.e, NA = 1 << d;
-  const double h = 1.0 / e;
-  const double* dir = p.load_dir + (size_t)load * d;
-  const int cc[3] = {cx, cy, cz};
-  std::fill(f.begin(), f.end(), 0.0);
-  if (p.load_kind[load] == 1) {   // body force per unit physical volume
-    for (int el = 0; el < c.nelem; ++el) {
-      const int ec[3] = {el % e, (el / e) % e, el / (e * e)};
-      for (int gp = 0; gp < NA; ++gp) {
-        double eta[3], xi[3], J[3][3];
-        gauss_point(g, cx, cy, cz, ec[0], ec[1], ec[2], gp, eta, xi);
-        macro_jacobian(g, xi, J);
-        double det;
-        if (d == 2) det = J[0][0] * J[1][1] - J[0][1] * J[1][0];
-        else
-          det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
-                J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-                J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-        const double wq = std::pow(0.5 * h, d) * det;
-        for (int A = 0; A < NA; ++A) {
-          double NAv = 1.0;
-          for (int k = 0; k < d; ++k) {
-            const double tk = gauss_t((gp >> k) & 1);
-            NAv *= ((A >> k) & 1) ? tk : 1.0 - tk;
-          }
-          const int node = (ec[0] + (A & 1)) + (e + 1) * ((ec[1] + ((A >> 1) & 1)) +
-                                                          (e + 1) * (d == 3 ? ec[2] + ((A >> 2) & 1) : 0));
-          for (int i = 0; i < d; ++i) f[(size_t)node * d + i] += wq * NAv * dir[i];
-        }
-      }
-    }
-    return;
-  }
-  const int ax = p.load_axis[load], side = p.load_side[load];
-  if (cc[ax] != (side ? g.nc[ax] - 1 : 0)) return;
-  int tang[2], nt = 0;
-  for (int k = 0; k < d; ++k)
-    if (k != ax) tang[nt++] = k;
-  for (int el = 0; el < c.nelem; ++el) {
-    const int ec[3] = {el % e, (el / e) % e, el / (e * e)};
-    if (ec[ax] != (side ? e - 1 : 0)) continue;
-    for (int fg = 0; fg < (1 << (d - 1)); ++fg) {
-      double t[3] = {0.0, 0.0, 0.0};
-      t[ax] = side ? 1.0 : 0.0;
-      for (int q = 0; q < nt; ++q) t[tang[q]] = gauss_t((fg >> q) & 1);
-      double xi[3] = {0.0, 0.0, 0.0};
-      for (int k = 0; k < d; ++k) xi[k] = cc[k] + (ec[k] + t[k]) * h;
-      double J[3][3];
-      macro_jacobian(g, xi, J);
-      double meas;
-      if (d == 2) {
-        meas = std::sqrt(J[0][tang[0]] * J[0][tang[0]] + J[1][tang[0]] * J[1][tang[0]]);
-      } else {
-        const double a[3] = {J[0][tang[0]], J[1][tang[0]], J[2][tang[0]]};
-        const double b[3] = {J[0][tang[1]], J[1][tang[1]], J[2][tang[1]]};
-        const double cr[3] = {a[1] * b[2] - a[2] * b[1], a[2] * b[0] - a[0] * b[2],
-                              a[0] * b[1] - a[1] * b[0]};
-        meas = std::sqrt(cr[0] * cr[0] + cr[1] * cr[1] + cr[2] * cr[2]);
-      }
-      const double wq = std::pow(0.5 * h, d - 1) * meas;
-      for (int A = 0; A < NA; ++A) {
-        if (((A >> ax) & 1) != (side ? 1 : 0)) continue;
-        double NAv = 1.0;
-        for (int k = 0; k < d; ++k) NAv *= ((A >> k) & 1) ? t[k] : 1.0 - t[k];
-        const int node = (ec[0] + (A & 1)) + (e + 1) * ((ec[1] + ((A >> 1) & 1)) +
-                                                        (e + 1) * (d == 3 ? ec[2] + ((A >> 2) & 1) : 0));
-        for (int i = 0; i < d; ++i) f[(size_t)node * d + i] += wq * NAv * dir[i];
-      }
-    }
-  }
 }
 
 template <typename T>
@@ -307,98 +231,20 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   FD_TRY(upload(c, &c.r_dev, c.r_cell));
   phase("reference tables");
 
-  // ---------------------------------------------------------------- multipliers (Eqs. 14-15)
+  // ---------------------------------------------------------------- maps (Eqs. 14-15, 18)
   const int nn1 = e + 1;
-  std::vector<int> gath((size_t)c.N * c.nd * 2, 0);
-  std::vector<int> scat;
-  std::vector<int> dinfo;   // per row: (chain rows n of its node << 8) | chain position q
   {
-    // about one multiplier per dual DOF of every cell and component (upper bound for reserve)
-    const size_t est = (size_t)c.N * c.nd;
-    scat.reserve(2 * est);
-    dinfo.reserve(est);
+    int* dual_pos = nullptr;
+    FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&dual_pos), sizeof(int) * ref.dual_pos.size()));
+    FD_CUDA(cudaMemcpyAsync(dual_pos, ref.dual_pos.data(), sizeof(int) * ref.dual_pos.size(), cudaMemcpyHostToDevice,
+                            c.stream));
+    const fetidp_status st = k_build_maps(c, dual_pos);
+    tmp_free(c, dual_pos);
+    FD_TRY(st);
   }
-  for (int bl = 0; bl < nprob; ++bl) {
-  const fetidp_problem& pl = probs[bl];
-  const long long cell0 = c.lat[bl].cell0;
-  c.lat[bl].L0 = (long long)dinfo.size();
-  const int nx = pl.cells[0], ny = pl.cells[1], nz = pl.cells[2];
-  const long long gd[3] = {(long long)nx * e + 1, (long long)ny * e + 1, d == 3 ? (long long)nz * e + 1 : 1};
-  const long long clamp_coord = pl.clamp_side ? (long long)pl.cells[pl.clamp_axis] * e : 0;
-  for (long long gz = 0; gz < gd[2]; ++gz)
-    for (long long gy = 0; gy < gd[1]; ++gy)
-      for (long long gx = 0; gx < gd[0]; ++gx) {
-        const long long gc[3] = {gx, gy, gz};
-        int on = 0;
-        for (int k = 0; k < d; ++k) on += (gc[k] % e == 0) ? 1 : 0;
-        if (on == 0 || on == d) continue;   // cell interior or lattice vertex (primal)
-        // owner cells: Cartesian product of candidate cell coordinates
-        int cand[3][2], ncand[3];
-        for (int k = 0; k < 3; ++k) {
-          if (k >= d) { cand[k][0] = 0; ncand[k] = 1; continue; }
-          const int nk = pl.cells[k];
-          if (gc[k] % e == 0) {
-            const int q = (int)(gc[k] / e);
-            ncand[k] = 0;
-            if (q - 1 >= 0) cand[k][ncand[k]++] = q - 1;
-            if (q < nk) cand[k][ncand[k]++] = q;
-          } else {
-            cand[k][0] = (int)(gc[k] / e);
-            ncand[k] = 1;
-          }
-        }
-        std::pair<long long, int> own[8];   // (cell, dual node position), sorted by cell
-        int mult = 0;
-        for (int a = 0; a < ncand[0]; ++a)
-          for (int b = 0; b < ncand[1]; ++b)
-            for (int q = 0; q < ncand[2]; ++q) {
-              const int cx = cand[0][a], cy = cand[1][b], cz = cand[2][q];
-              const long long s = cell0 + cx + (long long)nx * (cy + (long long)ny * cz);
-              const int lx = (int)(gx - (long long)cx * e), ly = (int)(gy - (long long)cy * e);
-              const int lz = d == 3 ? (int)(gz - (long long)cz * e) : 0;
-              const int lnode = lx + nn1 * (ly + nn1 * lz);
-              int pos = mult++;
-              while (pos > 0 && own[pos - 1].first > s) { own[pos] = own[pos - 1]; --pos; }
-              own[pos] = {s, ref.dual_pos[lnode]};
-            }
-        const bool clamped = gc[pl.clamp_axis] == clamp_coord;
-        auto add_gath = [&](long long s, int j, int code) {
-          int* gp2 = &gath[((size_t)s * c.nd + j) * 2];
-          if (gp2[0] == 0) gp2[0] = code;
-          else gp2[1] = code;
-        };
-        if (clamped) {
-          for (int q = 0; q < mult; ++q)
-            for (int comp = 0; comp < d; ++comp) {
-              const auto& ow = own[q];
-              const long long row = (long long)dinfo.size();
-              const int j = ow.second * d + comp;
-              scat.push_back((int)(ow.first * c.nd + j + 1));
-              scat.push_back(0);
-              dinfo.push_back(0);
-              add_gath(ow.first, j, (int)(row + 1));
-            }
-        } else {
-          for (int q = 0; q + 1 < mult; ++q)
-            for (int comp = 0; comp < d; ++comp) {
-              const long long row = (long long)dinfo.size();
-              const int j1 = own[q].second * d + comp, j2 = own[q + 1].second * d + comp;
-              scat.push_back((int)(own[q].first * c.nd + j1 + 1));
-              scat.push_back(-(int)(own[q + 1].first * c.nd + j2 + 1));
-              dinfo.push_back(((mult - 1) << 8) | q);
-              add_gath(own[q].first, j1, (int)(row + 1));
-              add_gath(own[q + 1].first, j2, -(int)(row + 1));
-            }
-        }
-      }
-  c.lat[bl].nL = (long long)dinfo.size() - c.lat[bl].L0;
-  }
-  c.L = (long long)dinfo.size();
-  FD_TRY(upload(c, &c.gath, gath));
-  FD_TRY(upload(c, &c.scat, scat));
-  FD_TRY(upload(c, &c.dinfo, dinfo));
+  c.ntot = c.N * c.nr + c.nP + c.L;
   if (d == 3) {   // 2D entries and rows all take the one-term path
-    std::vector<int> jo, ro;
+    std::vector<int> jo;
     for (int part = 0; part < 2; ++part)
       for (int j = 0; j < c.nd; ++j) {
         const int nat = ref.perm[c.ni + j] / d;
@@ -407,155 +253,12 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
         for (int k = 0; k < 3; ++k) on += ijk[k] == 0 || ijk[k] == e;
         if ((on == 1) == (part == 0)) jo.push_back(j);
       }
-    ro.reserve(dinfo.size());
-    for (int part = 0; part < 2; ++part)
-      for (size_t r = 0; r < dinfo.size(); ++r)
-        if (((dinfo[r] >> 8) <= 1) == (part == 0)) ro.push_back((int)r);
     FD_TRY(upload(c, &c.dual_order, jo));
-    FD_TRY(upload(c, &c.row_order, ro));
     FD_CUDA(cudaStreamSynchronize(c.stream));   // host tables go out of scope
   }
-  phase("multiplier maps");
-
-  // ---------------------------------------------------------------- primal DOF (Eq. 18)
-  // free vertices numbered lattice by lattice, lexicographic (x fastest) inside each lattice
-  std::vector<int> corner_v((size_t)c.N * c.ncorner);
-  std::vector<int> vert_cells;
-  int nV = 0;
-  for (int bl = 0; bl < nprob; ++bl) {
-    const fetidp_problem& pl = probs[bl];
-    const long long cell0 = c.lat[bl].cell0;
-    const int nx = pl.cells[0], ny = pl.cells[1], nz = pl.cells[2];
-    const int vd[3] = {nx + 1, ny + 1, d == 3 ? nz + 1 : 1};
-    const long long nvert = (long long)vd[0] * vd[1] * vd[2];
-    const int cvert = pl.clamp_side ? vd[pl.clamp_axis] - 1 : 0;
-    std::vector<int> vnum(nvert, -1);
-    const int V0 = nV;
-    for (long long v = 0; v < nvert; ++v) {
-      const int ijk[3] = {(int)(v % vd[0]), (int)((v / vd[0]) % vd[1]), (int)(v / ((long long)vd[0] * vd[1]))};
-      if (ijk[pl.clamp_axis] != cvert) vnum[v] = nV++;
-    }
-    c.lat[bl].V0 = V0;
-    c.lat[bl].nV = nV - V0;
-    vert_cells.resize((size_t)nV * c.ncorner, -1);
-    std::vector<int> vfill(nV - V0, 0);
-    for (long long sl = 0; sl < c.lat[bl].ncell; ++sl) {
-      const long long s = cell0 + sl;
-      const int cijk[3] = {(int)(sl % nx), (int)((sl / nx) % ny), (int)(sl / ((long long)nx * ny))};
-      for (int k = 0; k < c.ncorner; ++k) {
-        const int o[3] = {k & 1, (k >> 1) & 1, (k >> 2) & 1};
-        long long v = 0, stride = 1;
-        for (int q = 0; q < 3; ++q) {
-          v += (cijk[q] + (q < d ? o[q] : 0)) * stride;
-          stride *= vd[q];
-        }
-        const int vn = vnum[v];
-        corner_v[(size_t)s * c.ncorner + k] = vn;
-        if (vn >= 0) vert_cells[(size_t)vn * c.ncorner + vfill[vn - V0]++] = (int)(s * c.ncorner + k);
-      }
-    }
-  }
-  c.nV = nV;
-  c.nP = (long long)nV * d;
-  FD_TRY(upload(c, &c.corner_v, corner_v));
-  FD_TRY(upload(c, &c.vert_cells, vert_cells));
-  c.ntot = c.N * c.nr + c.nP + c.L;
-
-  // ---------------------------------------------------------------- loads: rhs = (f_R, f_P, 0)
-  {
-    std::vector<double> rhs((size_t)c.m * c.ntot, 0.0), fpc((size_t)c.m * c.N * c.np, 0.0);
-    // a single lattice's body-force loads are integrated on the GPU (every cell's Gauss points);
-    // tractions (face cells only) and batches stay on the host threads
-    bool any_body = false;
-    for (int l = 0; l < c.m; ++l) any_body = any_body || probs[0].load_kind[l] == 1;
-    const bool gpu_body = nprob == 1 && any_body;
-    // each cell's loads (Eq. 5b) on the host threads; every cell writes only its own entries
-    auto cells_range = [&](long long s0, long long s1) {
-      std::vector<double> f(c.n);
-      for (int l = 0; l < c.m; ++l) {
-        if (gpu_body && probs[0].load_kind[l] == 1) continue;
-        double* rl = rhs.data() + (size_t)l * c.ntot;
-        for (long long s = s0; s < s1; ++s) {
-          int bl = 0;
-          while (bl + 1 < nprob && s >= c.lat[bl + 1].cell0) ++bl;
-          const fetidp_problem& pl = probs[bl];
-          const long long sl = s - c.lat[bl].cell0;
-          const int nx = pl.cells[0], ny = pl.cells[1];
-          const int cx = (int)(sl % nx), cy = (int)((sl / nx) % ny), cz = (int)(sl / ((long long)nx * ny));
-          cell_load(c, c.lat[bl].geo, pl, l, cx, cy, cz, f);
-          for (int li = 0; li < c.nr; ++li) rl[s * c.nr + li] = f[ref.perm[li]];
-          for (int q = 0; q < c.np; ++q) fpc[((size_t)l * c.N + s) * c.np + q] = f[ref.perm[c.nr + q]];
-        }
-      }
-    };
-    {
-      const long long nthr = std::max(1LL, std::min<long long>(std::thread::hardware_concurrency(), 32));
-      const long long per = (c.N + nthr - 1) / nthr;
-      std::vector<std::thread> pool;
-      for (long long t = 0; t < nthr; ++t) {
-        const long long s0 = t * per, s1 = std::min(c.N, s0 + per);
-        if (s0 < s1) pool.emplace_back(cells_range, s0, s1);
-      }
-      for (auto& th : pool) th.join();
-    }
-    // primal loads f_P = sum_s A_p f_p (Eq. 18), assembled in cell order (on the GPU below when the
-    // body forces are integrated there)
-    for (int l = 0; l < c.m && !gpu_body; ++l) {
-      double* rl = rhs.data() + (size_t)l * c.ntot;
-      for (long long s = 0; s < c.N; ++s)
-        for (int k = 0; k < c.ncorner; ++k) {
-          const int vn = corner_v[(size_t)s * c.ncorner + k];
-          if (vn < 0) continue;
-          for (int comp = 0; comp < d; ++comp)
-            rl[c.N * c.nr + (size_t)vn * d + comp] += fpc[((size_t)l * c.N + s) * c.np + k * d + comp];
-        }
-    }
-    FD_TRY(upload(c, &c.rhs, rhs));
-    FD_TRY(upload(c, &c.rhs_p_cells, fpc));
-    if (gpu_body) {
-      std::vector<int> body(c.m);
-      std::vector<double> dirs((size_t)c.m * d);
-      for (int l = 0; l < c.m; ++l) {
-        body[l] = probs[0].load_kind[l] == 1 ? 1 : 0;
-        for (int i = 0; i < d; ++i) dirs[(size_t)l * d + i] = probs[0].load_dir[(size_t)l * d + i];
-      }
-      int *perm_d = nullptr, *body_d = nullptr;
-      double* dirs_d = nullptr;
-      FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&perm_d), sizeof(int) * c.n));
-      FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&body_d), sizeof(int) * c.m));
-      FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&dirs_d), sizeof(double) * dirs.size()));
-      FD_CUDA(cudaMemcpyAsync(perm_d, ref.perm.data(), sizeof(int) * c.n, cudaMemcpyHostToDevice, c.stream));
-      FD_CUDA(cudaMemcpyAsync(body_d, body.data(), sizeof(int) * c.m, cudaMemcpyHostToDevice, c.stream));
-      FD_CUDA(cudaMemcpyAsync(dirs_d, dirs.data(), sizeof(double) * dirs.size(), cudaMemcpyHostToDevice, c.stream));
-      FD_TRY(k_body_loads(c, c.lat[0].geo, perm_d, dirs_d, body_d, c.rhs, c.ntot, c.rhs_p_cells));
-      // f_P from every cell's corner loads (tractions and body forces)
-      FD_TRY(k_primal_assemble(c, CCellVec{c.rhs_p_cells, c.N * c.np, c.np}, c.rhs + c.N * c.nr, c.ntot, 1.0,
-                               1.0, c.m));
-      FD_CUDA(cudaStreamSynchronize(c.stream));   // host vectors go out of scope
-      tmp_free(c, perm_d);
-      tmp_free(c, body_d);
-      tmp_free(c, dirs_d);
-    }
-    // per RHS: min over lattices of ||f_b|| / ||f|| (f_b: the lattice's remaining and primal loads)
-    c.tol_scale.assign(c.m, 1.0);
-    if (nprob > 1)
-      for (int l = 0; l < c.m; ++l) {
-        const double* rl = rhs.data() + (size_t)l * c.ntot;
-        double all = 0.0, mn = -1.0;
-        std::vector<double> nb(nprob, 0.0);
-        for (int bl = 0; bl < nprob; ++bl) {
-          for (long long t = c.lat[bl].cell0 * c.nr; t < (c.lat[bl].cell0 + c.lat[bl].ncell) * c.nr; ++t)
-            nb[bl] += rl[t] * rl[t];
-          for (long long t = c.N * c.nr + c.lat[bl].V0 * d; t < c.N * c.nr + (c.lat[bl].V0 + c.lat[bl].nV) * d; ++t)
-            nb[bl] += rl[t] * rl[t];
-          all += nb[bl];
-        }
-        for (int bl = 0; bl < nprob; ++bl)
-          if (nb[bl] > 0.0 && (mn < 0.0 || nb[bl] < mn)) mn = nb[bl];
-        c.tol_scale[l] = (all > 0.0 && mn > 0.0) ? std::sqrt(mn / all) : 1.0;
-      }
-  }
-  phase("primal maps + loads");
+  phase("maps");
+  FD_TRY(k_build_loads(c, probs));
+  phase("loads");
 
   // ---------------------------------------------------------------- snapshots (Eq. 52)
   // node graph of the reference cell in local order: the up to 3^d nodes that share an element
@@ -987,6 +690,28 @@ fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, cons
   const size_t nscal = 64 * m + (size_t)m * (c.kry + 2) * 2;
   FD_CUDA(cudaMallocHost(&c.h_scal, sizeof(double) * (nscal + 1)));   // host-mapped: kernels may write the flags
   c.h_flag = reinterpret_cast<int*>(c.h_scal + nscal);
+  // per RHS: min over lattices of ||f_b|| / ||f|| (f_b: the lattice's remaining and primal loads)
+  c.tol_scale.assign(c.m, 1.0);
+  if (nprob > 1) {
+    std::vector<std::vector<double>> nb(nprob, std::vector<double>(2 * m));
+    for (int bl = 0; bl < nprob; ++bl) {
+      const LatticeSpan& ls = c.lat[bl];
+      const double *fr = c.rhs + ls.cell0 * c.nr, *fp = c.rhs + c.N * c.nr + ls.V0 * d;
+      FD_TRY(k_dot(c, fr, c.ntot, fr, c.ntot, ls.ncell * c.nr, c.m, c.scal));
+      FD_TRY(k_dot(c, fp, c.ntot, fp, c.ntot, ls.nV * d, c.m, c.scal + m));
+      FD_CUDA(cudaMemcpyAsync(nb[bl].data(), c.scal, sizeof(double) * 2 * m, cudaMemcpyDeviceToHost, c.stream));
+    }
+    FD_CUDA(cudaStreamSynchronize(c.stream));
+    for (int l = 0; l < c.m; ++l) {
+      double all = 0.0, mn = -1.0;
+      for (int bl = 0; bl < nprob; ++bl) {
+        const double v = nb[bl][l] + nb[bl][m + l];
+        all += v;
+        if (v > 0.0 && (mn < 0.0 || v < mn)) mn = v;
+      }
+      c.tol_scale[l] = (all > 0.0 && mn > 0.0) ? std::sqrt(mn / all) : 1.0;
+    }
+  }
   FD_CUDA(cudaStreamSynchronize(c.stream));
   phase("workspace");
   c.t_setup_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

@@ -5,6 +5,7 @@ pure applications of a Dirichlet operator 1e-11): the kernels only order the sum
 """
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 from paper_2308_11371_gb300 import workloads as W
 
@@ -205,3 +206,43 @@ def test_dense_and_block_coarse_solves_agree(kind, copies, n_rhs):
         ref = _oracle(kind)
         for r in range(n_rhs):
             assert _rel(x[r].cpu(), ref.rom.coarse_solve(b[r])) < 1e-9
+
+
+@pytest.mark.parametrize("cells,elems,clamp,load", [
+    ((1, 1), 2, (0, 0), (1, 1)), ((5, 1), 3, (1, 1), (0, 0)), ((3, 7), 7, (0, 1), (0, 0)), ((40, 33), 8, (1, 0), (1, 1)),
+    ((1, 1, 1), 2, (0, 0), (0, 1)), ((1, 3, 2), 3, (2, 1), (1, 0)), ((4, 2, 3), 4, (1, 0), (2, 1)),
+    ((3, 3, 5), 5, (0, 1), (0, 0)),
+])
+def test_maps_and_loads_match_oracle(cells, elems, clamp, load):
+    """B, B^T, the corner map and the loads are built per node: grids of one cell, several scan blocks
+    (2048 nodes), each clamped face, a traction and a body force, alone and as the second lattice of a batch."""
+    from oracle.discretization import Lattice
+    from paper_2308_11371_gb300 import binding
+    d = len(cells)
+    make = W.lattice_2d if d == 2 else W.lattice_3d
+    loads = [W.Load(W.LOAD_TRACTION, tuple(np.arange(1.0, d + 1)), axis=load[0], side=load[1]),
+             W.Load(W.LOAD_BODY, tuple(np.arange(d, 0.0, -1.0)))]
+    kw = dict(a=0.3) if d == 2 else dict(map_kind=W.MAP_SHEAR_BEND_3D, map_params=(0.2, 2.0, 0.1, -0.05))
+    prob = make(*cells, e=elems, n_rb=1, **kw)
+    prob.clamp_axis, prob.clamp_side = clamp
+    first = make(*((2, 1) if d == 2 else (1, 2, 1)), e=elems, n_rb=1, **kw)
+    first.loads, prob.loads = loads[::-1], loads
+    rng = np.random.default_rng(11)
+    for probs in ([prob], [first, prob]):
+        lats = [Lattice(q) for q in probs]
+        Bd = sp.block_diag([q.Bd for q in lats]).tocsr()
+        f = np.concatenate([np.stack([q.load(c) for c in range(q.N)], 1) for q in lats], 1)
+        s = binding.Solver(probs if len(probs) > 1 else prob)
+        assert (s.L, s.n_P) == (Bd.shape[0], sum(q.n_P for q in lats))
+        lam = rng.standard_normal((2, s.L))
+        xd = s.gather_BT(_dev(lam)).cpu().numpy()
+        yd = rng.standard_normal((2, s.N, s.n_d))
+        z = s.scatter_B(_dev(yd)).cpu().numpy()
+        u = rng.standard_normal(f.shape)
+        c = s.compliance(_dev(u))
+        for r in range(2):
+            assert np.array_equal(xd[r].ravel(), Bd.T @ lam[r])
+            assert np.array_equal(z[r], Bd @ yd[r].ravel())
+            # sums of at most 2^d loads per node and n_dof N products, in another order
+            assert abs(c[r] - (f[r] * u[r]).sum()) < 1e-12 * np.abs(f[r] * u[r]).sum()
+        s.close()
