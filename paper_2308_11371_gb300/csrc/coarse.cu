@@ -205,7 +205,7 @@ struct BcrCoopF {
   long long b_rs;
   double* xout;
   long long x_rs;
-  unsigned* bar;                        // [0] arrivals, [1] generation (arrivals zeroed before launch)
+  unsigned* bar;                        // [0] arrivals, [1] blocks that have left; zero between launches
   int* err;
   unsigned long long wait_ns;
 };
@@ -216,49 +216,56 @@ __device__ __forceinline__ unsigned long long bcr_gtime() {
   return t;
 }
 
-// Grid-wide barrier for a cooperative launch.  The last block to arrive resets the arrival count
-// and advances the generation; the others spin on the generation until the kernel's deadline, after
-// which they record error 7 and go on (every later wait then ends at once, so the kernel finishes).
-__device__ __forceinline__ void bcr_grid_sync(unsigned* bar, unsigned nblocks, unsigned long long deadline,
+// Grid-wide barrier for a cooperative launch: arrivals are counted up over the whole kernel (step = its
+// number, from 1), a block waits until all of this step's have come.  One reduction and one poll per block;
+// a count that the last block resets, with a generation beside it, needs four dependent L2 round trips.
+// The wait ends at the kernel's deadline, after which error 7 is recorded and the block goes on (every
+// later wait then ends at once, so the kernel finishes).
+__device__ __forceinline__ void bcr_grid_sync(unsigned* bar, unsigned target, unsigned long long deadline,
                                               int* err) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = bar + 1;
-    const unsigned g = *gen;
-    __threadfence();
-    if (atomicAdd(bar, 1u) == nblocks - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      while (*gen == g) {
-        if (bcr_gtime() > deadline) {
-          atomicExch(err, 7);
-          break;
-        }
-        __nanosleep(32);
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned seen;
+    for (int k = 1;; ++k) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= target) break;
+      if ((k & 15) == 0 && bcr_gtime() > deadline) {
+        atomicExch(err, 7);
+        break;
       }
     }
-    __threadfence();
   }
   __syncthreads();
 }
 
 // acc[a][r] += sgn * sum_q M[(row0 + a) b + q] v[q][r] over this lane's columns q (every 32nd),
-// for the rows row0 + a < b.  One pair of 16-byte reads of v serves the four rows.
-__device__ __forceinline__ void bcr_rows4_f32(const float* __restrict__ M, int row0, const float* __restrict__ v,
-                                              int b, int lane, float sgn, float acc[4][8]) {
+// for the rows row0 + a < b.  One pair of 16-byte reads of v serves the four rows; the reads of four
+// columns are in flight together (six spill).
+constexpr int kBcrAhead = 4;
+__device__ __forceinline__ void bcr_rows4_f32(const float* __restrict__ M, int row0, const float* v, int b, int lane,
+                                              float sgn, float acc[4][8]) {
   const int na = min(4, b - row0);
-#pragma unroll 2
-  for (int q = lane; q < b; q += 32) {
-    const float4 x0 = *reinterpret_cast<const float4*>(v + (size_t)q * 8);
-    const float4 x1 = *reinterpret_cast<const float4*>(v + (size_t)q * 8 + 4);
-    const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+  for (int q0 = lane; q0 < b; q0 += 32 * kBcrAhead) {
+    float4 x0[kBcrAhead], x1[kBcrAhead];
+    float mv[kBcrAhead][4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float mv = a < na ? sgn * __ldcs(M + (size_t)(row0 + a) * b + q) : 0.f;
+    for (int u = 0; u < kBcrAhead; ++u) {
+      const int q = q0 + 32 * u;
+      const bool ok = q < b;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) acc[a][r] = fmaf(mv, xv[r], acc[a][r]);
+      for (int a = 0; a < 4; ++a) mv[u][a] = ok && a < na ? __ldg(M + (size_t)(row0 + a) * b + q) : 0.f;
+      x0[u] = ok ? *reinterpret_cast<const float4*>(v + (size_t)q * 8) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x1[u] = ok ? *reinterpret_cast<const float4*>(v + (size_t)q * 8 + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < kBcrAhead; ++u) {
+      if (q0 + 32 * u >= b) break;
+      const float xv[8] = {x0[u].x, x0[u].y, x0[u].z, x0[u].w, x1[u].x, x1[u].y, x1[u].z, x1[u].w};
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[a][r] = fmaf(sgn * mv[u][a], xv[r], acc[a][r]);
     }
   }
 }
@@ -291,15 +298,28 @@ __device__ __forceinline__ void bcr_zero(float acc[4][8]) {
     for (int y = 0; y < 8; ++y) acc[x][y] = 0.f;
 }
 
-__global__ void __launch_bounds__(256) bcr_coop_f32_kernel(BcrCoopF P) {
+// Bound by latency: 2 L + 2 dependent steps of a barrier and a few reads each.  The solution is kept by level-0
+// block (block j of level l is block j 2^l of level 0), so nothing is copied from level to level and each value
+// goes to its primal DOF as it is formed.  With the counting barrier and the reads of four columns in flight, a
+// solve takes 62 us for 8 x 8 x 4 cells (84 before), 67 for 64 x 64 cells (100), 183 for 12 x 12 x 6 (221).
+// Asking the blocks into L2 at the start gives nothing; all three products' reads in flight at once, with
+// fewer RHS a lane where there are fewer, gives 62 -> 60 and 67 -> 61 us but costs the large lattices 1 to 3%
+// of F through the registers.
+__global__ void __launch_bounds__(256, 2) bcr_coop_f32_kernel(BcrCoopF P) {
   const unsigned long long deadline = bcr_gtime() + P.wait_ns;
   const unsigned nblocks = gridDim.x;
+  unsigned target = 0;
   const int lane = threadIdx.x & 31;
   const long long gthreads = (long long)gridDim.x * blockDim.x;
   const long long gt0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nwarps = gthreads >> 5, gw0 = gt0 >> 5;
   const int b = P.b, g4 = (b + 3) / 4;
   const int a = lane >> 3, r = lane & 7;
+  auto put = [&](int ch, long long q, float x) {   // solution entry q (level-0 numbering) of RHS 8 ch + r
+    P.xl[((size_t)ch * P.rs + q) * 8 + r] = x;
+    const int pq = P.perm[q], rr = ch * 8 + r;
+    if (pq >= 0 && rr < P.nrhs) P.xout[rr * P.x_rs + pq] = (double)x;
+  };
   // level-0 right-hand sides: bl[ch][q][r8] = b[8 ch + r8][perm[q]] (0 on padding and absent RHS)
   for (long long t = gt0; t < (long long)P.nch * P.len0 * 8; t += gthreads) {
     const int r8 = (int)(t & 7);
@@ -310,7 +330,7 @@ __global__ void __launch_bounds__(256) bcr_coop_f32_kernel(BcrCoopF P) {
     const int pq = P.perm[q];
     P.bl[((size_t)ch * P.rs + q) * 8 + r8] = (pq >= 0 && rr < P.nrhs) ? (float)P.bin[rr * P.b_rs + pq] : 0.f;
   }
-  bcr_grid_sync(P.bar, nblocks, deadline, P.err);
+  bcr_grid_sync(P.bar, target += nblocks, deadline, P.err);
   // forward: bl[l+1][i/2] = bl[l][i] - U_{i-1}^T bl[l][i-1] - V_{i+1}^T bl[l][i+1]
   for (int l = 0; l < P.L; ++l) {
     const int n = P.n_at[l], n_new = (n + 1) / 2;
@@ -333,7 +353,7 @@ __global__ void __launch_bounds__(256) bcr_coop_f32_kernel(BcrCoopF P) {
         P.bl[((size_t)ch * P.rs + P.vec_off[l + 1]) * 8 + (size_t)inew * b * 8 + o] = vl[(size_t)i * b * 8 + o] - s;
       }
     }
-    bcr_grid_sync(P.bar, nblocks, deadline, P.err);
+    bcr_grid_sync(P.bar, target += nblocks, deadline, P.err);
   }
   // the last remaining block: x = A^{-1} bl
   for (long long task = gw0; task < (long long)g4 * P.nch; task += nwarps) {
@@ -342,42 +362,38 @@ __global__ void __launch_bounds__(256) bcr_coop_f32_kernel(BcrCoopF P) {
     bcr_zero(acc);
     bcr_rows4_f32(P.mats + P.off_final, row0, P.bl + ((size_t)ch * P.rs + P.vec_off[P.L]) * 8, b, lane, 1.f, acc);
     const float s = bcr_warp_reduce32(acc, lane);
-    if (row0 + a < b) P.xl[((size_t)ch * P.rs + P.vec_off[P.L]) * 8 + (size_t)(row0 + a) * 8 + r] = s;
+    if (row0 + a < b) put(ch, row0 + a, s);
   }
-  bcr_grid_sync(P.bar, nblocks, deadline, P.err);
-  // backward: x[l][j] = Ainv_j bl[l][j] - V_j x[l][j-1] - U_j x[l][j+1] (odd j), x[l][j] = x[l+1][j/2]
+  // backward: x[j] = Ainv_j bl[l][j] - V_j x[j-1] - U_j x[j+1] for odd j (even j are level l + 1's)
   for (int l = P.L - 1; l >= 0; --l) {
-    const int n = P.n_at[l];
+    bcr_grid_sync(P.bar, target += nblocks, deadline, P.err);
+    const int n = P.n_at[l], n_odd = n / 2;
     const long long* tA = P.tables + P.tab_off[l];
     const long long* tU = tA + n;
     const long long* tV = tA + 3LL * n;
-    for (long long task = gw0; task < (long long)n * g4 * P.nch; task += nwarps) {
-      const int ch = (int)(task / ((long long)n * g4));
-      const long long tr = task - (long long)ch * n * g4;
-      const int j = (int)(tr / g4), row0 = 4 * (int)(tr - (long long)j * g4);
-      const size_t cl = ((size_t)ch * P.rs + P.vec_off[l]) * 8, cn = ((size_t)ch * P.rs + P.vec_off[l + 1]) * 8;
-      const size_t o = (size_t)(row0 + a) * 8 + r;
-      if ((j & 1) == 0) {
-        if (row0 + a < b) P.xl[cl + (size_t)j * b * 8 + o] = P.xl[cn + (size_t)(j / 2) * b * 8 + o];
-        continue;
-      }
+    for (long long task = gw0; task < (long long)n_odd * g4 * P.nch; task += nwarps) {
+      const int ch = (int)(task / ((long long)n_odd * g4));
+      const long long tr = task - (long long)ch * n_odd * g4;
+      const int k = (int)(tr / g4), j = 2 * k + 1, row0 = 4 * (int)(tr - (long long)k * g4);
+      const float* bl = P.bl + ((size_t)ch * P.rs + P.vec_off[l]) * 8;
+      const float* xl = P.xl + (size_t)ch * P.rs * 8;
+      const auto at0 = [&](int jj) { return ((long long)jj << l) * b; };
       float acc[4][8];
       bcr_zero(acc);
-      bcr_rows4_f32(P.mats + tA[j], row0, P.bl + cl + (size_t)j * b * 8, b, lane, 1.f, acc);
-      bcr_rows4_f32(P.mats + tV[j], row0, P.xl + cn + (size_t)((j - 1) / 2) * b * 8, b, lane, -1.f, acc);
-      if (j + 1 < n)
-        bcr_rows4_f32(P.mats + tU[j], row0, P.xl + cn + (size_t)((j + 1) / 2) * b * 8, b, lane, -1.f, acc);
+      bcr_rows4_f32(P.mats + tA[j], row0, bl + (size_t)j * b * 8, b, lane, 1.f, acc);
+      bcr_rows4_f32(P.mats + tV[j], row0, xl + at0(j - 1) * 8, b, lane, -1.f, acc);
+      if (j + 1 < n) bcr_rows4_f32(P.mats + tU[j], row0, xl + at0(j + 1) * 8, b, lane, -1.f, acc);
       const float s = bcr_warp_reduce32(acc, lane);
-      if (row0 + a < b) P.xl[cl + (size_t)j * b * 8 + o] = s;
+      if (row0 + a < b) put(ch, at0(j) + row0 + a, s);
     }
-    bcr_grid_sync(P.bar, nblocks, deadline, P.err);
   }
-  // scatter of level 0 back to the primal DOF
-  for (long long t = gt0; t < P.len0 * P.nrhs; t += gthreads) {
-    const int rr = (int)(t / P.len0);
-    const long long q = t - rr * P.len0;
-    const int pq = P.perm[q];
-    if (pq >= 0) P.xout[rr * P.x_rs + pq] = (double)P.xl[((size_t)(rr >> 3) * P.rs + q) * 8 + (rr & 7)];
+  // the last block out clears the counters for the next launch: every arrival has been counted by then
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(P.bar + 1, 1u) == nblocks - 1) {
+      atomicExch(P.bar, 0u);
+      atomicExch(P.bar + 1, 0u);
+    }
   }
 }
 
@@ -679,7 +695,7 @@ fetidp_status coarse_setup(Ctx& c, const double* Spp_dev) {
     const int nch = (c.m + 7) / 8;
     FD_TRY(dalloc_t(c, &B.bl_f, (size_t)nch * B.vec_len * 8));
     FD_TRY(dalloc_t(c, &B.xl_f, (size_t)nch * B.vec_len * 8));
-    // cooperative grid: every block resident (occupancy x SMs), no more than the widest level needs
+    // cooperative grid: every block resident (occupancy x SMs), no more than the widest step needs
     int dev = 0, nsm = 0, per_sm = 0;
     FD_CUDA(cudaGetDevice(&dev));
     FD_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -688,8 +704,8 @@ fetidp_status coarse_setup(Ctx& c, const double* Spp_dev) {
     FD_CUDA(cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, dev));
     if (coop_ok && per_sm > 0) {
       // up to two CTAs per SM (measured faster than one at both the 2D and the 3D benchmark sizes),
-      // no more than one warp per task of the widest level
-      const long long widest = (long long)std::max(nb, 1) * ((b + 3) / 4) * nch;   // warp tasks
+      // no more than one warp per task of the widest step: the odd blocks of level 0
+      const long long widest = (long long)((std::max(nb, 1) + 1) / 2) * ((b + 3) / 4) * nch;   // warp tasks
       const long long want = (widest * 32 + 255) / 256;
       B.coop_grid = (int)std::max<long long>(1, std::min<long long>((long long)std::min(per_sm, 2) * nsm, want));
       FD_TRY(dalloc_t(c, &B.coop_bar, 2));
@@ -800,7 +816,6 @@ fetidp_status coarse_solve_f32(Ctx& c, const double* b, long long b_rs, double* 
   P.bar = B.coop_bar;
   P.err = c.tc_err;
   P.wait_ns = c.wait_ns;
-  FD_CUDA(cudaMemsetAsync(B.coop_bar, 0, sizeof(unsigned), c.stream));   // arrivals (the generation runs on)
   void* args[] = {&P};
   FD_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(bcr_coop_f32_kernel), dim3((unsigned)B.coop_grid),
                                       dim3(256), args, 0, c.stream));
