@@ -228,7 +228,7 @@ fetidp_status fetidp_precond(fetidp_ctx *ctx, const double *r, double *z);
 
 /* z = M_D^{-ROM} r (Eq. 47): D-scaled gather, per cell K_dd g - K_di x_i with x_i the ROM
  * approximation of K_ii^(s)^{-1} K_id g (basis [K_ii^(sigma_k)^{-1} K_id g]_k, K_ii^(s)-orthogonal
- * projection), D-scaled scatter; K_s matrix-free (Eq. 52), FP64.  The context must have been set
+ * projection), D-scaled scatter; K_s sparse, FP64.  The context must have been set
  * up with the option interface = 1 (EINVAL otherwise).  r, z: device [n_rhs][L].            */
 fetidp_status fetidp_precond_rom(fetidp_ctx *ctx, const double *r, double *z);
 
@@ -268,8 +268,8 @@ fetidp_status fetidp_gather_BT(fetidp_ctx *ctx, const double *lambda, double *x_
  * [n_rhs][L].  Row-wise, no atomics, bit-exact.                            */
 fetidp_status fetidp_scatter_B(fetidp_ctx *ctx, const double *y_d, double *z);
 
-/* y_s = K_s u_s for every cell (Eq. 5a with Eq. 52), matrix-free from the
- * Gauss-point field C_hat: u, y device [n_rhs][N][n_dof] (natural order).   */
+/* y_s = K_s u_s for every cell (Eq. 5a with Eq. 52), from the sparse FP64 K_s
+ * assembled at setup: u, y device [n_rhs][N][n_dof] (natural order).        */
 fetidp_status fetidp_apply_K(fetidp_ctx *ctx, const double *u, double *y);
 
 /* x = S_PP_ring^{-1} b, the coarse solve of Sec. 3.2.1 (FP64 block cyclic
@@ -297,7 +297,7 @@ fetidp_status fetidp_rom_data(fetidp_ctx *ctx, int *sigma, double *alpha, double
 /* Kernel classes timed by the profiler. */
 enum {
   FETIDP_K_GROUPED_GEMM = 0,  /* principal-operator contraction, FP64 CUDA cores (Eqs. 43, 46a) */
-  FETIDP_K_APPLY_K = 1,       /* matrix-free K_s (Eq. 52) */
+  FETIDP_K_APPLY_K = 1,       /* sparse K_s, FP64 (Eq. 5a) */
   FETIDP_K_MAPS = 2,          /* B_d gather / scatter, A_p assembly / extraction (Eqs. 15, 18) */
   FETIDP_K_COARSE = 3,        /* coarse block cyclic reduction sweeps (Sec. 3.2.1) */
   FETIDP_K_CELL_GEMV = 4,     /* per-cell ROM operators (Eq. 43) */

@@ -550,8 +550,6 @@ fetidp_status k_df_gemm_planes(Ctx& c, const float* Ah, const float* Al, int M, 
                                long long ncols, double* Y, int y_cs);
 int df_pad_rows(long long rows);
 int df_pad_k(int K);
-fetidp_status k_df_gemm(Ctx& c, const double* A, int lda, int M, int K, const double* X, int x_cs, long long ncols,
-                        double* Y, int y_cs);
 fetidp_status k_batched_gemm(Ctx& c, bool ta, bool tb, int M, int N, int K, double alpha, const double* A,
                              long long sa, int lda, const double* B, long long sb, int ldb, double beta, double* C,
                              long long sc, int ldc, int batch);

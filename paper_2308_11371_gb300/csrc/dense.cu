@@ -789,23 +789,6 @@ fetidp_status k_df_gemm_planes(Ctx& c, const float* Ah, const float* Al, int M, 
   return st;
 }
 
-fetidp_status k_df_gemm(Ctx& c, const double* A, int lda, int M, int K, const double* X, int x_cs, long long ncols,
-                        double* Y, int y_cs) {
-  if (M <= 0 || ncols <= 0) return FETIDP_OK;
-  const int Kp = df_pad_k(K);
-  const long long Mp = df_pad_rows(M);
-  float* buf = nullptr;
-  FD_TRY(tmp_alloc(c, reinterpret_cast<void**>(&buf), sizeof(float) * 2 * (size_t)Mp * Kp));
-  {
-    ProfScope ps(c, FETIDP_K_SETUP, 0.0, 16.0 * (double)M * K);
-    df_split_kernel<<<grid_for(Mp * Kp, 256), 256, 0, c.stream>>>(A, M, K, lda, Mp, Kp, buf, buf + (size_t)Mp * Kp);
-    count_launch();
-  }
-  const fetidp_status st = k_df_gemm_planes(c, buf, buf + (size_t)Mp * Kp, M, K, X, x_cs, ncols, Y, y_cs);
-  tmp_free(c, buf);
-  return st;
-}
-
 fetidp_status k_batched_gemm(Ctx& c, bool ta, bool tb, int M, int N, int K, double alpha, const double* A,
                              long long sa, int lda, const double* B, long long sb, int ldb, double beta, double* C,
                              long long sc, int ldc, int batch) {

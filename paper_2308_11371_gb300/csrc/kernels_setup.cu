@@ -64,16 +64,6 @@ __global__ void row_normalise_kernel(const double* __restrict__ A, const double*
   }
 }
 
-// Delta[row] -= beta[row] * zeta
-__global__ void row_update_kernel(double* __restrict__ D, const double* __restrict__ beta,
-                                  const double* __restrict__ zeta, long long len, long long rows) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < rows * len;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long r = t / len;
-    D[t] -= beta[r] * zeta[t - r * len];
-  }
-}
-
 // Selection of step i of Algorithm 4 (one block): the largest infinity norm of the current
 // residual snapshots; the selected cell is the lowest index within relative `tie` of it, and the
 // 2-norm of its residual row is kept for the normalisation.  Stops (and every later kernel of the
@@ -392,13 +382,6 @@ __global__ void greedy_step_df_kernel(float* __restrict__ Dh, float* __restrict_
   }
 }
 
-__global__ void scale_copy_kernel(const double* __restrict__ x, const double* __restrict__ s,
-                                  double* __restrict__ y, long long len) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < len;
-       t += (long long)gridDim.x * blockDim.x)
-    y[t] = x[t] / s[0];
-}
-
 // Reference gradients G_ia (xi-derivatives) of column vectors at every Gauss point.
 // Column (k, l): values at local (i,d,p) index li taken from
 //   mode 0: src[k*kstride + l*lstride + li] for li < len_in, 0 otherwise
@@ -661,13 +644,6 @@ fetidp_status k_row_normalise(Ctx& c, const double* A, const double* nrm, double
   return FETIDP_OK;
 }
 
-fetidp_status k_row_update(Ctx& c, double* D, const double* beta, const double* zeta,
-                           long long rows, long long len) {
-  row_update_kernel<<<gridn(rows * len), kThreads, 0, c.stream>>>(D, beta, zeta, len, rows);
-  FD_CHECK_LAUNCH();
-  return FETIDP_OK;
-}
-
 fetidp_status k_greedy_step(Ctx& c, double* D, const double* zeta, long long rows, long long len, double* beta,
                             double* inf, const GreedyState* st, int i) {
   ProfScope ps(c, FETIDP_K_GREEDY, 4.0 * rows * (double)len, 16.0 * rows * (double)len);
@@ -732,12 +708,6 @@ fetidp_status k_greedy_alpha(Ctx& c, const double* Z, const double* nrm, const d
   greedy_T_kernel<<<(unsigned)(nrb * nrb), kThreads, 0, c.stream>>>(Z, c.snap, c.nsnap, nrb, st, T);
   FD_CHECK_LAUNCH();
   greedy_alpha_kernel<<<gridn(c.N), kThreads, 0, c.stream>>>(T, nrm, beta, c.N, nrb, alpha);
-  FD_CHECK_LAUNCH();
-  return FETIDP_OK;
-}
-
-fetidp_status k_scale_copy(Ctx& c, const double* x, const double* s, double* y, long long len) {
-  scale_copy_kernel<<<gridn(len), kThreads, 0, c.stream>>>(x, s, y, len);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }

@@ -21,9 +21,6 @@ fetidp_status k_row_reduce(Ctx& c, const double* X, long long rows, long long le
                            int mode, double* out);
 fetidp_status k_row_normalise(Ctx& c, const double* A, const double* nrm, double* D, long long rows,
                               long long len);
-fetidp_status k_row_update(Ctx& c, double* D, const double* beta, const double* zeta,
-                           long long rows, long long len);
-fetidp_status k_scale_copy(Ctx& c, const double* x, const double* s, double* y, long long len);
 fetidp_status k_column_gradients(Ctx& c, const double* src, long long kstride, long long lstride,
                                  int len_in, int mode, int unit_base, int nk, int ncol, double* out);
 fetidp_status k_trace_tables(Ctx& c, const TraceTableSpec* specs_dev, int ntab, double* T,

@@ -322,7 +322,7 @@ fetidp_status op_apply_MD(Ctx& c, const double* r, long long r_rs, double* z, lo
 // z = M_D^{-ROM} r: the Dirichlet preconditioner of Eq. 30 whose interior solves K_ii^(s)^{-1} are
 // approximated like Eq. 46 approximates K_rr^(s)^{-1}: R = [K_ii^(sigma_k)^{-1} v_i]_k and the
 // K_ii^(s)-orthogonal projection x_i = R (R^T K_ii R)^{-1} R^T v_i.  Every product with the cell's
-// own stiffness is the matrix-free K_s of Eq. 52 on full local vectors.
+// own stiffness is the sparse FP64 K_s on full local vectors.
 fetidp_status op_apply_MD_rom(Ctx& c, const double* r, long long r_rs, double* z, long long z_rs) {
   if (!c.Kii_inv) { set_error("the context was set up without the Eq. 47 interface option"); return FETIDP_EINVAL; }
   const int m = c.m, nd = c.nd, ni = c.ni, n = c.n, nrb = c.nrb;
