@@ -269,7 +269,7 @@ fetidp_status fetidp_gather_BT(fetidp_ctx *ctx, const double *lambda, double *x_
 fetidp_status fetidp_scatter_B(fetidp_ctx *ctx, const double *y_d, double *z);
 
 /* y_s = K_s u_s for every cell (Eq. 5a with Eq. 52), from the sparse FP64 K_s
- * assembled at setup: u, y device [n_rhs][N][n_dof] (natural order).        */
+ * assembled at setup: u, y device [n_rhs][N][n_dof] (natural order); may alias. */
 fetidp_status fetidp_apply_K(fetidp_ctx *ctx, const double *u, double *y);
 
 /* x = S_PP_ring^{-1} b, the coarse solve of Sec. 3.2.1 (FP64 block cyclic

@@ -142,6 +142,12 @@ __device__ __forceinline__ bool fd_finite(double x) { return ((unsigned)__double
 __device__ __forceinline__ double fd_load(double v) { return v; }
 __device__ __forceinline__ double fd_load(float v) { return fd_widen(v); }
 
+// Whether the arrays a[0, na) and b[0, nb) overlap (an operator called in place).
+inline bool share_memory(const double* a, long long na, const double* b, long long nb) {
+  const std::uintptr_t pa = reinterpret_cast<std::uintptr_t>(a), pb = reinterpret_cast<std::uintptr_t>(b);
+  return pa < pb + sizeof(double) * nb && pb < pa + sizeof(double) * na;
+}
+
 // Per-cell vector view: element (rhs, cell, i) at p[rhs*rs + cell*cs + i].
 struct CellVec {
   double* p;

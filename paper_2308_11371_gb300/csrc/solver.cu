@@ -1184,7 +1184,12 @@ fetidp_status fetidp_scatter_B(fetidp_ctx* ctx, const double* y_d, double* z) {
 fetidp_status fetidp_apply_K(fetidp_ctx* ctx, const double* u, double* y) {
   FD_TRY(enter(ctx));
   Ctx& c = ctx->c;
-  FD_TRY(check_inputs(c, {{u, (long long)c.m * c.N * c.n, "u"}}, y));
+  const long long len = (long long)c.m * c.N * c.n;
+  FD_TRY(check_inputs(c, {{u, len, "u"}}, y));
+  if (share_memory(u, len, y, len)) {   // several blocks read each cell's u while others store y
+    FD_CUDA(cudaMemcpyAsync(c.w_cell_a, u, sizeof(double) * len, cudaMemcpyDeviceToDevice, c.stream));
+    u = c.w_cell_a;
+  }
   return k_apply_K_natural(c, CCellVec{u, c.N * c.n, c.n}, CellVec{y, c.N * c.n, c.n}, c.m);
 }
 

@@ -1,0 +1,42 @@
+"""Operators called with the output buffer equal to the input buffer give the bits of the call into a
+buffer of its own (the kernels of one call read a cell's input from several blocks)."""
+import numpy as np
+import pytest
+
+from paper_2308_11371_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _problem(dim, n_rhs):
+    """Cells of several 64-node blocks and 32-output tiles each; n_rhs body loads."""
+    rng = np.random.default_rng(n_rhs)
+    loads = [W.Load(W.LOAD_BODY, tuple(rng.standard_normal(dim))) for _ in range(n_rhs)]
+    if dim == 2:
+        p = W.lattice_2d(5, 3, 11, a=0.2, r=0.12, n_rb=2)
+        p.loads = loads
+        return p
+    return W.lattice_3d(3, 2, 2, e=5, r=0.2, r_spread=0.05, seed=3, n_rb=3, mask_kind=W.MASK_BCC_SIGMOID, loads=loads)
+
+
+def _vector(*shape):
+    return torch.randn(*shape, generator=torch.Generator(device="cuda").manual_seed(7), dtype=torch.float64,
+                       device="cuda")
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n_rhs", [1, 9])
+def test_cell_stiffness_in_place_and_overlapping(dim, n_rhs):
+    from paper_2308_11371_gb300 import binding
+    s = binding.Solver(_problem(dim, n_rhs))
+    u = _vector(s.n_rhs, s.N, s.n_dof)
+    want = s.apply_K(u)
+    for _ in range(5):
+        y = u.clone()
+        assert torch.equal(s.apply_K(y, out=y), want)
+    buf = torch.zeros(u.numel() + 3, dtype=torch.float64, device="cuda")   # output three entries further on
+    buf[:-3] = u.ravel()
+    s.apply_K(buf[:-3].view_as(u), out=buf[3:].view_as(u))
+    assert torch.equal(buf[3:].view_as(u), want)
