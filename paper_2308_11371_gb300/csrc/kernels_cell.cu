@@ -870,10 +870,12 @@ constexpr int kTraceK = 32, kTraceLd = 33;   // row stride: a warp's 16 (or 8) r
 template <int T>
 __global__ void __launch_bounds__(T * T) trace_gemm_kernel(const double* __restrict__ A, int lda, int M, int K,
                                                            const double* __restrict__ X, long long x_cs,
-                                                           double* __restrict__ Y, long long y_cs, long long ncols) {
+                                                           double* __restrict__ Y, long long y_cs, long long ncols,
+                                                           int mtiles) {
   __shared__ double As[2][T][kTraceLd], Xs[2][T][kTraceLd];
-  const int m0 = blockIdx.x * T;
-  const long long col0 = (long long)blockIdx.y * T;
+  // row tiles fastest; all tiles on blockIdx.x, whose range does not limit the number of cells
+  const long long ct = blockIdx.x / mtiles, col0 = ct * T;
+  const int m0 = (int)(blockIdx.x - ct * mtiles) * T;
   const int tx = threadIdx.x % T, ty = threadIdx.x / T;
   auto load = [&](int buf, int k0) {
     for (int t = threadIdx.x; t < 2 * T * kTraceK; t += T * T) {
@@ -1816,10 +1818,11 @@ fetidp_status k_trace_gemm(Ctx& c, const double* A, int lda, int M, int K, const
   // 16 x 16 outputs per block; 8 x 8 while those blocks do not cover the SMs twice over
   const bool small = (long long)ceil_div(M, 16) * ceil_div(ncols, 16) < 2 * 152;
   const int T = small ? 8 : 16;
-  if (ceil_div(ncols, T) > 65535) { set_error("trace contraction: too many cells for one launch"); return FETIDP_EINVAL; }
-  const dim3 grid((unsigned)ceil_div(M, T), (unsigned)ceil_div(ncols, T));
-  if (small) trace_gemm_kernel<8><<<grid, 64, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols);
-  else trace_gemm_kernel<16><<<grid, 256, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols);
+  const int mtiles = ceil_div(M, T);
+  const long long grid = mtiles * ((ncols + T - 1) / T);
+  if (grid >= (1LL << 31)) { set_error("trace contraction: too many blocks for one launch"); return FETIDP_EINVAL; }
+  if (small) trace_gemm_kernel<8><<<(unsigned)grid, 64, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols, mtiles);
+  else trace_gemm_kernel<16><<<(unsigned)grid, 256, 0, c.stream>>>(A, lda, M, K, X, x_cs, Y, y_cs, ncols, mtiles);
   FD_CHECK_LAUNCH();
   return FETIDP_OK;
 }
