@@ -569,14 +569,15 @@ template <int E>
 __global__ void __launch_bounds__(256, 4) df_gemm_kernel(const float* __restrict__ Ah, const float* __restrict__ Al,
                                                       const float* __restrict__ Xh, const float* __restrict__ Xl,
                                                       int ldk, int nkc, int M, long long ncols,
-                                                      double* __restrict__ Y, int y_cs) {
+                                                      double* __restrict__ Y, int y_cs, int mtiles) {
   constexpr int T = 16 * E;
   __shared__ __align__(16) float sA[2][2][T][DF_LD];   // [buffer][hi, lo][row m][k]
   __shared__ __align__(16) float sX[2][2][T][DF_LD];   // [buffer][hi, lo][column][k]
   // row tiles fastest: the blocks resident together share their X (snapshot) tiles, which are
-  // then read from DRAM about once, while the table planes stay in L2
-  const long long m0 = (long long)blockIdx.x * T;
-  const long long col0 = (long long)blockIdx.y * T;
+  // then read from DRAM about once, while the table planes stay in L2; all tiles on blockIdx.x,
+  // whose range does not limit the number of cells
+  const long long ct = blockIdx.x / mtiles, col0 = ct * T;
+  const long long m0 = (long long)(blockIdx.x - ct * mtiles) * T;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   // one chunk: 4 planes x T rows x 4 quads of 16 bytes, E copies per thread
   auto load = [&](int buf, int kc) {
@@ -759,8 +760,11 @@ fetidp_status k_df_gemm_planes(Ctx& c, const float* Ah, const float* Al, int M, 
   if (M <= 0 || ncols <= 0) return FETIDP_OK;
   const int Kp = df_pad_k(K);
   const long long Mp = df_pad_rows(M), Np = (ncols + DF_T - 1) / DF_T * DF_T;
-  if (Np / DF_T > 65535) {
-    set_error("trace contraction: too many cells for one launch");
+  const bool wide = (Mp / DF_T) * (Np / DF_T) >= 152;
+  const int t = wide ? 32 : 16, mtiles = (M + t - 1) / t;
+  const long long grid = mtiles * ((ncols + t - 1) / t);
+  if (grid >= (1LL << 31)) {
+    set_error("trace contraction: too many blocks for one launch");
     return FETIDP_EINVAL;
   }
   float* buf = nullptr;
@@ -774,11 +778,8 @@ fetidp_status k_df_gemm_planes(Ctx& c, const float* Ah, const float* Al, int M, 
   }
   {
     ProfScope ps(c, FETIDP_K_TRACES, 2.0 * M * (double)K * ncols, 8.0 * ((double)M * K + (double)ncols * (K + M)));
-    const bool wide = (Mp / DF_T) * (Np / DF_T) >= 152;
-    const int t = wide ? 32 : 16;
-    const dim3 grid((unsigned)((M + t - 1) / t), (unsigned)((ncols + t - 1) / t));
-    if (wide) df_gemm_kernel<2><<<grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs);
-    else df_gemm_kernel<1><<<grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs);
+    if (wide) df_gemm_kernel<2><<<(unsigned)grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs, mtiles);
+    else df_gemm_kernel<1><<<(unsigned)grid, 256, 0, c.stream>>>(Ah, Al, Xh, Xl, Kp, Kp / DF_K, M, ncols, Y, y_cs, mtiles);
     count_launch();
   }
   if (cudaPeekAtLastError() != cudaSuccess) {

@@ -29,3 +29,9 @@ def test_fp64_traces_of_a_million_cells():
     from paper_2308_11371_gb300 import binding
     for a in _projections(11, binding.FETIDP_FP64):
         assert np.abs(a - 1.0).max() < 1e-9
+
+
+def test_mixed_traces_of_two_million_cells():
+    from paper_2308_11371_gb300 import binding
+    for a in _projections(22, binding.FETIDP_MIXED_BF16):
+        assert np.abs(a - 1.0).max() < 1e-9
