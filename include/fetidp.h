@@ -278,12 +278,13 @@ fetidp_status fetidp_apply_K(fetidp_ctx *ctx, const double *u, double *y);
 fetidp_status fetidp_coarse_solve(fetidp_ctx *ctx, const double *b, double *x);
 
 /* x_r = K_rr_ring^{-ROM} v_r (Eq. 46a-b) for every cell: v, x device
- * [n_rhs][N][n_r] in local (i, d) order.                                     */
+ * [n_rhs][N][n_r] in local (i, d) order; may alias.                          */
 fetidp_status fetidp_local_rom_solve(fetidp_ctx *ctx, const double *v, double *x);
 
 /* y = A x with A the saddle-point matrix of Eq. 16, and y = P x with P the
  * preconditioner of Eq. 44 (Algorithm 1).  x, y device [n_rhs][n_tot] laid
- * out as (u_R [N][n_r] local (i,d) order, u_P [n_P], lambda [L]).           */
+ * out as (u_R [N][n_r] local (i,d) order, u_P [n_P], lambda [L]).  x may be y
+ * in apply_P; the two may not alias in apply_A.                             */
 fetidp_status fetidp_apply_A(fetidp_ctx *ctx, const double *x, double *y);
 fetidp_status fetidp_apply_P(fetidp_ctx *ctx, const double *x, double *y);
 

@@ -388,7 +388,16 @@ fetidp_status U_apply(Ctx& c, CCellVec vR, const double* vP, long long vP_rs, do
 // standard FETI-DP: x_r = K_rr^(s)^{-1} v_r with the cell's own inverse
 fetidp_status local_rom(Ctx& c, CCellVec vR, CellVec xR) {
   const int m = c.m, nr = c.nr, nrb = c.nrb;
-  if (c.exact) return cell_opt(c, c.Kinv, (long long)nr * nr, nr, nr, nr, vR, xR, 1.0, 0.0);
+  if (c.exact) {
+    // a cell's outputs are several blocks, each reading all of its v: in place, v comes from a copy
+    const long long cells = c.N * nr;
+    if (share_memory(vR.p, (m - 1) * vR.rs + cells, xR.p, (m - 1) * xR.rs + cells)) {
+      const CellVec v{c.w_cell_a, c.N * nr, nr};
+      FD_TRY(copy_cells(c, vR, v, nr, m));
+      vR = cview(v);
+    }
+    return cell_opt(c, c.Kinv, (long long)nr * nr, nr, nr, nr, vR, xR, 1.0, 0.0);
+  }
   if (c.mixed) {
     float* Rf = reinterpret_cast<float*>(c.w_R);
     float* KRf = reinterpret_cast<float*>(c.w_KR);

@@ -40,3 +40,18 @@ def test_cell_stiffness_in_place_and_overlapping(dim, n_rhs):
     buf[:-3] = u.ravel()
     s.apply_K(buf[:-3].view_as(u), out=buf[3:].view_as(u))
     assert torch.equal(buf[3:].view_as(u), want)
+
+
+@pytest.mark.parametrize("options", [dict(method=1), dict(), dict(precision=1)], ids=["standard", "rom", "rom_mixed"])
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n_rhs", [1, 9])
+def test_local_solve_and_preconditioner_in_place(options, dim, n_rhs):
+    """Standard FETI-DP (one inverse per cell, several output blocks) and the reduced-order local solve,
+    alone and as part of the block preconditioner, whose local solve runs beside the inner PCG."""
+    from paper_2308_11371_gb300 import binding
+    s = binding.Solver(_problem(dim, n_rhs), **options)
+    for name, x in (("local_rom_solve", _vector(s.n_rhs, s.N, s.n_r)), ("apply_P", _vector(s.n_rhs, s.n_tot))):
+        want = getattr(s, name)(x)
+        for _ in range(3):
+            y = x.clone()
+            assert torch.equal(getattr(s, name)(y, out=y), want), name
