@@ -723,7 +723,7 @@ fetidp_status coarse_solve(Ctx& c, const double* b, long long b_rs, double* x, l
   CoarseBCR& B = c.bcr;
   if (B.dense) {
     ProfScope ps(c, FETIDP_K_COARSE, 2.0 * (B.mat_bytes / 8.0) * nrhs, (double)B.mat_bytes + 16.0 * nrhs * c.nP);
-    if (b == x) {   // the product reads all of b for every output
+    if (share_memory(b, (nrhs - 1) * b_rs + c.nP, x, (nrhs - 1) * x_rs + c.nP)) {   // every output reads all of b
       FD_TRY(k_copy_scale(c, b, B.bl, c.nP, nrhs, b_rs, c.nP, nullptr, 1.0));
       b = B.bl;
       b_rs = c.nP;

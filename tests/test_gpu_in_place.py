@@ -55,3 +55,20 @@ def test_local_solve_and_preconditioner_in_place(options, dim, n_rhs):
         for _ in range(3):
             y = x.clone()
             assert torch.equal(getattr(s, name)(y, out=y), want), name
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n_rhs", [1, 9])
+@pytest.mark.parametrize("shift", [0, 1, 40])
+def test_coarse_solve_in_place_and_overlapping(precision, n_rhs, shift):
+    """The stored inverse (FP64) and the block factors (mixed), output `shift` entries after the input."""
+    from paper_2308_11371_gb300 import binding
+    s = binding.Solver(_problem(3, n_rhs), precision=precision)
+    b = _vector(s.n_rhs, s.n_P)
+    want = s.coarse_solve(b)
+    for lo, hi in ((0, shift), (shift, 0)):
+        buf = torch.zeros(b.numel() + shift, dtype=torch.float64, device="cuda")
+        src, dst = (buf[o:o + b.numel()].view_as(b) for o in (lo, hi))
+        src.copy_(b)
+        s.coarse_solve(src, out=dst)
+        assert torch.equal(dst, want)
