@@ -15,7 +15,7 @@ void set_error(const std::string& msg);
 struct Ctx;
 // blocks of the deterministic two-stage reductions (2 x 152 SMs)
 constexpr int kReductionBlocks = 304;
-// stream-ordered temporaries of the setup phase (not tracked by the context)
+// stream-ordered temporaries of the setup phase; what an error return leaves is freed with the context
 fetidp_status tmp_alloc(Ctx& c, void** p, size_t bytes);
 void tmp_free(Ctx& c, void* p);
 void count_launch();
@@ -279,6 +279,7 @@ struct Ctx {
   double t_setup_s = 0.0;
   size_t device_bytes = 0;
   std::vector<void*> allocations;
+  std::vector<void*> temporaries;   // tmp_alloc, until tmp_free
 
   // reference-cell tables
   int* perm = nullptr;        // [2n]: local (i,d,p) index -> natural index node*d + c,

@@ -154,11 +154,15 @@ fetidp_status tmp_alloc(Ctx& c, void** p, size_t bytes) {
     set_error(std::string("cudaMallocAsync(") + std::to_string(bytes) + "): " + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? FETIDP_ENOMEM : FETIDP_ECUDA;
   }
+  c.temporaries.push_back(*p);
   return FETIDP_OK;
 }
 
 void tmp_free(Ctx& c, void* p) {
-  if (p) cudaFreeAsync(p, c.stream);
+  const auto it = std::find(c.temporaries.begin(), c.temporaries.end(), p);
+  if (!p || it == c.temporaries.end()) return;
+  c.temporaries.erase(it);
+  cudaFreeAsync(p, c.stream);
 }
 
 fetidp_status dalloc(Ctx& c, void** p, size_t bytes) {
@@ -1100,6 +1104,7 @@ void fetidp_destroy(fetidp_ctx* ctx) {
     if (ctx->c.ev_fork[k]) cudaEventDestroy(ctx->c.ev_fork[k]);
     if (ctx->c.ev_join[k]) cudaEventDestroy(ctx->c.ev_join[k]);
   }
+  for (void* p : ctx->c.temporaries) cudaFreeAsync(p, ctx->c.stream);   // left by a failed setup
   for (void* p : ctx->c.allocations) cudaFreeAsync(p, ctx->c.stream);
   cudaStreamSynchronize(ctx->c.stream);
   if (ctx->c.h_scal) cudaFreeHost(ctx->c.h_scal);
