@@ -38,7 +38,7 @@ constexpr double kDropRel = 1e-12;    // pivot drop of the N_rb x N_rb Gram syst
 // FP64 path: U_id_ring is assembled per cell (both orientations) up to this size.  Combining the
 // principal operators at every use costs n_rb m FMAs per entry and application on the FP64 pipe, the
 // assembly n_rb once and m per application: 17 ms per application on 32 cells of 6^3 elements with 16
-// principals and 6 RHS against 0.2 ms.  8 GB (2,200 such cells) leaves the largest lattices, whose
+// principals and 6 RHS against 0.2 ms.  8 GiB (2,272 such cells) leaves the largest lattices, whose
 // F_dd and S_dd already fill most of the memory, on the combined form.
 constexpr size_t kUidBytes = (size_t)8 << 30;
 
