@@ -317,7 +317,10 @@ enum {
 /* Start (mask != 0) or stop (mask == 0) timing the kernel classes whose bit is set in
  * mask: a CUDA event pair on the context stream around every launch of those classes
  * (at most 65536 launches until the next read), plus the algorithmic FLOP and byte
- * counts of each launch computed from its shapes.  Resets the accumulators.       */
+ * counts of each launch computed from its shapes.  While classes are timed, the branches
+ * that otherwise run beside each other (coarse correction, local ROM solve) run one after
+ * the other, so that a class's time is its kernels' own; results keep their bits.
+ * Resets the accumulators.                                                          */
 fetidp_status fetidp_profile_enable(fetidp_ctx *ctx, unsigned mask);
 
 /* Synchronise the stream and return per-class totals since the last enable/read

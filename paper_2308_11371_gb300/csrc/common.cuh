@@ -443,7 +443,8 @@ fetidp_status dalloc_t(Ctx& c, T** p, size_t count) {
 // what the main stream holds at that point and runs beside what the main stream gets next, until join().
 // Both ends are events, so the branch becomes a parallel path of a graph when the main stream is being
 // captured.  The destructor joins whatever happened in between (an error return too): nothing of a branch
-// outlives the call on the context's buffers.
+// outlives the call on the context's buffers.  While kernel classes are timed the work stays in line on the
+// main stream: beside each other, a short kernel's event pair would measure how long it waits for SMs.
 struct SideBranch {
   Ctx& c;
   const int k;
@@ -451,6 +452,7 @@ struct SideBranch {
   bool inside = false, open = false;
   SideBranch(Ctx& ctx, int which) : c(ctx), k(which), main(ctx.stream) {}
   fetidp_status enter() {
+    if (c.prof.mask) return FETIDP_OK;
     FD_CUDA(cudaEventRecord(c.ev_fork[k], main));
     FD_CUDA(cudaStreamWaitEvent(c.side[k], c.ev_fork[k], 0));
     c.stream = c.side[k];
