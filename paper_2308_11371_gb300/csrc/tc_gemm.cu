@@ -1477,7 +1477,7 @@ static fetidp_status comb2_apply(Ctx& c, const TcComb& op, CCellVec X, const dou
     FD_CHECK_LAUNCH();
   }
   {
-    ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)ngroups * ncols * op.M * 4.0 + (double)ncols * op.M * 8.0);
+    ProfScope ps(c, FETIDP_K_MAPS, 0.0, (double)ncols * op.M * (4.0 * ngroups + (y_f64 ? 8.0 : 4.0)));
     comb2_reduce_kernel<<<gridn(ncols * op.M), 256, 0, c.stream>>>(c.tc_yp, ngroups, ncols, op.M, ncell, Y,
                                                                   y_f64 ? 1 : 0, y_rs, y_cs, alpha, beta);
     FD_CHECK_LAUNCH();
