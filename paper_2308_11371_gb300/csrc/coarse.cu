@@ -15,10 +15,10 @@
 // of 1,024 columns costs about 10 us for up to eight RHS (FP64 pipe), a cyclic reduction of such a problem 46-170 us;
 // the inverse costs a sweep of n_P pivots at setup (2-3 ms at 1,024, as much as the factorisation it
 // replaces at 400).  n_P = 864, 1 RHS: 67 -> 11 us; 972, 6 RHS: 163 -> 28 us.
+#include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
-#include "host_linalg.h"
 
 namespace fetidp {
 

@@ -13,7 +13,6 @@
 #include <cstring>
 
 #include "common.cuh"
-#include "host_linalg.h"
 
 namespace fetidp {
 
@@ -46,7 +45,6 @@ struct RefCell {
   std::vector<int> perm;        // idp -> natural
   std::vector<int> iperm;       // natural -> idp
   std::vector<int> dual_pos;    // node -> position among dual nodes, or -1
-  std::vector<int> corner_pos;  // node -> corner index, or -1
 };
 
 RefCell build_ref(int d, int e, int& ni, int& nd, int& np) {
@@ -61,11 +59,9 @@ RefCell build_ref(int d, int e, int& ni, int& nd, int& np) {
     cls[nidx] = nb == d ? 2 : (nb > 0 ? 1 : 0);
   }
   R.dual_pos.assign(nnode, -1);
-  R.corner_pos.assign(nnode, -1);
   int cnt[3] = {0, 0, 0};
   for (int nidx = 0; nidx < nnode; ++nidx) {
     if (cls[nidx] == 1) R.dual_pos[nidx] = cnt[1];
-    if (cls[nidx] == 2) R.corner_pos[nidx] = cnt[2];
     cnt[cls[nidx]]++;
   }
   for (int cl = 0; cl < 3; ++cl)
@@ -92,7 +88,6 @@ fetidp_status upload(Ctx& c, T** dst, const std::vector<T>& src) {
 }  // namespace
 
 fetidp_status setup_context(Ctx& c, const fetidp_problem* probs, int nprob, const fetidp_options& o) {
-  using namespace host;
   auto t0 = std::chrono::steady_clock::now();
   // FETIDP_VERBOSE=1: synchronise after each phase and print its wall time to stderr
   const bool verbose = std::getenv("FETIDP_VERBOSE") != nullptr;
