@@ -11,10 +11,11 @@
 // of a sequential sparse triangular substitution.
 //
 // Small coarse problems of the FP64 path (n_P <= kDenseP) keep S_PP^{-1} itself: a solve is one launch over
-// all SMs instead of 2 log2(slabs) + 3 dependent ones of a few microseconds each.  The line: a product
-// of 1,024 columns costs about 10 us for up to eight RHS (FP64 pipe), a cyclic reduction of such a problem 46-170 us;
-// the inverse costs a sweep of n_P pivots at setup (2-3 ms at 1,024, as much as the factorisation it
-// replaces at 400).  n_P = 864, 1 RHS: 67 -> 11 us; 972, 6 RHS: 163 -> 28 us.
+// all SMs instead of 2 log2(slabs) + 3 dependent ones of a few microseconds each.  The line, at n_P = 1,012
+// of 22 x 22 cells: the product takes 9, 23 and 28 us for 1, 6 and 8 RHS (FP64 pipe: 2 FMAs per clock and SM
+// on at most 128 SMs), the cyclic reduction 68, 141 and 160; the sweep of n_P pivots makes set-up 1.7 ms
+// longer (2.8 against 1.1 ms), which 29, 15 and 13 solves pay back.  A whole analysis makes 80 or more.
+// n_P = 612: 8.5, 17 and 21 us against 63, 126 and 145, and 0.5 ms of set-up.
 #include <algorithm>
 #include <cstring>
 
@@ -300,7 +301,10 @@ __device__ __forceinline__ void bcr_zero(float acc[4][8]) {
 
 // Bound by latency: 2 L + 2 dependent steps of a barrier and a few reads each.  The solution is kept by level-0
 // block (block j of level l is block j 2^l of level 0), so nothing is copied from level to level and each value
-// goes to its primal DOF as it is formed.  With the counting barrier and the reads of four columns in flight, a
+// goes to its primal DOF as it is formed.  The wait budget runs from a block's start, also where the launch is
+// a branch beside a product that fills the SMs: a cooperative grid starts when all of it fits (24 x 16 x 8
+// cells, 6 RHS, local solves of 3.5 to 5.4 ms beside: a budget of 0.15 ms is enough, as for the kernel alone,
+// and 0.1 ms is not).  With the counting barrier and the reads of four columns in flight, a
 // solve takes 62 us for 8 x 8 x 4 cells (84 before), 67 for 64 x 64 cells (100), 183 for 12 x 12 x 6 (221).
 // Asking the blocks into L2 at the start gives nothing; all three products' reads in flight at once, with
 // fewer RHS a lane where there are fewer, gives 62 -> 60 and 67 -> 61 us but costs the large lattices 1 to 3%

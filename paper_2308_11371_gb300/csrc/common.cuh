@@ -188,9 +188,9 @@ struct CoarseBCR {
   long long* tables_f = nullptr;
   long long off_final_f = 0;
   float* bl_f = nullptr;
-  float* xl_f = nullptr;
+  float* xl_f = nullptr;           // one solution per level-0 row (chunk stride as bl_f's)
   size_t mat_bytes_f = 0;
-  unsigned* coop_bar = nullptr;    // grid barrier of the cooperative FP32 solve (arrivals, generation)
+  unsigned* coop_bar = nullptr;    // grid barrier of the cooperative FP32 solve (arrivals, blocks that have left)
   int coop_grid = 0;
 };
 
@@ -268,7 +268,9 @@ struct Ctx {
   cudaStream_t ws = nullptr;             // the context's own stream for graph capture and replay
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   // streams of the branches that run beside the main one (SideBranch): 0 the coarse correction of
-  // F_ring (high priority), 1 the local ROM solve; made first in setup, so a use inside a capture makes none
+  // F_ring, 1 the local ROM solve; made first in setup, so a use inside a capture makes none.  Stream 0 has the
+  // highest priority, which direct calls have the use of; the replayed PCG graph is instantiated without node
+  // priorities and runs all its branches at the launch stream's
   cudaStream_t side[2] = {nullptr, nullptr};
   cudaEvent_t ev_fork[2] = {nullptr, nullptr}, ev_join[2] = {nullptr, nullptr};
   // per RHS: min over lattices of ||f_b|| / ||f||; the outer solve targets tol * this so that

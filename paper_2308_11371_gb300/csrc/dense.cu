@@ -541,8 +541,10 @@ __global__ void coarse_assemble_kernel(const double* __restrict__ Spp, long long
 // Bound: FP32 issue, and with few outputs the K = 77,760 steps of one output's chain (K is not split: the
 // Gram solves behind the traces amplify a change of summation order).  E = 2 leaves registers for enough
 // warps to hide the chains (4,096 cells of 16^2 elements, 32 principals: 18.0 ms against 20.2 with E = 4);
-// E = 1 is taken while E = 2 gives less than a block per SM: 46 cells of 6^3 elements and 37 principals
-// 20.1 (E = 4), 5.5 (2), 3.4 ms (1); 256 cells and 32 principals 20.2, 10.1, 12.2; 864 and 15 20.2, 10.1, 9.2.
+// E = 1 is taken while E = 2 gives less than a block per SM: 46 cells of 6^3 elements and 37 principals (92
+// blocks) 20.1 (E = 4), 5.5 (2), 3.4 ms (1); above that a second block on some SMs doubles the time of E = 2,
+// so the two cross more than once and the line stays at one block per SM: 864 cells and 15 principals (216
+// blocks) 20.2, 10.1, 9.2; 256 cells and 32 principals (272 blocks) 20.2, 10.1, 12.2.
 constexpr int DF_K = 16, DF_LD = 20;   // smem rows of 16 floats + 4 pad (16-byte aligned)
 constexpr int DF_T = 32;               // rows and columns of the planes are padded to the wider tile
 

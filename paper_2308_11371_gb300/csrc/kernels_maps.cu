@@ -5,8 +5,8 @@
 //   fixed order, so they are bit-exact and need no atomics.
 // * A_p assembly / extraction of corner values (Eq. 18).
 // * Deterministic FP64 reductions for the Krylov recurrences: a fixed
-//   partition into kRedBlocks blocks, warp-shuffle trees, then the partials
-//   summed in block order by a second kernel.
+//   partition into at most kRedBlocks blocks, warp-shuffle trees, then the
+//   partials summed in a fixed order by the last block to arrive.
 #include "common.cuh"
 
 namespace fetidp {
